@@ -11,7 +11,7 @@
 // overlaps on the device.
 //
 // A request runs in at most two stages, the same two as a direct library
-// call (lb_tiles_kernel, then lb_kint_kernel):
+// call (lb_tiles_kernel, then lb_ktrap_kernel or lb_kint_kernel):
 //   stage A, tile items: each tile goes through classify, bin and the
 //     per-thread expressions (lb_tile.cuh); the K pairs of the fallback
 //     region are appended to per-class queues in the arena, one queue per
@@ -20,10 +20,10 @@
 //   stage B, K-window items: when a request's last tile is done, the device
 //     posts the per-class queue lengths to mapped host memory and the
 //     scheduler publishes windows of each class's queue, costliest class
-//     first; a CTA evaluates a window 32 pairs per warp with the K-integral
-//     code of lb_kint_kernel.  Every window holds pairs of one rule class, so
-//     the warps that run it never switch code paths (mixed rules thrashed the
-//     instruction cache of the direct kernel before it was phased by class).
+//     first; a CTA evaluates a window with the K-integral code of the direct
+//     kernels (a pair per thread in FP64 tight mode, 32 pairs per warp
+//     otherwise).  Every window holds pairs of one class, so the warps that
+//     run it never switch code paths.
 // A request is done when its last item is; the scheduler then copies the
 // results of a host request back and frees the slot and memory.
 //
@@ -56,12 +56,9 @@ using namespace lb;
 namespace {
 
 constexpr int kItemsPerRequest = 64;   // stage A: a request is split into at most this many tile items
-constexpr int kKClasses = 6;           // quadrature rule classes of the FP64 Gauss K integral (kint_class)
+constexpr int kKClasses = 6;           // classes of the FP64 tight K integral (kt_class)
 constexpr int kKItemsPerClass = 64;    // stage B: at most this many windows per class
 constexpr int kKWindowMin = 512;       // smallest window of a class queue (pairs)
-// Costliest class first, as the phases of lb_kint_kernel: the split rule,
-// the 64- and 32-node fixed rules, the packed rule, the one-slot rules.
-constexpr int kKClassOrder[kKClasses] = {0, 5, 4, 3, 2, 1};
 // Item families of the device time accounts (lb_server_device_stats): FP64
 // tiles of log I and log K, FP32 tiles of log I and log K, FP64 K windows of
 // each rule class (or the one queue of the paper modes, as class 0), FP32 K
@@ -73,7 +70,7 @@ struct SlotDesc {          // mapped host memory: written by the host, read by t
   int kind;                // 0 = I, 1 = K
   int dtype;               // LB_F64 or LB_F32
   int mode;
-  int nclass;              // K: queues (kKClasses for the FP64 Gauss rules, else 1); I: 0
+  int nclass;              // K: queues (kKClasses in FP64 tight mode, else 1); I: 0
   long long n;
   long long v_stride;
   unsigned long long v, x, out;   // device addresses (arena, or the caller's for device requests)
@@ -101,12 +98,12 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-// Shared memory of the persistent kernel: one tile, or the node table of a
-// K window with one order for all pairs.
+// Shared memory of the persistent kernel: one tile, the exponential's
+// table (FP64 K windows) or the node table of an FP32 K window with one order.
 union ServeShared {
   TileShared<double, LB_THREADS> d;
   TileShared<float, LB_THREADS> f;
-  KintScalar ks;
+  __align__(16) unsigned long long kt[2048];
   KintScalar32 ks32;
 };
 
@@ -144,7 +141,7 @@ __device__ __forceinline__ void serve_tile(TileShared<T, LB_THREADS>& S, ServeAu
           li[q] = S.list[f0 + j];
           int k = 0;
           if constexpr (sizeof(T) == 8) {
-            if (d.nclass > 1) k = kint_class((double)S.sv[li[q]], (double)S.sx[li[q]], false);   // sv holds |v|
+            if (d.nclass > 1) k = kt_class((double)S.sv[li[q]], (double)S.sx[li[q]], false);   // sv holds |v|
           }
           cl[q] = k;
           rk[q] = atomicAdd(&A.kc[k], 1);
@@ -162,21 +159,29 @@ __device__ __forceinline__ void serve_tile(TileShared<T, LB_THREADS>& S, ServeAu
   __syncthreads();
 }
 
-// Stage B: a window [q0, q1) of one class queue, 32 pairs per warp batch.
+// Stage B: a window [q0, q1) of one class queue: one pair per thread (FP64,
+// tight mode), or 32 pairs per warp batch.
 template <typename T>
 __device__ __forceinline__ void serve_kwindow(ServeShared& U, const SlotDesc& d, int cls, int q0, int q1) {
   const T* v = reinterpret_cast<const T*>(d.v);
   const T* x = reinterpret_cast<const T*>(d.x);
   T* out = reinterpret_cast<T*>(d.out);
   const uint32_t* queue = reinterpret_cast<const uint32_t*>(d.queue) + (int64_t)cls * d.n;
-  const bool gauss = d.mode == MODE_TIGHT;
-  const KintScalar* ks = nullptr;
+  if constexpr (sizeof(T) == 8) {
+    if (d.mode == MODE_TIGHT) {
+      kt_load_table<LB_THREADS>(U.kt);
+      __syncthreads();
+      for (int j = q0 + (int)threadIdx.x; j < q1; j += LB_THREADS) {
+        const int64_t idx = (int64_t)queue[j];
+        out[idx] = kt_eval<false>(fabs(v[idx * d.v_stride]), x[idx], cls, U.kt);
+      }
+      __syncthreads();                             // U is reused by the next item
+      return;
+    }
+  }
   const KintScalar32* ks32 = nullptr;
-  if (d.v_stride == 0 && gauss) {                  // one order for all pairs: its node table once
-    if constexpr (sizeof(T) == 8) {
-      kint_scalar_setup(U.ks, fabs((double)v[0]));
-      ks = &U.ks;
-    } else {
+  if constexpr (sizeof(T) == 4) {
+    if (d.v_stride == 0) {                         // one order for all pairs: its node table once
       kint_scalar_setup32(U.ks32, fabsf((float)v[0]));
       ks32 = &U.ks32;
     }
@@ -187,7 +192,7 @@ __device__ __forceinline__ void serve_kwindow(ServeShared& U, const SlotDesc& d,
     const int64_t idx = (int64_t)queue[b + (lane < k ? lane : 0)];
     const T vi = fabs(v[idx * d.v_stride]);
     const T xi = x[idx];
-    const T val = kint_warp_batch<false, T>(vi, xi, k, lane, gauss, ks, ks32);
+    const T val = kint_warp_batch<T>(vi, xi, k, lane, ks32);
     if (lane < k) out[idx] = val;
   }
   __syncthreads();                                 // U is reused by the next item
@@ -538,7 +543,7 @@ void lb_server::publish_k(Request* r) {
   for (int pass = 0; pass < 2; ++pass) {
     if (pass == 1) slots[r->slot].kitems = items;            // read by the device with the items
     for (int o = 0; o < kKClasses; ++o) {
-      const int c = r->nclass == 1 ? (o == 0 ? 0 : -1) : kKClassOrder[o];
+      const int c = r->nclass == 1 ? (o == 0 ? 0 : -1) : o;      // kt_class: costliest first
       if (c < 0) continue;
       const long long m = kc[c];
       if (m == 0) continue;

@@ -22,6 +22,7 @@
 #include "lb_expr.cuh"
 #include "lb_expr32.cuh"
 #include "lb_kint.cuh"
+#include "lb_ktrap.cuh"
 
 // Threads per block of the serving kernel and of the K-integral and
 // auxiliary kernels; the per-call tile kernel takes its own block size
@@ -390,19 +391,14 @@ __device__ __forceinline__ void tile_eval(TileShared<T, NT>& S, T* __restrict__ 
   __syncthreads();
 }
 
-// K integral of a batch of up to 32 pairs by one warp: lane e holds pair e;
+// K integral of a batch of up to 32 pairs by one warp (the paper's Simpson
+// rule in FP64, the Gauss rules in single precision): lane e holds pair e;
 // each lane computes its pair's prefactor, then the warp evaluates the
 // integrals one pair at a time with the nodes spread over the lanes.
-// CLS >= 0: every pair is of that rule class (FP64 Gauss values; see
-// kint_batch_gauss).
-template <bool DX, typename T, int CLS = -1>
-__device__ __forceinline__ T kint_warp_batch(T vi, T xi, int m, int lane, bool gauss,
-                                            const KintScalar* ks = nullptr, const KintScalar32* ks32 = nullptr) {
-  if constexpr (sizeof(T) == 8) {
-    if (gauss) return kint_batch_gauss<DX, CLS>(vi, xi, m, lane, ks);
-  }
+template <typename T>
+__device__ __forceinline__ T kint_warp_batch(T vi, T xi, int m, int lane, const KintScalar32* ks32 = nullptr) {
   T pre;
-  if constexpr (sizeof(T) == 8) pre = DX ? -(vi / xi + 1.0) : kint_prefactor(vi, xi);
+  if constexpr (sizeof(T) == 8) pre = kint_prefactor(vi, xi);
   else pre = kint_prefactor32(vi, xi);
   float beta_i = 0.0f, logbeta_i = 0.0f;
   if constexpr (sizeof(T) == 4) {
@@ -424,6 +420,15 @@ __device__ __forceinline__ T kint_warp_batch(T vi, T xi, int m, int lane, bool g
     if (lane == e) mine = li;
   }
   return pre + mine;
+}
+
+// The 16 KB table of kt_exp2_q58 in shared memory (random lookups cost a few
+// bank conflicts there, up to 32 cache-line accesses in global memory).  All
+// NT threads of the block call it; the caller synchronizes.
+template <int NT>
+__device__ __forceinline__ void kt_load_table(unsigned long long* tab) {
+  for (int i = 2 * threadIdx.x; i < 2048; i += 2 * NT)
+    *reinterpret_cast<ulonglong2*>(tab + i) = *reinterpret_cast<const ulonglong2*>(lb_kt_exp2 + i);
 }
 
 }  // namespace lb

@@ -10,10 +10,12 @@
 //      32-pair chunks of the lists from shared counters, so every warp runs
 //      one expression (mu_20, U_K, power series) at a time.  K pairs of the
 //      fallback region are appended to a global queue instead.
-//   2. lb_kint_kernel: one warp per queued K pair evaluates the integral with
-//      the nodes spread over the lanes (lb_kint.cuh).
+//   2. lb_ktrap_kernel (tight FP64): one thread per queued K pair evaluates the
+//      integral by the trapezoid rule (lb_ktrap.cuh); lb_kint_kernel (the
+//      paper's dispatches, FP32): one warp per pair with the nodes spread over
+//      the lanes (lb_kint.cuh, lb_expr32.cuh).
 // A call with one order for all pairs (v_stride 0) has its order's
-// constants computed once per block (ScalarOrder, KintScalar).
+// constants computed once per block (ScalarOrder, KintScalar32).
 //
 // The plain form computes in FP64; its exps and logs are evaluated in
 // integer arithmetic where that is faster (lb_intmath.cuh).
@@ -55,35 +57,13 @@ namespace {
 #ifndef LB_KINT_CTAS_PER_SM
 #define LB_KINT_CTAS_PER_SM 4
 #endif
-// The class-specialized K-integral kernels (FP64 Gauss values, one per rule
-// class of kint_class: split, one-slot s0 = 8, one-slot s0 = 3, packed,
-// fixed 32 and 64 g nodes) each hold only their own rule's registers, so the
-// short rules run with more resident warps (budgets measured on the sweep and
-// the robustness sweep: 4, 8, 8, 6, 6, 6 CTAs per SM beat 4 everywhere by
-// 1-2 %; the split rule keeps 4).
-#ifndef LB_KINT_CTAS_C0
-#define LB_KINT_CTAS_C0 4
+#ifndef LB_KTRAP_CTAS_PER_SM
+#define LB_KTRAP_CTAS_PER_SM 4
 #endif
-#ifndef LB_KINT_CTAS_C12
-#define LB_KINT_CTAS_C12 8
-#endif
-#ifndef LB_KINT_CTAS_C3
-#define LB_KINT_CTAS_C3 6
-#endif
-#ifndef LB_KINT_CTAS_C45
-#define LB_KINT_CTAS_C45 6
-#endif
-constexpr int kKintCtasCls[6] = {LB_KINT_CTAS_C0, LB_KINT_CTAS_C12, LB_KINT_CTAS_C12,
-                                 LB_KINT_CTAS_C3, LB_KINT_CTAS_C45, LB_KINT_CTAS_C45};
-// The x-derivative's class kernels carry the weighted sum besides the
-// integer one and keep the general kernel's budget (64 registers).
-__host__ __device__ constexpr int kint_ctas_per_sm(int cls, bool dx = false) {
-  return (cls < 0 || dx) ? LB_KINT_CTAS_PER_SM : kKintCtasCls[cls];
-}
 
 // K-integral queue entries: the pair's offset within its chunk (chunks hold
-// at most 2^26 pairs) in the low 26 bits, the quadrature rule class of the
-// FP64 Gauss rules (kint_class; 0 otherwise) above them, so that a kernel
+// at most 2^26 pairs) in the low 26 bits, the pair's class
+// and band of work (8 kt_class + kt_band; FP64 tight, 0 otherwise) above them, so that a kernel
 // that takes one class finds its pairs by reading the queue alone.
 constexpr int kTileThreads = LB_TILE_THREADS;
 constexpr int kTile = kTileThreads * LB_ITEMS;     // pairs per tile of the tile kernel
@@ -123,22 +103,18 @@ lb_tiles_kernel(const T* __restrict__ v, int64_t v_stride, const T* __restrict__
         if (tid == 0) S.qbase = atomicAdd(qcount, (unsigned int)c);
         __syncthreads();
         const unsigned int b = S.qbase;
-        unsigned cls = 0;                          // quadrature rule classes of the queued pairs
         for (int j = tid; j < c; j += kTileThreads) {
           const int li = S.list[f0 + j];
           uint32_t cl = 0;
           if constexpr (sizeof(T) == 8) {
             if (mode == MODE_TIGHT) {
-              cl = (uint32_t)kint_class((double)S.sv[li], (double)S.sx[li], DX);   // sv holds |v|
-              cls |= 1u << cl;
+              const double vi = S.sv[li], xi = S.sx[li];           // sv holds |v|
+              const int c6 = kt_class(vi, xi, DX);
+              cl = (uint32_t)(8 * c6 + kt_band(vi, xi, c6));
             }
           }
-          // the pair's offset in the chunk (< 2^26) and its rule class above it
+          // the pair's offset in the chunk (< 2^26) and its key above it
           if (LB_CHECK(b + j < qcap, 4u)) queue[b + j] = (uint32_t)(t0 + li) | (cl << kQueueOffsetBits);
-        }
-        if constexpr (sizeof(T) == 8) {
-          cls = __reduce_or_sync(0xffffffffu, cls);
-          if ((tid & 31) == 0 && cls) atomicOr(qcount + 1, cls);
         }
       }
     }
@@ -146,30 +122,105 @@ lb_tiles_kernel(const T* __restrict__ v, int64_t v_stride, const T* __restrict__
   }
 }
 
-// K integral: one warp per queued pair, 32 pairs per warp batch.  CLS = -1:
-// every queued pair; CLS = c (FP64 Gauss values): the pairs of rule class c
-// only, with that class's code alone compiled in (the kernel returns at once
-// when the queue holds none of them).
-template <bool GAUSS, bool DX, typename T, int CLS = -1>
-__global__ void __launch_bounds__(LB_THREADS, kint_ctas_per_sm(CLS, DX))
+// K integral, tight FP64: one thread per queued pair (lb_ktrap.cuh).  A
+// block takes windows of the queue, sorts each by the pairs' classes and
+// bands in shared memory (a counting sort of 48 keys) and hands out chunks of
+// 32 pairs of one class to its warps, costliest class first, so that a warp
+// runs one class's code on lanes that need about as many nodes.  The order of
+// a key's pairs varies from run to run; a pair's result depends on the pair
+// alone.  A window is the queue's share of a block, at most 2048.
+constexpr int kKtWindow = 2048;
+template <bool DX>
+__global__ void __launch_bounds__(LB_THREADS, LB_KTRAP_CTAS_PER_SM)
+lb_ktrap_kernel(const double* __restrict__ v, int64_t v_stride, const double* __restrict__ x,
+                double* __restrict__ out, const unsigned int* __restrict__ qcount,
+                const uint32_t* __restrict__ queue, int64_t n, int64_t qcap) {
+  constexpr int kPer = kKtWindow / LB_THREADS;
+  __shared__ __align__(16) unsigned long long tab[2048];
+  __shared__ uint32_t list[kKtWindow];
+  __shared__ int count[64], beg[64], next_chunk;
+  unsigned int cnt = *qcount;
+  if (!LB_CHECK(cnt <= qcap, 8u)) cnt = (unsigned int)qcap;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int64_t share = (((int64_t)cnt + gridDim.x - 1) / gridDim.x + 31) & ~(int64_t)31;
+  const int W = (int)(share < kKtWindow ? share : kKtWindow);
+  if ((int64_t)blockIdx.x * W >= (int64_t)cnt) return;     // the same for every thread of the block
+  kt_load_table<LB_THREADS>(tab);
+  for (int64_t w0 = (int64_t)blockIdx.x * W; w0 < (int64_t)cnt; w0 += (int64_t)gridDim.x * W) {
+    const int m = (int)min((int64_t)W, (int64_t)cnt - w0);
+    if (tid < 64) count[tid] = 0;
+    if (tid == 0) next_chunk = 0;
+    __syncthreads();
+    uint32_t ent[kPer];
+    int rank[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int j = tid + q * LB_THREADS;
+      rank[q] = -1;
+      if (j < m) {
+        uint32_t e = queue[w0 + j];
+        if (!LB_CHECK((e >> kQueueOffsetBits) < 48u, 32u)) e &= kQueueOffsetMask;
+        ent[q] = e;
+        if (LB_CHECK((int64_t)(e & kQueueOffsetMask) < n, 16u)) rank[q] = atomicAdd(&count[e >> kQueueOffsetBits], 1);
+      }
+    }
+    __syncthreads();
+    if (tid < 32) {                                // exclusive prefix over the 64 key slots
+      const int a = count[2 * lane], b = count[2 * lane + 1];
+      int p = a + b;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, p, o);
+        if (lane >= o) p += u;
+      }
+      beg[2 * lane] = p - a - b;
+      beg[2 * lane + 1] = p - b;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kPer; ++q)
+      if (rank[q] >= 0) list[beg[ent[q] >> kQueueOffsetBits] + rank[q]] = ent[q] & kQueueOffsetMask;
+    __syncthreads();
+    for (;;) {
+      int ch = 0;
+      if (lane == 0) ch = atomicAdd(&next_chunk, 1);
+      ch = __shfl_sync(0xffffffffu, ch, 0);
+      // the chunk's class: chunks hold pairs of one class
+      int c = 0, b = 0, e = 0;
+#pragma unroll 1
+      for (; c < 6; ++c) {
+        b = beg[8 * c];
+        e = beg[8 * c + 8];                        // 8 * 6 = 48: the end of the last class
+        const int nc = (e - b + 31) >> 5;
+        if (ch < nc) break;
+        ch -= nc;
+      }
+      if (c == 6) break;
+      const int j = b + (ch << 5) + lane;
+      if (j < e) {
+        const int64_t idx = (int64_t)list[j];
+        out[idx] = kt_eval<DX>(fabs(v[idx * v_stride]), x[idx], c, tab);
+      }
+      __syncwarp();
+    }
+    __syncthreads();
+  }
+}
+
+// K integral of the paper's dispatches (FP64, Simpson's rule) and of the
+// FP32-mixed form (Gauss rules): one warp per queued pair, 32 pairs per warp
+// batch, in queue order.
+template <typename T>
+__global__ void __launch_bounds__(LB_THREADS, LB_KINT_CTAS_PER_SM)
 lb_kint_kernel(const T* __restrict__ v, int64_t v_stride, const T* __restrict__ x, T* __restrict__ out,
                const unsigned int* __restrict__ qcount, const uint32_t* __restrict__ queue, int64_t n,
                int64_t qcap) {
   unsigned int cnt = *qcount;
   if (!LB_CHECK(cnt <= qcap, 8u)) cnt = (unsigned int)qcap;
-  const unsigned present = (GAUSS && sizeof(T) == 8) ? qcount[1] : 0u;
-  if (CLS >= 0 && !(present & (1u << CLS))) return;     // the same for every thread of the grid
   const int lane = threadIdx.x & 31;
-  const KintScalar* ks = nullptr;
   const KintScalar32* ks32 = nullptr;
-  if constexpr (GAUSS && sizeof(T) == 8) {
+  if constexpr (sizeof(T) == 4) {
     // one order for every pair: its node positions once per block
-    __shared__ KintScalar KS;
-    if (v_stride == 0 && cnt > 0) {
-      kint_scalar_setup(KS, fabs((double)v[0]));
-      ks = &KS;
-    }
-  } else if constexpr (GAUSS && sizeof(T) == 4) {
     __shared__ KintScalar32 KS32;
     if (v_stride == 0 && cnt > 0) {
       kint_scalar_setup32(KS32, fabsf((float)v[0]));
@@ -178,66 +229,15 @@ lb_kint_kernel(const T* __restrict__ v, int64_t v_stride, const T* __restrict__ 
   }
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  // FP64 Gauss rules with pairs of several quadrature rule classes queued
-  // (split, 64 and 32 g nodes, packed, the two one-slot rules; the tile
-  // kernel marks the classes it queues): the queue is processed in phases,
-  // one present class each, costliest first: in phase c a warp scans its
-  // windows of the queue (256 pairs when the queue gives every warp a full
-  // window, else 32) for the pairs of class c, collects them in a ring in
-  // its slice of shared memory and evaluates them 32 at a time.  So the
-  // warps of an SM run one rule's code at a time; with the classes mixed,
-  // every warp switching between up to six code paths, the instruction
-  // cache thrashed (the K call of the robustness sweep took 2.2x the time of
-  // its rule classes evaluated one after another).  A phase re-reads the
-  // queue only, 4 bytes per pair: each entry carries its pair's class.  A pair's result
-  // does not depend on its batch.  A queue of one class, and the other
-  // kernels, take the queue in order, 32 pairs at a time.  A class kernel
-  // is one phase of this: the host launches the six, costliest first.
-  __shared__ uint32_t ring[LB_THREADS / 32][512];
-  uint32_t* my = ring[threadIdx.x >> 5];
-  const bool phased = __popc(present) > 1;
-  const int P = phased && (int64_t)cnt >= nwarps * 256 ? 256 : 32;
-  const int nphase = (phased && CLS < 0) ? 6 : 1;
-  const unsigned lt = (1u << lane) - 1u;
-  unsigned head = 0, nb = 0;                       // ring: first entry, entries held (warp-uniform)
-  for (int ph = 0; ph < nphase; ++ph) {
-    // costliest class first; -1: every pair
-    const int c = !phased ? -1 : (CLS >= 0 ? CLS : (ph == 0 ? 0 : 6 - ph));
-    if (phased && !(present & (1u << c))) continue;
-    for (int64_t b = warp * P;; b += nwarps * P) {
-      const bool last = b >= (int64_t)cnt;
-      if (!last) {
-        const int m = (int)min((int64_t)P, (int64_t)cnt - b);
-        for (int j = 0; 32 * j < m; ++j) {
-          const int t = 32 * j + lane;
-          uint32_t id = 0;
-          int cl = -1;
-          if (t < m) {
-            const uint32_t e = queue[b + t];       // offset and rule class: no gather of v and x to scan
-            id = e & kQueueOffsetMask;
-            cl = (int)(e >> kQueueOffsetBits);
-            if (!LB_CHECK(cl <= 5, 32u)) cl = 0;
-          }
-          const bool take = t < m && (c < 0 || cl == c) && LB_CHECK((int64_t)id < n, 16u);
-          const unsigned mk = __ballot_sync(0xffffffffu, take);
-          if (take) my[(head + nb + __popc(mk & lt)) & 511u] = id;   // nb <= 31 + 256 < 512: no overrun
-          nb += __popc(mk);
-        }
-        __syncwarp();
-      }
-      while (nb >= 32 || (last && nb > 0)) {
-        const int k = nb < 32 ? (int)nb : 32;
-        const int64_t idx = (int64_t)my[(head + (lane < k ? lane : 0)) & 511u];
-        const T vi = fabs(v[idx * v_stride]);
-        const T xi = x[idx];
-        const T val = kint_warp_batch<DX, T, CLS>(vi, xi, k, lane, GAUSS, ks, ks32);
-        if (lane < k) out[idx] = val;
-        head += k;
-        nb -= k;
-      }
-      __syncwarp();
-      if (last) break;
-    }
+  for (int64_t b = warp * 32; b < (int64_t)cnt; b += nwarps * 32) {
+    const int k = (int)min((int64_t)32, (int64_t)cnt - b);
+    int64_t idx = (int64_t)(queue[b + (lane < k ? lane : 0)] & kQueueOffsetMask);
+    const bool ok = LB_CHECK(idx < n, 16u);
+    if (!ok) idx = 0;                              // clamped: the warp still runs the batch together
+    const T vi = fabs(v[idx * v_stride]);
+    const T xi = x[idx];
+    const T val = kint_warp_batch<T>(vi, xi, k, lane, ks32);
+    if (lane < k && ok) out[idx] = val;
   }
 }
 
@@ -426,29 +426,6 @@ lb_status validate(lb_dtype dtype, const void* v, int64_t v_stride, const void* 
   return LB_OK;
 }
 
-template <bool DX, typename T, int CLS>
-lb_status launch_kint_class(int sms, cudaStream_t st, const T* v, int64_t v_stride, const T* x, T* out,
-                            const unsigned int* qcount, const uint32_t* queue, int64_t n, int64_t qcap) {
-  const int grid = sms * 2 * kint_ctas_per_sm(CLS, DX);
-  return launch(PS_KINT, st, [&] {
-    lb_kint_kernel<true, DX, T, CLS><<<grid, LB_THREADS, 0, st>>>(v, v_stride, x, out, qcount, queue, n, qcap);
-  });
-}
-
-// The six class kernels of the FP64 Gauss rules (values or x-derivatives),
-// in the order of the phases.
-template <bool DX, typename T>
-lb_status launch_kint_classes(int sms, cudaStream_t st, const T* v, int64_t v_stride, const T* x, T* out,
-                              const unsigned int* qcount, const uint32_t* queue, int64_t n, int64_t qcap) {
-  lb_status s = launch_kint_class<DX, T, 0>(sms, st, v, v_stride, x, out, qcount, queue, n, qcap);
-  if (s == LB_OK) s = launch_kint_class<DX, T, 5>(sms, st, v, v_stride, x, out, qcount, queue, n, qcap);
-  if (s == LB_OK) s = launch_kint_class<DX, T, 4>(sms, st, v, v_stride, x, out, qcount, queue, n, qcap);
-  if (s == LB_OK) s = launch_kint_class<DX, T, 3>(sms, st, v, v_stride, x, out, qcount, queue, n, qcap);
-  if (s == LB_OK) s = launch_kint_class<DX, T, 2>(sms, st, v, v_stride, x, out, qcount, queue, n, qcap);
-  if (s == LB_OK) s = launch_kint_class<DX, T, 1>(sms, st, v, v_stride, x, out, qcount, queue, n, qcap);
-  return s;
-}
-
 // Largest chunk handled with one queue: the queue entries hold 26-bit offsets.
 const int64_t kChunk = (int64_t)1 << kQueueOffsetBits;
 // Smallest caller workspace: the counters and the queue of one tile.
@@ -456,8 +433,7 @@ const int64_t kWsMin = 256 + 4 * kTile;
 static_assert(256 + 4 * kTile == 8448, "the documented smallest workspace");
 
 // Enqueue the evaluation of n pairs.  The K fallback goes through a queue
-// of 32-bit pair offsets in scratch memory (qcount: the counter and the
-// mask of the quadrature rule classes queued, queue:
+// of 32-bit pair offsets in scratch memory (qcount: the counter, queue:
 // min(n, chunk) entries), processed chunk by chunk; `scratch` supplies it,
 // or, when NULL, it comes from the stream-ordered allocator.
 template <int KIND, bool DX, typename T>
@@ -494,7 +470,7 @@ lb_status run_impl(const T* v, int64_t v_stride, const T* x, T* out, int64_t n, 
   lb_status status = LB_OK;
   for (int64_t c0 = 0; c0 < n && status == LB_OK; c0 += chunk) {
     const int64_t cn = (n - c0) < chunk ? (n - c0) : chunk;
-    if (cudaMemsetAsync(qcount, 0, 2 * sizeof(unsigned int), st) != cudaSuccess) { status = check_launch("cudaMemsetAsync"); break; }
+    if (cudaMemsetAsync(qcount, 0, sizeof(unsigned int), st) != cudaSuccess) { status = check_launch("cudaMemsetAsync"); break; }
     const T* vc = v + c0 * v_stride;
     const T* xc = x + c0;
     T* oc = out + c0;
@@ -512,18 +488,19 @@ lb_status run_impl(const T* v, int64_t v_stride, const T* x, T* out, int64_t n, 
     bool done = false;
     if constexpr (sizeof(T) == 8) {
       if (mode == MODE_TIGHT) {
-        // one kernel per rule class, costliest first (the phases of a mixed queue)
-        status = launch_kint_classes<DX, T>(sms, st, vc, v_stride, xc, oc, qcount, queue, cn, cap);
+        // the queue's length is on the device: a block per 32 pairs it can hold, at most the resident ones
+        const int64_t want = (cn + 31) / 32, most = (int64_t)sms * LB_KTRAP_CTAS_PER_SM;
+        const int kgrid = (int)(want < most ? want : most);
+        status = launch(PS_KINT, st, [&] {
+          lb_ktrap_kernel<DX><<<kgrid, LB_THREADS, 0, st>>>(vc, v_stride, xc, oc, qcount, queue, cn, cap);
+        });
         done = true;
       }
     }
     if (!done) {
       const int kgrid = sms * 2 * LB_KINT_CTAS_PER_SM;
       status = launch(PS_KINT, st, [&] {
-        if (mode == MODE_TIGHT)
-          lb_kint_kernel<true, DX, T><<<kgrid, LB_THREADS, 0, st>>>(vc, v_stride, xc, oc, qcount, queue, cn, cap);
-        else
-          lb_kint_kernel<false, DX, T><<<kgrid, LB_THREADS, 0, st>>>(vc, v_stride, xc, oc, qcount, queue, cn, cap);
+        lb_kint_kernel<T><<<kgrid, LB_THREADS, 0, st>>>(vc, v_stride, xc, oc, qcount, queue, cn, cap);
       });
     }
   }
