@@ -38,8 +38,8 @@
 #include "lb_intmath.cuh"
 #include "ktrap_tables.h"
 
-// kt_any is a called function: a copy of its code inlined in every kernel
-// would sit in the middle of the hot classes'.
+// The per-pair functions are called, not inlined: the warps of an SM run
+// several classes at a time out of one instruction cache.
 #if defined(__CUDACC__)
 #define LB_KT_CALL static __device__ __noinline__
 #else
@@ -47,6 +47,18 @@
 #endif
 
 namespace lb {
+
+#if defined(__CUDACC__)
+static __device__ __noinline__ double kt_exp(double y) { return ix_exp(y); }
+LB_IX_FN double kt_log(double z) { return ix_log_call(z); }
+LB_IX_FN double kt_rcp(double z) { return ix_rcp_call(z); }
+LB_IX_FN double kt_rsqrt(double z) { return ix_rsqrt_call(z); }
+#else
+LB_IX_FN double kt_exp(double y) { return ix_exp(y); }
+LB_IX_FN double kt_log(double z) { return ix_log(z); }
+LB_IX_FN double kt_rcp(double z) { return ix_rcp(z); }
+LB_IX_FN double kt_rsqrt(double z) { return ix_rsqrt(z); }
+#endif
 
 constexpr double kKtLn2 = 0.693147180559945309417232121458;
 
@@ -99,8 +111,9 @@ LB_IX_FN uint64_t kt_root(int j) {
 // A is the factor that grows on a side (a to the right of the maximum, b to
 // the left) times 2^(j/M), B the one that shrinks; A[j] >> sa is in Q54, so
 // A 2^(i + j/M) is A[j] >> (sa - i).  Each side goes on by groups of M nodes
-// to the first whose last term is below 2^-59.  While terms are above that,
-// the growing factor stays below 2^8 through the end of its group (v <= 16.5,
+// to the first whose last term is below 2^-54 (what follows it is below
+// 2^-57 of the sum).  While terms are above that, the
+// growing factor stays below 2^8 through the end of its group (v <= 16.5,
 // r <= 30.1), so sa - i - 1 >= 0.
 template <int M, bool DX>
 LB_IX_FN void kt_sum(double v, double a2, double b2, const unsigned long long* tab, uint64_t& S, uint64_t& G) {
@@ -121,10 +134,9 @@ LB_IX_FN void kt_sum(double v, double a2, double b2, const unsigned long long* t
   G = (uint64_t)base + 1;
 #pragma unroll 1
   for (int side = 0; side < 2; ++side) {                    // one copy of the code for both sides
-    int64_t c = base;
+    int64_t c = base, N = 0;
 #pragma unroll 1
-    for (int i = 0; i < 64; ++i) {
-      int64_t N = 0;
+    for (int i = 0; i < 64 && N >= -(54ll << 54); ++i) {
       const int s0 = sa - i, s1 = s0 > 1 ? s0 - 1 : 0, sd = sb + i + 1 < 63 ? sb + i + 1 : 63;
 #pragma unroll
       for (int j = 1; j <= M; ++j) {
@@ -136,7 +148,6 @@ LB_IX_FN void kt_sum(double v, double a2, double b2, const unsigned long long* t
         if (DX) G += ix_umulhi(w << 6, (uint64_t)t + 1);    // + 1: the two shifts' mean truncation; w < 2^58
       }
       if (DX) G += M / 2;                                   // the products' mean truncation
-      if (N < -(59ll << 54)) break;
     }
 #pragma unroll
     for (int j = 0; j < M; ++j) {
@@ -154,7 +165,7 @@ LB_IX_FN void kt_sum(double v, double a2, double b2, const unsigned long long* t
 // n / d with the reciprocal's and the product's rounding corrected by the
 // remainder (quotients above 2^993 as they come, infinities among them).
 LB_IX_FN double kt_div(double n, double d) {
-  const double r = ix_rcp(d), q = n * r;
+  const double r = kt_rcp(d), q = n * r;
   if ((ix_bits(q) & 0x7fffffffffffffffull) >= 0x7e00000000000000ull) return q;
   return fma(r, fma(-q, d, n), q);
 }
@@ -168,7 +179,7 @@ template <bool DX>
 LB_IX_FN double kt_small(double v, double x) {
   const int n = (int)(v + 0.5);
   double mu = v - (double)n;
-  const double L = kKtLn2 - ix_log(x);                      // log(2/x) >= 6.9
+  const double L = kKtLn2 - kt_log(x);                      // log(2/x) >= 6.9
   const int64_t mq = ix_fix(mu, 62);
   const int64_t m2 = ix_mulhi(mq, mq) << 4;                 // mu^2, Q64
   int64_t q1 = LB_KT_G1_8, q2 = LB_KT_G2_8;
@@ -190,9 +201,9 @@ LB_IX_FN double kt_small(double v, double x) {
   q2 = LB_KT_G2_0 + ix_mulhi(q2, m2);
   const double G1 = (double)q1 * 0x1p-62, G2 = (double)q2 * 0x1p-62;
   const double mg = mu * G1;
-  const double gp = ix_rcp(G2 - mg), gm = ix_rcp(G2 + mg);   // Gamma(1 + mu), Gamma(1 - mu)
+  const double gp = kt_rcp(G2 - mg), gm = kt_rcp(G2 + mg);   // Gamma(1 + mu), Gamma(1 - mu)
   const double s = mu * L;
-  const double ep = ix_exp(s), em = ix_rcp(ep);
+  const double ep = kt_exp(s), em = kt_rcp(ep);
   double shc;                                               // sinh(s) / s
   if (fabs(s) < 0.5) {
     const double z = s * s;
@@ -205,7 +216,7 @@ LB_IX_FN double kt_small(double v, double x) {
     shc = fma(shc, z, 1.0 / 6.0);
     shc = fma(shc, z, 1.0);
   } else {
-    shc = (ep - em) * (0.5 * ix_rcp(fabs(s)));
+    shc = (ep - em) * (0.5 * kt_rcp(fabs(s)));
     shc = s < 0.0 ? -shc : shc;
   }
   double f = gp * gm * fma(0.5 * (ep + em), G1, shc * L * G2);
@@ -218,7 +229,7 @@ LB_IX_FN double kt_small(double v, double x) {
   }
   const double y = 0.25 * x * x;
   const double w = mu * mu;
-  const double r1 = ix_rcp(1.0 - w), r2 = ix_rcp(4.0 - w);
+  const double r1 = kt_rcp(1.0 - w), r2 = kt_rcp(4.0 - w);
   double s0 = f, s1 = p;
   f = (f + p + q) * r1;                                     // k = 1: c = y
   p *= (1.0 + mu) * r1;
@@ -232,8 +243,8 @@ LB_IX_FN double kt_small(double v, double x) {
   s1 = fma(c2, fma(-2.0, f, p), s1);
   // s0 = K_mu, s1 = (x/2) K_(mu+1); d/dx log K_v = -v/x - K_(v-1)/K_v
   if (n == 0) {
-    if (DX) return -kt_div(fma(2.0 * s1, ix_rcp(s0), v), x);
-    return ix_log(s0);
+    if (DX) return -kt_div(fma(2.0 * s1, kt_rcp(s0), v), x);
+    return kt_log(s0);
   }
   double u = mu + 1.0;
 #pragma unroll 1
@@ -243,8 +254,8 @@ LB_IX_FN double kt_small(double v, double x) {
     s1 = t;
     u += 1.0;
   }
-  if (DX) return -kt_div(fma(2.0 * y * s0, ix_rcp(s1), v), x);
-  return fma((double)n, L, ix_log(s1));
+  if (DX) return -kt_div(fma(2.0 * y * s0, kt_rcp(s1), v), x);
+  return fma((double)n, L, kt_log(s1));
 }
 
 // Any (v, x) with finite r (pairs outside the other classes' ranges, which
@@ -309,8 +320,8 @@ LB_IX_FN double kt_eval(double v, double x, int cls, const unsigned long long* t
   if (cls == 2) return kt_small<DX>(v, x);
   if (cls == 0) return kt_any<DX>(v, x);
   const double r2 = fma(v, v, x * x);
-  const double a2 = fma(r2, ix_rsqrt(r2), v);               // r + v = 2a
-  const double b2 = x * x * ix_rcp(a2);                     // r - v = 2b
+  const double a2 = fma(r2, kt_rsqrt(r2), v);               // r + v = 2a
+  const double b2 = x * x * kt_rcp(a2);                     // r - v = 2b
   uint64_t S, G;
   switch (cls) {
     case 1: kt_sum<3, DX>(v, a2, b2, tab, S, G); break;
@@ -322,7 +333,7 @@ LB_IX_FN double kt_eval(double v, double x, int cls, const unsigned long long* t
   if (DX) return -kt_div((double)ix_umulhi(G, 0xb17217f7d1cf79acull) * 16.0, (double)S * x);
   // h/2 = ln2 / (2m)
   const double hh = cls == 1 ? kKtLn2 / 6.0 : (cls == 5 ? kKtLn2 / 8.0 : (cls == 4 ? kKtLn2 / 10.0 : kKtLn2 / 12.0));
-  return fma(v, ix_log(a2 * ix_rcp(x)), fma(-0.5, a2 + b2, ix_log((double)S * (0x1p-58 * hh))));
+  return fma(v, kt_log(a2 * kt_rcp(x)), fma(-0.5, a2 + b2, kt_log((double)S * (0x1p-58 * hh))));
 }
 
 }  // namespace lb

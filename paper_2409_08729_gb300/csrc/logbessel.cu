@@ -58,8 +58,12 @@ namespace {
 #define LB_KINT_CTAS_PER_SM 4
 #endif
 #ifndef LB_KTRAP_CTAS_PER_SM
-#define LB_KTRAP_CTAS_PER_SM 4
+#define LB_KTRAP_CTAS_PER_SM 6
 #endif
+#ifndef LB_KTRAP_CTAS_PER_SM_DX
+#define LB_KTRAP_CTAS_PER_SM_DX 4
+#endif
+__host__ __device__ constexpr int ktrap_ctas(bool dx) { return dx ? LB_KTRAP_CTAS_PER_SM_DX : LB_KTRAP_CTAS_PER_SM; }
 
 // K-integral queue entries: the pair's offset within its chunk (chunks hold
 // at most 2^26 pairs) in the low 26 bits, the pair's class
@@ -131,7 +135,7 @@ lb_tiles_kernel(const T* __restrict__ v, int64_t v_stride, const T* __restrict__
 // alone.  A window is the queue's share of a block, at most 2048.
 constexpr int kKtWindow = 2048;
 template <bool DX>
-__global__ void __launch_bounds__(LB_THREADS, LB_KTRAP_CTAS_PER_SM)
+__global__ void __launch_bounds__(LB_THREADS, ktrap_ctas(DX))
 lb_ktrap_kernel(const double* __restrict__ v, int64_t v_stride, const double* __restrict__ x,
                 double* __restrict__ out, const unsigned int* __restrict__ qcount,
                 const uint32_t* __restrict__ queue, int64_t n, int64_t qcap) {
@@ -142,8 +146,10 @@ lb_ktrap_kernel(const double* __restrict__ v, int64_t v_stride, const double* __
   unsigned int cnt = *qcount;
   if (!LB_CHECK(cnt <= qcap, 8u)) cnt = (unsigned int)qcap;
   const int tid = threadIdx.x, lane = tid & 31;
-  const int64_t share = (((int64_t)cnt + gridDim.x - 1) / gridDim.x + 31) & ~(int64_t)31;
-  const int W = (int)(share < kKtWindow ? share : kKtWindow);
+  // equal windows: as many per block as the queue needs, so that no block's last one is short
+  const int64_t share = ((int64_t)cnt + gridDim.x - 1) / gridDim.x;
+  const int64_t rounds = (share + kKtWindow - 1) / kKtWindow;
+  const int W = rounds ? (int)(((share + rounds - 1) / rounds + 31) & ~(int64_t)31) : 32;
   if ((int64_t)blockIdx.x * W >= (int64_t)cnt) return;     // the same for every thread of the block
   kt_load_table<LB_THREADS>(tab);
   for (int64_t w0 = (int64_t)blockIdx.x * W; w0 < (int64_t)cnt; w0 += (int64_t)gridDim.x * W) {
@@ -489,7 +495,7 @@ lb_status run_impl(const T* v, int64_t v_stride, const T* x, T* out, int64_t n, 
     if constexpr (sizeof(T) == 8) {
       if (mode == MODE_TIGHT) {
         // the queue's length is on the device: a block per 32 pairs it can hold, at most the resident ones
-        const int64_t want = (cn + 31) / 32, most = (int64_t)sms * LB_KTRAP_CTAS_PER_SM;
+        const int64_t want = (cn + 31) / 32, most = (int64_t)sms * ktrap_ctas(DX);
         const int kgrid = (int)(want < most ? want : most);
         status = launch(PS_KINT, st, [&] {
           lb_ktrap_kernel<DX><<<kgrid, LB_THREADS, 0, st>>>(vc, v_stride, xc, oc, qcount, queue, cn, cap);
