@@ -104,7 +104,7 @@ union ServeShared {
   TileShared<double, LB_THREADS> d;
   TileShared<float, LB_THREADS> f;
   __align__(16) unsigned long long kt[2048];
-  KintScalar32 ks32;
+  Warp32 w32[LB_THREADS / 32];
 };
 
 struct ServeAux {          // per-tile class counts and queue bases of the K pairs
@@ -125,7 +125,7 @@ __device__ __forceinline__ void serve_tile(TileShared<T, LB_THREADS>& S, ServeAu
   const int tid = threadIdx.x;
   tile_bin<KIND, false, T>(S, v, d.v_stride, x, t0, d.n, d.mode, -1);
   tile_eval<KIND, false, T>(S, out, t0, d.n);
-  if (KIND == KIND_K) {
+  if (KIND == KIND_K && sizeof(T) == 8) {
     const int c = S.rcount(R_FALLBACK), f0 = S.rbeg(R_FALLBACK);
     if (c > 0) {                                   // block-uniform
       if (tid < 8) A.kc[tid] = 0;
@@ -159,41 +159,28 @@ __device__ __forceinline__ void serve_tile(TileShared<T, LB_THREADS>& S, ServeAu
   __syncthreads();
 }
 
-// Stage B: a window [q0, q1) of one class queue: one pair per thread (FP64,
-// tight mode), or 32 pairs per warp batch.
-template <typename T>
+// Stage B (FP64): a window [q0, q1) of one class queue, one pair per thread
+// (tight mode) or 32 pairs per warp batch.
 __device__ __forceinline__ void serve_kwindow(ServeShared& U, const SlotDesc& d, int cls, int q0, int q1) {
-  const T* v = reinterpret_cast<const T*>(d.v);
-  const T* x = reinterpret_cast<const T*>(d.x);
-  T* out = reinterpret_cast<T*>(d.out);
+  const double* v = reinterpret_cast<const double*>(d.v);
+  const double* x = reinterpret_cast<const double*>(d.x);
+  double* out = reinterpret_cast<double*>(d.out);
   const uint32_t* queue = reinterpret_cast<const uint32_t*>(d.queue) + (int64_t)cls * d.n;
-  if constexpr (sizeof(T) == 8) {
-    if (d.mode == MODE_TIGHT) {
-      kt_load_table<LB_THREADS>(U.kt);
-      __syncthreads();
-      for (int j = q0 + (int)threadIdx.x; j < q1; j += LB_THREADS) {
-        const int64_t idx = (int64_t)queue[j];
-        out[idx] = kt_eval<false>(fabs(v[idx * d.v_stride]), x[idx], cls, U.kt);
-      }
-      __syncthreads();                             // U is reused by the next item
-      return;
+  if (d.mode == MODE_TIGHT) {
+    kt_load_table<LB_THREADS>(U.kt);
+    __syncthreads();
+    for (int j = q0 + (int)threadIdx.x; j < q1; j += LB_THREADS) {
+      const int64_t idx = (int64_t)queue[j];
+      out[idx] = kt_eval<false>(fabs(v[idx * d.v_stride]), x[idx], cls, U.kt);
     }
-  }
-  const KintScalar32* ks32 = nullptr;
-  if constexpr (sizeof(T) == 4) {
-    if (d.v_stride == 0) {                         // one order for all pairs: its node table once
-      kint_scalar_setup32(U.ks32, fabsf((float)v[0]));
-      ks32 = &U.ks32;
+  } else {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int b = q0 + 32 * warp; b < q1; b += LB_THREADS) {
+      const int k = min(32, q1 - b);
+      const int64_t idx = (int64_t)queue[b + (lane < k ? lane : 0)];
+      const double val = kint_warp_batch(fabs(v[idx * d.v_stride]), x[idx], k, lane);
+      if (lane < k) out[idx] = val;
     }
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int b = q0 + 32 * warp; b < q1; b += LB_THREADS) {
-    const int k = min(32, q1 - b);
-    const int64_t idx = (int64_t)queue[b + (lane < k ? lane : 0)];
-    const T vi = fabs(v[idx * d.v_stride]);
-    const T xi = x[idx];
-    const T val = kint_warp_batch<T>(vi, xi, k, lane, ks32);
-    if (lane < k) out[idx] = val;
   }
   __syncthreads();                                 // U is reused by the next item
 }
@@ -259,13 +246,30 @@ lb_serve_kernel(Ctl* ctl, const SlotDesc* slots, const WorkItem* ring, int ring_
     const WorkItem it = item;
     unsigned* qc = qcount + 8 * it.slot;
     if (it.type == 0) {
-      for (int64_t tile = it.begin; tile < it.end; ++tile) {
-        if (d.dtype == LB_F64) {
-          if (d.kind == 0) serve_tile<KIND_I, double>(U.d, A, d, tile, qc);
-          else serve_tile<KIND_K, double>(U.d, A, d, tile, qc);
+      if (d.dtype == LB_F32 && d.mode == MODE_TIGHT) {
+        // the item's pairs as one range: the warps take its slices in turn
+        const float *v = reinterpret_cast<const float*>(d.v), *x = reinterpret_cast<const float*>(d.x);
+        float* out = reinterpret_cast<float*>(d.out);
+        const int64_t p0 = (int64_t)it.begin * LB_TILE, p1 = min((int64_t)it.end * LB_TILE, (int64_t)d.n);
+        const bool wide = ((d.x | d.out | (d.v_stride ? d.v : 0)) & 15) == 0;
+        const int w = threadIdx.x >> 5;
+        if (d.kind == 0) {
+          if (wide) warp_pairs32<KIND_I, 4>(U.w32[w], v, d.v_stride, x, out, p0, p1, w, LB_THREADS / 32);
+          else warp_pairs32<KIND_I, 1>(U.w32[w], v, d.v_stride, x, out, p0, p1, w, LB_THREADS / 32);
         } else {
-          if (d.kind == 0) serve_tile<KIND_I, float>(U.f, A, d, tile, qc);
-          else serve_tile<KIND_K, float>(U.f, A, d, tile, qc);
+          if (wide) warp_pairs32<KIND_K, 4>(U.w32[w], v, d.v_stride, x, out, p0, p1, w, LB_THREADS / 32);
+          else warp_pairs32<KIND_K, 1>(U.w32[w], v, d.v_stride, x, out, p0, p1, w, LB_THREADS / 32);
+        }
+        __syncthreads();
+      } else {
+        for (int64_t tile = it.begin; tile < it.end; ++tile) {
+          if (d.dtype == LB_F32) {
+            serve_tile<KIND_I, float>(U.f, A, d, tile, qc);   // FP32 log K is served in tight mode only
+          } else if (d.kind == 0) {
+            serve_tile<KIND_I, double>(U.d, A, d, tile, qc);
+          } else {
+            serve_tile<KIND_K, double>(U.d, A, d, tile, qc);
+          }
         }
       }
       if (threadIdx.x == 0) {
@@ -288,8 +292,7 @@ lb_serve_kernel(Ctl* ctl, const SlotDesc* slots, const WorkItem* ring, int ring_
         }
       }
     } else {
-      if (d.dtype == LB_F64) serve_kwindow<double>(U, d, it.type - 1, it.begin, it.end);
-      else serve_kwindow<float>(U, d, it.type - 1, it.begin, it.end);
+      serve_kwindow(U, d, it.type - 1, it.begin, it.end);
       if (threadIdx.x == 0) {
         __threadfence();
         const long long old = atomicAdd((unsigned long long*)&kdone[it.slot], 1ull);

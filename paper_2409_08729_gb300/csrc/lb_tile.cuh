@@ -15,7 +15,7 @@
 //              that need about the same number of terms; then stores the
 //              tile's results coalesced (two per store instruction).
 // The per-call kernels (logbessel.cu) and the persistent serving kernel
-// (lb_serve.cu) are both built from these two steps; K pairs of the
+// (lb_serve.cu) are both built from these two steps; FP64 K pairs of the
 // fallback region are left in the list for the K integral.
 #pragma once
 
@@ -128,7 +128,7 @@ __device__ __forceinline__ T tile_expr(int r, T v, T x, int n) {
       case R_U4: return u_expr32<KIND, 4>(v, x);
       case R_U6: return u_expr32<KIND, 6>(v, x);
       case R_U9: return u_expr32<KIND, 9>(v, x);
-      default: return (KIND == KIND_I) ? series_log_i32(v, x) : __int_as_float(0x7fc00000);
+      default: return (KIND == KIND_I) ? series_log_i32(v, x) : kt_log_k32(v, x);
     }
   } else if constexpr (DX) {
     switch (r) {
@@ -249,7 +249,7 @@ __device__ __forceinline__ void tile_bin(TileShared<T, NT>& S, const T* __restri
         int nterm;
         k = tile_key<KIND, DX, T>(r, vi, xi, &nterm);
         S.nt[li] = (uint8_t)nterm;
-        keep = (KIND == KIND_K && r == R_FALLBACK) ? 0 : 1;   // K integral pairs are stored later
+        keep = (KIND == KIND_K && sizeof(T) == 8 && r == R_FALLBACK) ? 0 : 1;   // FP64 K integral pairs are stored later
       }
     }
     S.keep[li] = keep;
@@ -356,7 +356,7 @@ __device__ __forceinline__ void tile_eval_region(TileShared<T, NT>& S, int lane,
 // close together); every warp runs a single expression at a time, and the
 // result of a pair does not depend on which warp takes its chunk.  Then the
 // tile's results (domain edges included) are stored, two pairs per
-// instruction where both are kept and the buffer is aligned.  The K fallback
+// instruction where both are kept and the buffer is aligned.  The FP64 K fallback
 // pairs are left to the K integral: neither evaluated nor stored (so out may
 // equal x: their arguments stay in place for it).  Ends with a barrier.
 template <int KIND, bool DX, typename T, int NT>
@@ -364,7 +364,7 @@ __device__ __forceinline__ void tile_eval(TileShared<T, NT>& S, T* __restrict__ 
                                           const ScalarOrder* so = nullptr) {
   typedef typename Vec2<T>::type T2;
   const int tid = threadIdx.x, lane = tid & 31;
-  if (KIND == KIND_I) tile_eval_region<KIND, DX, T, R_FALLBACK, NT>(S, lane, so);
+  if (KIND == KIND_I || sizeof(T) == 4) tile_eval_region<KIND, DX, T, R_FALLBACK, NT>(S, lane, so);
   tile_eval_region<KIND, DX, T, R_U13, NT>(S, lane, so);
   tile_eval_region<KIND, DX, T, R_U9, NT>(S, lane, so);
   tile_eval_region<KIND, DX, T, R_MU20, NT>(S, lane, so);
@@ -392,31 +392,16 @@ __device__ __forceinline__ void tile_eval(TileShared<T, NT>& S, T* __restrict__ 
 }
 
 // K integral of a batch of up to 32 pairs by one warp (the paper's Simpson
-// rule in FP64, the Gauss rules in single precision): lane e holds pair e;
-// each lane computes its pair's prefactor, then the warp evaluates the
-// integrals one pair at a time with the nodes spread over the lanes.
-template <typename T>
-__device__ __forceinline__ T kint_warp_batch(T vi, T xi, int m, int lane, const KintScalar32* ks32 = nullptr) {
-  T pre;
-  if constexpr (sizeof(T) == 8) pre = kint_prefactor(vi, xi);
-  else pre = kint_prefactor32(vi, xi);
-  float beta_i = 0.0f, logbeta_i = 0.0f;
-  if constexpr (sizeof(T) == 4) {
-    beta_i = 16.0f / (2.0f * vi + 1.0f);
-    logbeta_i = logf(beta_i);
-  }
-  T mine = 0;
+// rule): lane e holds pair e; each lane computes its pair's prefactor, then
+// the warp evaluates the integrals one pair at a time with the nodes spread
+// over the lanes.
+__device__ __forceinline__ double kint_warp_batch(double vi, double xi, int m, int lane) {
+  const double pre = kint_prefactor(vi, xi);
+  double mine = 0;
   for (int e = 0; e < m; ++e) {
-    const T ve = __shfl_sync(0xffffffffu, vi, e);
-    const T xe = __shfl_sync(0xffffffffu, xi, e);
-    T li;
-    if constexpr (sizeof(T) == 8) {
-      li = kint_log_simpson(ve, xe, lane);
-    } else {
-      const float be = __shfl_sync(0xffffffffu, beta_i, e);
-      const float lbe = __shfl_sync(0xffffffffu, logbeta_i, e);
-      li = kint_gauss32(ve, xe, be, lbe, lane, ks32);
-    }
+    const double ve = __shfl_sync(0xffffffffu, vi, e);
+    const double xe = __shfl_sync(0xffffffffu, xi, e);
+    const double li = kint_log_simpson(ve, xe, lane);
     if (lane == e) mine = li;
   }
   return pre + mine;
@@ -429,6 +414,158 @@ template <int NT>
 __device__ __forceinline__ void kt_load_table(unsigned long long* tab) {
   for (int i = 2 * threadIdx.x; i < 2048; i += 2 * NT)
     *reinterpret_cast<ulonglong2*>(tab + i) = *reinterpret_cast<const ulonglong2*>(lb_kt_exp2 + i);
+}
+
+// FP32 pairs in tight mode (log I or log K).  Each warp works by itself, with
+// no block barrier: it takes slices of 32 VEC adjacent pairs (VEC = 4: one
+// 16-byte load of v and x per lane), evaluates u_all32 where
+// r^2 = v^2 + x^2 >= 14^2, and stores; the other pairs (series or K integral)
+// go to a list of the warp in shared memory, and whenever it holds 256 it is
+// sorted by an estimate of their loops' length (16 keys) and evaluated, 32
+// at a time.  Nothing else is binned: binning every pair by region, as the
+// FP64 tiles do, costs more instructions than the one merged expansion.  A
+// pair's result depends on the pair alone.  The listed pairs' arguments are
+// read again from global memory; their outputs are not written before (out
+// may be x).
+constexpr int kList32 = 256 + 128;                         // entries before a flush, and one slice's
+struct Warp32 {
+  uint32_t raw[kList32], list[kList32];                    // offsets from the base of v, x and out
+  uint8_t rkey[kList32], lkey[kList32];
+  int count[16];
+};
+
+// Sort key of a listed pair, 0 .. 15, in order of decreasing work.
+template <int KIND>
+__device__ __forceinline__ int key32(float v, float x) {
+  if (KIND == KIND_I) return 15 - min(15, (int)(3.8f * __log2f(1.0f + x)));   // term count grows with x
+  if (x < 0x1p-9f) return 15 - min(3, (int)(0.25f * v));
+  const float a2 = v + sqrtf(fmaf(v, v, x * x));
+  const float left = fminf(__log2f(2.0f + __fdividef(36.0f * a2, x * x)), __fdividef(18.0f + 0.5f * a2, 0.7f * v));
+  const int m = kt_step32(v, x);                           // left (2 + m) nodes a side
+  return 4 * m + 3 - max(0, min(3, (int)((left - 3.0f) * 0.25f)));
+}
+
+// Sort the warp's list (cnt entries) and evaluate it; all of it, or (last =
+// false) whole chunks of 32 only.  Returns the entries left in the list.
+template <int KIND>
+__device__ __forceinline__ int flush32(Warp32& W, int cnt, bool last, const float* __restrict__ v, int64_t v_stride,
+                                       const float* __restrict__ x, float* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+  const int c = lane < 16 ? W.count[lane] : 0;
+  int p = c;
+#pragma unroll
+  for (int o = 1; o < 16; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, p, o);
+    if (lane >= o) p += u;
+  }
+  if (lane < 16) W.count[lane] = p - c;                    // where each key's entries begin
+  __syncwarp();
+  for (int j = lane; j < cnt; j += 32) {
+    const int k = W.rkey[j], pos = atomicAdd(&W.count[k], 1);
+    if (LB_CHECK(pos < kList32, 1u)) {
+      W.list[pos] = W.raw[j];
+      W.lkey[pos] = (uint8_t)k;
+    }
+  }
+  __syncwarp();
+  const int m = last ? cnt : cnt & ~31;
+  for (int j = lane; j < m; j += 32) {
+    const int64_t i = W.list[j];
+    const float vi = v[i * v_stride], xi = x[i];
+    out[i] = KIND == KIND_I ? series_all32(vi, xi) : kt_log_k32(fabsf(vi), xi);
+  }
+  __syncwarp();
+  if (lane < 16) W.count[lane] = 0;
+  __syncwarp();
+  if (lane < cnt - m) {
+    const int k = W.lkey[m + lane];
+    W.raw[lane] = W.list[m + lane];
+    W.rkey[lane] = (uint8_t)k;
+    atomicAdd(&W.count[k], 1);
+  }
+  __syncwarp();
+  return cnt - m;
+}
+
+// This warp's share of the pairs [begin, end): slices warp, warp + nwarps, ...
+// Offsets fit 32 bits (the caller's pointers are based accordingly).
+template <int KIND, int VEC>
+__device__ __forceinline__ void warp_pairs32(Warp32& W, const float* __restrict__ v, int64_t v_stride,
+                                             const float* __restrict__ x, float* __restrict__ out, int64_t begin,
+                                             int64_t end, int64_t warp, int64_t nwarps) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  const float v0 = v_stride ? 0.0f : v[0];
+  int cnt = 0;                                             // entries in the list (warp-uniform)
+  if (lane < 16) W.count[lane] = 0;
+  __syncwarp();
+  for (int64_t s = begin + warp * (32 * VEC); s < end; s += nwarps * (32 * VEC)) {
+    const int64_t i = s + lane * VEC;
+    float vv[VEC], xx[VEC], rr[VEC];
+    const bool whole = VEC == 4 && i + 3 < end;
+    if (whole) {
+      const float4 a = *reinterpret_cast<const float4*>(x + i);
+      xx[0] = a.x;
+      if (VEC == 4) { xx[1 % VEC] = a.y; xx[2 % VEC] = a.z; xx[3 % VEC] = a.w; }
+      if (v_stride) {
+        const float4 b = *reinterpret_cast<const float4*>(v + i);
+        vv[0] = b.x;
+        if (VEC == 4) { vv[1 % VEC] = b.y; vv[2 % VEC] = b.z; vv[3 % VEC] = b.w; }
+      } else {
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) vv[e] = v0;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) {
+        xx[e] = i + e < end ? x[i + e] : 50.0f;
+        vv[e] = i + e < end ? (v_stride ? v[i + e] : v0) : 1.0f;
+      }
+    }
+    unsigned fb = 0;                                       // bit e: pair e goes to the list
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) {
+      const float xi = xx[e], vi = KIND == KIND_K ? fabsf(vv[e]) : vv[e];
+      float sp;
+      // one test for the domain edges and for squares out of range
+      if (!(xi > 0.0f && xi <= 1e18f && vi >= 0.0f && vi <= 1e18f)) {
+        if (special_value32<KIND>(vi, xi, &sp)) {
+          rr[e] = sp;
+        } else {
+          const int r = classify32(vi, xi, MODE_TIGHT, KIND == KIND_K ? WIDE_K : WIDE_I);
+          rr[e] = r == R_MU20 ? mu_expr32<KIND, 20>(vi, xi) : u_expr32<KIND, 4>(vi, xi);   // v or x > 1e18
+        }
+      } else {
+        const float s2 = fmaf(vi, vi, xi * xi);
+        if (s2 < kAllR2) fb |= 1u << e;
+        rr[e] = u_all32(KIND, vi, xi, s2);
+      }
+    }
+    if (whole && fb == 0) {
+      if (VEC == 4) *reinterpret_cast<float4*>(out + i) = make_float4(rr[0], rr[1 % VEC], rr[2 % VEC], rr[3 % VEC]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < VEC; ++e)
+        if (i + e < end && !((fb >> e) & 1u)) out[i + e] = rr[e];
+    }
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) {
+      const bool f = ((fb >> e) & 1u) && i + e < end;
+      const unsigned m = __ballot_sync(0xffffffffu, f);
+      if (f) {
+        const int b = cnt + __popc(m & lt), k = key32<KIND>(KIND == KIND_K ? fabsf(vv[e]) : vv[e], xx[e]);
+        if (LB_CHECK(b < kList32, 1u)) {
+          W.raw[b] = (uint32_t)(i + e);
+          W.rkey[b] = (uint8_t)k;
+          atomicAdd(&W.count[k], 1);
+        }
+      }
+      cnt += __popc(m);
+    }
+    if (cnt >= 256) cnt = flush32<KIND>(W, cnt, false, v, v_stride, x, out);
+  }
+  if (cnt > 0) flush32<KIND>(W, cnt, true, v, v_stride, x, out);
 }
 
 }  // namespace lb

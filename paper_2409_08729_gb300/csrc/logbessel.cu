@@ -12,10 +12,11 @@
 //      fallback region are appended to a global queue instead.
 //   2. lb_ktrap_kernel (tight FP64): one thread per queued K pair evaluates the
 //      integral by the trapezoid rule (lb_ktrap.cuh); lb_kint_kernel (the
-//      paper's dispatches, FP32): one warp per pair with the nodes spread over
-//      the lanes (lb_kint.cuh, lb_expr32.cuh).
-// A call with one order for all pairs (v_stride 0) has its order's
-// constants computed once per block (ScalarOrder, KintScalar32).
+//      paper's dispatches): one warp per pair with the nodes spread over the
+//      lanes (lb_kint.cuh).
+// An FP64 call with one order for all pairs (v_stride 0) has its order's
+// constants computed once per block (ScalarOrder).  FP32 calls in tight mode
+// run lb_tiles32_kernel alone.
 //
 // The plain form computes in FP64; its exps and logs are evaluated in
 // integer arithmetic where that is faster (lb_intmath.cuh).
@@ -56,6 +57,9 @@ namespace {
 #endif
 #ifndef LB_KINT_CTAS_PER_SM
 #define LB_KINT_CTAS_PER_SM 4
+#endif
+#ifndef LB_TILES32_CTAS_PER_SM
+#define LB_TILES32_CTAS_PER_SM 6
 #endif
 #ifndef LB_KTRAP_CTAS_PER_SM
 #define LB_KTRAP_CTAS_PER_SM 6
@@ -101,7 +105,7 @@ lb_tiles_kernel(const T* __restrict__ v, int64_t v_stride, const T* __restrict__
     const int64_t t0 = tile * kTile;
     tile_bin<KIND, DX, T>(S, v, v_stride, x, t0, n, mode, forced_region);
     tile_eval<KIND, DX, T>(S, out, t0, n, so);
-    if (KIND == KIND_K) {
+    if (KIND == KIND_K && sizeof(T) == 8) {
       const int c = S.rcount(R_FALLBACK), f0 = S.rbeg(R_FALLBACK);
       if (c > 0) {
         if (tid == 0) S.qbase = atomicAdd(qcount, (unsigned int)c);
@@ -213,26 +217,15 @@ lb_ktrap_kernel(const double* __restrict__ v, int64_t v_stride, const double* __
   }
 }
 
-// K integral of the paper's dispatches (FP64, Simpson's rule) and of the
-// FP32-mixed form (Gauss rules): one warp per queued pair, 32 pairs per warp
-// batch, in queue order.
-template <typename T>
+// K integral of the paper's dispatches (Simpson's rule): one warp per queued
+// pair, 32 pairs per warp batch, in queue order.
 __global__ void __launch_bounds__(LB_THREADS, LB_KINT_CTAS_PER_SM)
-lb_kint_kernel(const T* __restrict__ v, int64_t v_stride, const T* __restrict__ x, T* __restrict__ out,
-               const unsigned int* __restrict__ qcount, const uint32_t* __restrict__ queue, int64_t n,
-               int64_t qcap) {
+lb_kint_kernel(const double* __restrict__ v, int64_t v_stride, const double* __restrict__ x,
+               double* __restrict__ out, const unsigned int* __restrict__ qcount,
+               const uint32_t* __restrict__ queue, int64_t n, int64_t qcap) {
   unsigned int cnt = *qcount;
   if (!LB_CHECK(cnt <= qcap, 8u)) cnt = (unsigned int)qcap;
   const int lane = threadIdx.x & 31;
-  const KintScalar32* ks32 = nullptr;
-  if constexpr (sizeof(T) == 4) {
-    // one order for every pair: its node positions once per block
-    __shared__ KintScalar32 KS32;
-    if (v_stride == 0 && cnt > 0) {
-      kint_scalar_setup32(KS32, fabsf((float)v[0]));
-      ks32 = &KS32;
-    }
-  }
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t b = warp * 32; b < (int64_t)cnt; b += nwarps * 32) {
@@ -240,11 +233,20 @@ lb_kint_kernel(const T* __restrict__ v, int64_t v_stride, const T* __restrict__ 
     int64_t idx = (int64_t)(queue[b + (lane < k ? lane : 0)] & kQueueOffsetMask);
     const bool ok = LB_CHECK(idx < n, 16u);
     if (!ok) idx = 0;                              // clamped: the warp still runs the batch together
-    const T vi = fabs(v[idx * v_stride]);
-    const T xi = x[idx];
-    const T val = kint_warp_batch<T>(vi, xi, k, lane, ks32);
+    const double val = kint_warp_batch(fabs(v[idx * v_stride]), x[idx], k, lane);
     if (lane < k && ok) out[idx] = val;
   }
+}
+
+// FP32, tight mode: see warp_pairs32.
+template <int KIND, int VEC>
+__global__ void __launch_bounds__(LB_THREADS, LB_TILES32_CTAS_PER_SM)
+lb_tiles32_kernel(const float* __restrict__ v, int64_t v_stride, const float* __restrict__ x,
+                  float* __restrict__ out, int64_t n) {
+  __shared__ Warp32 W[LB_THREADS / 32];
+  const int warps = blockDim.x >> 5, w = threadIdx.x >> 5;
+  warp_pairs32<KIND, VEC>(W[w], v, v_stride, x, out, 0, n, (int64_t)w * gridDim.x + blockIdx.x,
+                          (int64_t)warps * gridDim.x);
 }
 
 template <int KIND>
@@ -438,7 +440,31 @@ const int64_t kChunk = (int64_t)1 << kQueueOffsetBits;
 const int64_t kWsMin = 256 + 4 * kTile;
 static_assert(256 + 4 * kTile == 8448, "the documented smallest workspace");
 
-// Enqueue the evaluation of n pairs.  The K fallback goes through a queue
+// FP32, tight mode.  16-byte loads when the pointers allow them and there are
+// enough pairs for every SM's resident warps; otherwise one pair per lane,
+// and slices dealt to the blocks in turn, so that a small call uses as many
+// SMs as it can.  2^31 pairs per launch (32-bit offsets in the lists).
+template <int KIND>
+lb_status run_tiles32(const float* v, int64_t v_stride, const float* x, float* out, int64_t n, cudaStream_t st) {
+  const int64_t most = (int64_t)sm_count() * LB_TILES32_CTAS_PER_SM;
+  const uintptr_t al = (uintptr_t)x | (uintptr_t)out | (v_stride ? (uintptr_t)v : 0);
+  const bool wide = (al & 15) == 0 && n > most * LB_THREADS;
+  lb_status s = LB_OK;
+  for (int64_t c0 = 0; c0 < n && s == LB_OK; c0 += (int64_t)1 << 31) {
+    const int64_t cn = n - c0 < ((int64_t)1 << 31) ? n - c0 : (int64_t)1 << 31;
+    const int64_t slices = (cn + (wide ? 127 : 31)) / (wide ? 128 : 32);
+    const int grid = (int)(slices < most ? slices : most);
+    const int64_t per = (slices + grid - 1) / grid;        // warps a block can use
+    const int threads = (int)(per < LB_THREADS / 32 ? per : LB_THREADS / 32) * 32;
+    s = launch(PS_TILES, st, [&] {
+      if (wide) lb_tiles32_kernel<KIND, 4><<<grid, threads, 0, st>>>(v + c0 * v_stride, v_stride, x + c0, out + c0, cn);
+      else lb_tiles32_kernel<KIND, 1><<<grid, threads, 0, st>>>(v + c0 * v_stride, v_stride, x + c0, out + c0, cn);
+    });
+  }
+  return s;
+}
+
+// Enqueue the evaluation of n pairs.  The FP64 K fallback goes through a queue
 // of 32-bit pair offsets in scratch memory (qcount: the counter, queue:
 // min(n, chunk) entries), processed chunk by chunk; `scratch` supplies it,
 // or, when NULL, it comes from the stream-ordered allocator.
@@ -448,7 +474,12 @@ lb_status run_impl(const T* v, int64_t v_stride, const T* x, T* out, int64_t n, 
   const int sms = sm_count();
   const int64_t ntiles_all = (n + kTile - 1) / kTile;
   const bool per_order = sizeof(T) == 8 && !DX && v_stride == 0 && forced_region < 0;
-  if (KIND == KIND_I || (forced_region >= 0 && forced_region != R_FALLBACK)) {
+  if (KIND == KIND_K && sizeof(T) == 4 && mode != MODE_TIGHT && (forced_region < 0 || forced_region == R_FALLBACK))
+    return fail(LB_ENOTSUP, "%sthe FP32 K integral is implemented for LB_TIGHT only", "", 0);
+  if constexpr (sizeof(T) == 4) {
+    if (mode == MODE_TIGHT && forced_region < 0) return run_tiles32<KIND>(v, v_stride, x, out, n, st);
+  }
+  if (KIND == KIND_I || sizeof(T) == 4 || (forced_region >= 0 && forced_region != R_FALLBACK)) {
     const int grid = (int)(ntiles_all < (int64_t)sms * LB_TILES_CTAS_PER_SM ? ntiles_all : (int64_t)sms * LB_TILES_CTAS_PER_SM);
     return launch(PS_TILES, st, [&] {
       if (per_order)
@@ -459,8 +490,6 @@ lb_status run_impl(const T* v, int64_t v_stride, const T* x, T* out, int64_t n, 
                                                                           forced_region, nullptr, nullptr, 0);
     });
   }
-  if (sizeof(T) == 4 && mode != MODE_TIGHT)
-    return fail(LB_ENOTSUP, "%sthe FP32 K integral is implemented for LB_TIGHT only", "", 0);
   // queue entries a pass can write: every workspace holds at least this many
   const int64_t cap = n < chunk ? n : chunk;
   void* ws = scratch;
@@ -503,11 +532,13 @@ lb_status run_impl(const T* v, int64_t v_stride, const T* x, T* out, int64_t n, 
         done = true;
       }
     }
-    if (!done) {
-      const int kgrid = sms * 2 * LB_KINT_CTAS_PER_SM;
-      status = launch(PS_KINT, st, [&] {
-        lb_kint_kernel<T><<<kgrid, LB_THREADS, 0, st>>>(vc, v_stride, xc, oc, qcount, queue, cn, cap);
-      });
+    if constexpr (sizeof(T) == 8) {
+      if (!done) {
+        const int kgrid = sms * 2 * LB_KINT_CTAS_PER_SM;
+        status = launch(PS_KINT, st, [&] {
+          lb_kint_kernel<<<kgrid, LB_THREADS, 0, st>>>(vc, v_stride, xc, oc, qcount, queue, cn, cap);
+        });
+      }
     }
   }
   if (!scratch) cudaFreeAsync(ws, st);
