@@ -138,6 +138,21 @@ LB_DF_FN dfloat df_mul_add(dfloat a, dfloat t, dfloat c) {
   return r;
 }
 
+// a * t + c for a float t: as df_mul_add, 14 FP32 instructions.
+LB_DF_FN dfloat df_mulf_add(dfloat a, float t, dfloat c) {
+  const float p = a.h * t;
+  float e = df_fma(a.h, t, -p);
+  e = df_fma(a.l, t, e);
+  const float s = p + c.h;
+  const float bp = s - p;
+  const float e2 = (p - (s - bp)) + (c.h - bp);
+  e = (e + e2) + c.l;
+  dfloat r;
+  r.h = s + e;
+  r.l = e - (r.h - s);
+  return r;
+}
+
 // a * b.  7 FP32 instructions.
 LB_DF_FN dfloat df_mul(dfloat a, dfloat b) {
   const float p = a.h * b.h;

@@ -22,6 +22,7 @@ template <> __host__ __device__ __forceinline__ float lb_fma<float>(float a, flo
 #include "debye_uk.h"
 #include "lb_fastmath.cuh"
 #include "lb_intmath.cuh"
+#include "lb_uniform.cuh"
 
 namespace lb {
 
@@ -203,26 +204,25 @@ __device__ __forceinline__ int classify(double v, double x, int mode, int w = WI
 //   r_k = (mu - (2k-1)^2) / (8 x k),  S = 1 + s r_1 (1 + s r_2 (1 + ... (1 + s r_K))).
 // ---------------------------------------------------------------------------
 // The number of terms actually summed is the smallest n <= K after which
-// the terms fall below 2^-56 (a later term is then below the rounding of S),
-// found with a single-precision pass (mu_terms) and made uniform across the
-// warp, so the double-precision Horner loop never diverges.  The tile kernel
-// estimates n while it bins the pairs and orders each region by it, so the
-// warps' lanes need similar counts.
-template <int K>
-__device__ __forceinline__ int mu_terms(float v, float x) {
-  int n = K;
-  // unrolled, so (2k-1)^2 and 1/k are constants: no division, no branch
-  const float muf = 4.0f * v * v, inv8xf = __fdividef(1.0f, 8.0f * x);
-  float t = 1.0f;
-  bool found = false;
-#pragma unroll
-  for (int k = 1; k <= K; ++k) {
-    t *= (muf - (float)((2 * k - 1) * (2 * k - 1))) * (inv8xf * (1.0f / (float)k));
-    const bool hit = !found && fabsf(t) < 1.4e-17f;
-    n = hit ? k : n;
-    found = found || hit;
-  }
-  return n;
+// the terms fall below 2^-56 (a later term is then below the rounding of S);
+// h is the first from which they are below 1e-3 (the leading h terms are
+// summed in FP64, the rest in double-float).  Both depend on v^2/(2x) and
+// 1/(8x) alone and come from a table over half octaves of the two
+// (muterms_table.h, the largest of each cell): 15 instructions, where a pass
+// over the 20 terms for each count took 160.  n averages 14.5 on the sweep's
+// mu_20 pairs (13.7 exact).  Made uniform across the warp, so the Horner loop
+// never diverges; the tile kernel orders the region by n while it bins the
+// pairs, so the warps' lanes need similar counts.
+#define LB_MUT_TABLE static __device__ const
+#include "muterms_table.h"
+
+// n | h << 8.
+__device__ __forceinline__ int mu_counts(float v, float x) {
+  const float w = __fdividef(1.0f, 8.0f * x), A = 4.0f * v * v * w;
+  const int ia = (int)(__float_as_uint(A) >> 22) - LB_MUT_A_BASE, iw = (int)(__float_as_uint(w) >> 22) - LB_MUT_W_BASE;
+  const int ca = ia < 0 ? 0 : (ia > LB_MUT_A_CELLS ? LB_MUT_A_CELLS : ia);
+  const int cw = iw < 0 ? 0 : (iw > LB_MUT_W_CELLS ? LB_MUT_W_CELLS : iw);
+  return (int)__ldg(lb_mut + cw * (LB_MUT_A_CELLS + 1) + ca);
 }
 
 // Terms of the power series of log I (series_log_i, series_so): the count
@@ -251,82 +251,53 @@ __device__ __forceinline__ int series_terms(float v, float x) {
 __device__ __forceinline__ int series_count(int packed) { return packed & 127; }
 __device__ __forceinline__ int series_head(int packed) { return packed >> 7; }
 
-// Leading terms of mu_K kept in FP64: the smallest k at which the running
-// product of the term ratios (the k-th term against the leading 1) falls
-// below 1e-3, by the single-precision pass of mu_terms; K when none does.
-// The terms past it hold less than 1e-3 of the sum and are summed in
-// double-float (relative error a few 2^-48, below 1e-17 of the sum).
-template <int K>
-__device__ __forceinline__ int mu_head(float v, float x) {
-  int m = K;
-  const float muf = 4.0f * v * v, inv8xf = __fdividef(1.0f, 8.0f * x);
-  float t = 1.0f;
-  bool found = false;
-#pragma unroll
-  for (int k = 1; k <= K; ++k) {
-    t *= (muf - (float)((2 * k - 1) * (2 * k - 1))) * (inv8xf * (1.0f / (float)k));
-    const bool hit = !found && fabsf(t) < 1e-3f;
-    m = hit ? k : m;
-    found = found || hit;
-  }
-  return m;
+// (2k-1)^2 for k = 1..20, and 20!/(k-1)! for k = 1..21 as doubles (exact) and
+// as pairs of floats (entries 0 unused).
+static __constant__ float kMuOdd[21] = {0.0f, 1.0f, 9.0f, 25.0f, 49.0f, 81.0f, 121.0f, 169.0f, 225.0f, 289.0f, 361.0f, 441.0f, 529.0f, 625.0f, 729.0f, 841.0f, 961.0f, 1089.0f, 1225.0f, 1369.0f, 1521.0f};
+static __constant__ double kMuOddD[21] = {0.0, 1.0, 9.0, 25.0, 49.0, 81.0, 121.0, 169.0, 225.0, 289.0, 361.0, 441.0, 529.0, 625.0, 729.0, 841.0, 961.0, 1089.0, 1225.0, 1369.0, 1521.0};
+static __constant__ double kMuF[22] = {0.0, 2432902008176640000.0, 2432902008176640000.0, 1216451004088320000.0, 405483668029440000.0, 101370917007360000.0, 20274183401472000.0, 3379030566912000.0, 482718652416000.0, 60339831552000.0, 6704425728000.0, 670442572800.0, 60949324800.0, 5079110400.0, 390700800.0, 27907200.0, 1860480.0, 116280.0, 6840.0, 380.0, 20.0, 1.0};
+static __constant__ float kMuFd[22][2] = {{0.0f, 0.0f}, {2.4329020231636746e+18f, -14987034624.0f}, {2.4329020231636746e+18f, -14987034624.0f}, {1.2164510115818373e+18f, -7493517312.0f}, {4.054836705272791e+17f, -2497839104.0f}, {1.0137091763181978e+17f, -624459776.0f}, {2.0274182667370496e+16f, 734101504.0f}, {3379030623518720.0f, -56606720.0f}, {482718655709184.0f, -3293184.0f}, {60339831963648.0f, -411648.0f}, {6704425598976.0f, 129024.0f}, {670442586112.0f, -13312.0f}, {60949323776.0f, 1024.0f}, {5079110656.0f, -256.0f}, {390700800.0f, 0.0f}, {27907200.0f, 0.0f}, {1860480.0f, 0.0f}, {116280.0f, 0.0f}, {6840.0f, 0.0f}, {380.0f, 0.0f}, {20.0f, 0.0f}, {1.0f, 0.0f}};
+constexpr long long kMuSoLogI = 2175819361628260ll, kMuSoLogK = 22797439711033177ll;   // log(8/(2 pi)), log(4 pi), Q53
+constexpr long long kLn2Q53 = 6243314768165359ll;
+constexpr long long kMuLogI = -760474846706970267ll;   // log(8/(2 pi)) - 2 log 20!, Q53
+constexpr long long kMuLogK = -739853226357565351ll;   // log(4 pi) - 2 log 20!, Q53
+
+// (log z + c) 2^53 for c in Q53: the fixed-point logarithm, or (z = 0,
+// subnormal, infinite or NaN, as a forced evaluation far outside gives) the
+// library's.
+static __device__ __noinline__ double log_q53_plus(double z, long long c) {
+  const uint32_t hi = (uint32_t)(ix_bits(z) >> 32);
+  if (hi - 0x00100000u < 0x7fe00000u) return (double)(ix_log_q53(z) + c);
+  return fma(log(z), 0x1p53, (double)c);
 }
 
-// 1/k and (2k-1)^2/k for k = 1..20, the constants of the term ratios of
-// mu_K, for a rolled loop over the warp's own number of terms (entry 0
-// unused).  A fully unrolled loop with the terms above n switched off by a
-// predicate would still issue every term's FP64 instructions.
-static __constant__ double kMuInvK[21] = {0.0, 1.0 / 1.0, 1.0 / 2.0, 1.0 / 3.0, 1.0 / 4.0, 1.0 / 5.0, 1.0 / 6.0, 1.0 / 7.0, 1.0 / 8.0, 1.0 / 9.0, 1.0 / 10.0, 1.0 / 11.0, 1.0 / 12.0, 1.0 / 13.0, 1.0 / 14.0, 1.0 / 15.0, 1.0 / 16.0, 1.0 / 17.0, 1.0 / 18.0, 1.0 / 19.0, 1.0 / 20.0};
-static __constant__ double kMuOddK[21] = {0.0, 1.0 / 1.0, 9.0 / 2.0, 25.0 / 3.0, 49.0 / 4.0, 81.0 / 5.0, 121.0 / 6.0, 169.0 / 7.0, 225.0 / 8.0, 289.0 / 9.0, 361.0 / 10.0, 441.0 / 11.0, 529.0 / 12.0, 625.0 / 13.0, 729.0 / 14.0, 841.0 / 15.0, 961.0 / 16.0, 1089.0 / 17.0, 1225.0 / 18.0, 1369.0 / 19.0, 1521.0 / 20.0};
-// 1/k as pairs of floats hi + lo (hi = 1/k rounded to single precision, lo
-// the rest), for the double-float terms.
-static __constant__ float kMuInvKh[21] = {0.0f, 0x1.p+0f, 0x1.p-1f, 0x1.555556p-2f, 0x1.p-2f, 0x1.99999ap-3f, 0x1.555556p-3f, 0x1.24924ap-3f, 0x1.p-3f, 0x1.c71c72p-4f, 0x1.99999ap-4f, 0x1.745d18p-4f, 0x1.555556p-4f, 0x1.3b13b2p-4f, 0x1.24924ap-4f, 0x1.111112p-4f, 0x1.p-4f, 0x1.e1e1e2p-5f, 0x1.c71c72p-5f, 0x1.af286cp-5f, 0x1.99999ap-5f};
-static __constant__ float kMuInvKl[21] = {0.0f, 0.0f, 0.0f, -0x1.555556p-27f, 0.0f, -0x1.99999ap-29f, -0x1.555556p-28f, -0x1.b6db6ep-28f, 0.0f, -0x1.c71c72p-31f, -0x1.99999ap-30f, -0x1.745d18p-29f, -0x1.555556p-29f, -0x1.89d89ep-29f, -0x1.b6db6ep-29f, -0x1.dddddep-29f, 0.0f, -0x1.e1e1e2p-33f, -0x1.c71c72p-32f, -0x1.af286cp-32f, -0x1.99999ap-31f};
-
-// mu_K with the lane's term count n given (at most K); all 32 lanes of the
-// warp call it together.
-template <int KIND, int K>
-__device__ __forceinline__ double mu_expr_n(double v, double x, int n) {
-  n = __reduce_max_sync(0xffffffffu, n);
-  const int h = __reduce_max_sync(0xffffffffu, mu_head<K>(f32_cut(v), f32_cut(x)));
-  const double mu = 4.0 * v * v;
+// mu_K with the lane's counts (mu_counts) given, at most cap terms; all 32
+// lanes of the warp call it together.  20! S by Horner's rule without the
+// divisions by k: with D_k = (mu - (2k-1)^2) s/(8x), Q <- D_k Q + 20!/(k-1)!
+// from Q = 20!/n! down to k = 1.
+template <int KIND>
+__device__ __forceinline__ double mu_expr_n(double v, double x, int counts, int cap) {
+  const int n = __reduce_max_sync(0xffffffffu, min(cap, counts & 255));
+  const int h = min(n, __reduce_max_sync(0xffffffffu, counts >> 8));
   const double rx = ix_rcp_call(8.0 * x);                             // 1/(8x) on the integer pipe
-  const double inv8x = (KIND == KIND_I) ? -rx : rx;                   // the sign s folded in
-  double P = 1.0;
-  int top = n;
+  const double w = (KIND == KIND_I) ? -rx : rx;                       // the sign s folded in
+  const double A = (4.0 * v * v) * w;
+  double Q = kMuF[n + 1];
   if (n > h) {
-    // terms h+1..n in double-float: r_k = (mu s/(8x) - (2k-1)^2 s/(8x)) / k,
-    // P <- 1 + r_k P
-    const dfloat wd = df_from_double(inv8x), muw = df_from_double(mu * inv8x);
-    dfloat Pd = df_make(1.0f, 0.0f);
+    // terms h+1..n in double-float
+    const dfloat wd = df_from_double(w), Ad = df_from_double(A);
+    dfloat Qd = df_make(kMuFd[n + 1][0], kMuFd[n + 1][1]);
 #pragma unroll 1
-    for (int k = n; k > h; --k) {
-      const float odd = (float)((2 * k - 1) * (2 * k - 1));           // exact
-      const dfloat ow = df_mul(wd, df_make(-odd, 0.0f));
-      const dfloat r = df_mul(df_add(muw, ow), df_make(kMuInvKh[k], kMuInvKl[k]));
-      Pd = df_mul_add(r, Pd, df_make(1.0f, 0.0f));
-    }
-    P = df_to_double(Pd);
-    top = h;
+    for (int k = n; k > h; --k)
+      Qd = df_mul_add(df_mulf_add(wd, -kMuOdd[k], Ad), Qd, df_make(kMuFd[k][0], kMuFd[k][1]));
+    Q = df_to_double(Qd);
   }
-  // Three FP64 operations per leading term: a = mu/k - (2k-1)^2/k,
-  // P = 1 + (a s/(8x)) P, for the warp's leading terms only.
 #pragma unroll 1
-  for (int k = top; k >= 1; --k) {
-    const double a = fma(mu, kMuInvK[k], -kMuOddK[k]);
-    P = fma(a * inv8x, P, 1.0);
-  }
+  for (int k = h; k >= 1; --k) Q = fma(fma(-kMuOddD[k], w, A), Q, kMuF[k]);
   // log(S / sqrt(2 pi x)) = log(S^2 / (2 pi x)) / 2 and
-  // log(S sqrt(pi / (2x))) = log(S^2 pi / (2x)) / 2, with 1/x = 8 |inv8x|:
-  // no square root needed.
-  const double S2 = P * P;
-  if (KIND == KIND_I) return fma(0.5, ix_log_call(S2 * rx * (8.0 / kTwoPi)), x);   // rx = |inv8x|
-  return fma(0.5, ix_log_call(S2 * rx * (4.0 * kPi)), -x);
-}
-
-template <int KIND, int K>
-__device__ __forceinline__ double mu_expr(double v, double x) {
-  return mu_expr_n<KIND, K>(v, x, mu_terms<K>(f32_cut(v), f32_cut(x)));
+  // log(S sqrt(pi / (2x))) = log(S^2 pi / (2x)) / 2, with 1/x = 8 rx: no
+  // square root needed; the constants join the logarithm in Q53.
+  return fma(0x1p-54, log_q53_plus(Q * Q * rx, KIND == KIND_I ? kMuLogI : kMuLogK), KIND == KIND_I ? x : -x);
 }
 
 // P_k(p) of the Debye polynomial u_k(t) = t^k P_k(t^2); k is a compile-time
@@ -401,8 +372,12 @@ __device__ __forceinline__ T debye_Q(int k, T p) {
 // recurrence of Eqs. "u0", "uk").  The two log terms are merged:
 // -log(2 pi v)/2 - log(r)/2 = log(1 / sqrt(2 pi v r)).
 // ---------------------------------------------------------------------------
-template <int KIND, int K>
-__device__ __forceinline__ double u_expr(double v, double x) {
+// Evaluated by u_fx (lb_uniform.cuh) wherever r = sqrt(v^2 + x^2) lies in
+// [16.04, 1e150] (every pair of the tight dispatch with v below that); this
+// form serves the rest: the paper's U_13 from v = 12.7 on, forced
+// evaluations, and extreme orders.
+template <int KIND>
+static __device__ __noinline__ double u_expr(double v, double x, int K) {
   const double inv_v = ix_rcp_call(v);           // reciprocal and root on the integer pipe
   const double xp = x * inv_v;
   double r, t;
@@ -520,23 +495,19 @@ __device__ __forceinline__ double series_log_i(double v, double x) {
 // the expressions are then the same for every pair, and a block computes
 // them once (scalar_order_setup):
 //   mu_K:   S = sum_k a_k w^k, w = 1/(8x), a_k = s^k prod_{j<=k} (mu - (2j-1)^2) / k!
-//           -- one FMA per term instead of three;
+//           -- one fixed-point multiply-add per term, no FP64;
 //   series: P <- 1 + (y / (k (k + v))) P with the reciprocals 1/(k (k + v))
 //           tabulated -- two operations per term instead of six, and
-//           lgamma(v + 1) once;
-//   U_K:    S(t) = 1 + sum_k (s/v)^k u_k(t) = sum_m C_m t^m as one polynomial
-//           of degree 3K in t -- 3K FMAs instead of K(K+3)/2, and 1/v once.
+//           lgamma(v + 1) once.
 // The sums are the same sums in another order of operations.
 // ---------------------------------------------------------------------------
 struct ScalarOrder {
-  double v, inv_v, lg1;                 // v, 1/v, lgamma(v + 1)
-  double sig;                           // sigma: a power of two near mu/8 (1 for mu < 8)
-  double mu[21];                        // a_0..a_20 / sigma^k (sign s of the kind folded in)
+  double v, lg1;                        // v, lgamma(v + 1)
+  int muj;                              // W = 2^muj w <= 1/2 wherever the dispatch takes mu_20
+  long long muc;                        // log constant of mu_K, Q53, the scale of mu[] included
+  long long mu[21];                     // a_0..a_20 / 2^(k muj) (sign s of the kind folded in), Q(60 - muq)
   double ser[91];                       // 1 / (k (k + v)), k = 1..90
-  double u4[4], u6[4], u9[4], u13[4];   // C_0..C_3 of U_K
-  dfloat mud[21];                       // mu[] in double-float
   dfloat serd[91];                      // ser[] in double-float
-  dfloat u4d[13], u6d[19], u9d[28], u13d[40];   // C_0..C_3K in double-float (C_4.. used)
 };
 
 // All threads of the block call it; ends with a barrier.
@@ -545,100 +516,41 @@ __device__ __forceinline__ void scalar_order_setup(ScalarOrder& so, double v) {
   const int tid = threadIdx.x;
   if (tid == 0) {
     so.v = v;
-    so.inv_v = 1.0 / v;
     so.lg1 = lgamma(v + 1.0);
+    // the smallest x at which a dispatch takes mu_20 for this order (tight:
+    // 18.5, or v^2 < 3.24 x; paper: 0.5113 log x + 0.7939 > log v)
+    const double xmin = v < 15.4 ? 18.4 : fmax(59.0, 0.98 * fmin(v * v / 3.24, pow(v / 2.212, 1.9558)));
+    const int j = ilogb(4.0 * xmin);                // 2^j / (8 x) <= 1/2
     const double mu = 4.0 * v * v, s = KIND == KIND_I ? -1.0 : 1.0;
-    // a_k w^k = (a_k / sigma^k) (sigma w)^k: with sigma near mu/8 the scaled
-    // coefficients stay below 8^k / k! (the unscaled ones overflow for
-    // orders above about 1e9, and the double-float ones above 1e38)
-    int j = 0;
-    if (mu >= 16.0) j = ilogb(mu) - 3;
-    so.sig = ldexp(1.0, j);
-    double a = 1.0;
-    so.mu[0] = 1.0;
-    so.mud[0] = df_make(1.0f, 0.0f);
+    double c[21], a = 1.0, big = 1.0;
+    c[0] = 1.0;
     for (int k = 1; k <= 20; ++k) {
       a = ldexp(a * (s * (mu - (double)((2 * k - 1) * (2 * k - 1)))) / (double)k, -j);
-      so.mu[k] = a;
-      so.mud[k] = df_from_double(a);
+      c[k] = a;
+      big = fmax(big, fabs(a));
     }
+    // |c_k| 2^(60 - muq) < 2^61: with W <= 1/2 every Horner step stays below 2^62
+    const int muq = big < 1e15 ? ilogb(big) : 50;
+    for (int k = 0; k <= 20; ++k) so.mu[k] = ix_fix(c[k], 60 - muq);
+    so.muj = j;
+    so.muc = (KIND == KIND_I ? kMuSoLogI : kMuSoLogK) - 2 * (60 - muq) * kLn2Q53;
   } else if (tid <= 90) {
     so.ser[tid] = 1.0 / ((double)tid * ((double)tid + v));
     so.serd[tid] = df_from_double(so.ser[tid]);
-  } else if (tid >= 128 && tid < 228) {
-    // C_m of U_K: the coefficients of t^m, sum over k + 2i = m of c_{k,i} (s/v)^k
-    int j = tid - 128, K, m;
-    double* dst;
-    dfloat* dstd;
-    if (j < 13) { K = 4; m = j; dst = so.u4; dstd = so.u4d; }
-    else if (j < 32) { K = 6; m = j - 13; dst = so.u6; dstd = so.u6d; }
-    else if (j < 60) { K = 9; m = j - 32; dst = so.u9; dstd = so.u9d; }
-    else { K = 13; m = j - 60; dst = so.u13; dstd = so.u13d; }
-    const double sv = (KIND == KIND_I ? 1.0 : -1.0) / v;
-    double c = 0.0, pk = 1.0;
-    for (int k = 0; k <= K; ++k) {
-      if (k > 0) pk *= sv;
-      const int twoi = m - k;
-      if (twoi >= 0 && (twoi & 1) == 0 && (twoi >> 1) <= k) c = fma(lb_debye_c[k][twoi >> 1], pk, c);
-    }
-    if (m < 4) dst[m] = c;
-    dstd[m] = df_from_double(c);
   }
   __syncthreads();
 }
 
 template <int KIND>
-__device__ __forceinline__ double mu_expr_so(const ScalarOrder& so, double x, int n) {
-  n = __reduce_max_sync(0xffffffffu, n);
-  const int h = __reduce_max_sync(0xffffffffu, mu_head<20>(f32_cut(so.v), f32_cut(x)));
-  const double w = ix_rcp_call(8.0 * x);
-  const double ws = w * so.sig;                   // exact: sigma is a power of two
-  double P = 0.0;
-  int top = n;
-  if (n > h) {                                    // terms h+1..n in double-float
-    const dfloat wd = df_from_double(ws);
-    dfloat Pd = so.mud[n];
+__device__ __forceinline__ double mu_expr_so(const ScalarOrder& so, double x, int counts) {
+  const int n = __reduce_max_sync(0xffffffffu, counts & 255);
+  const double rx = ix_rcp_call(8.0 * x);
+  const long long W = ix_fix(rx, 64 + so.muj);    // below 2^63
+  long long acc = so.mu[n];
 #pragma unroll 1
-    for (int k = n - 1; k > h; --k) Pd = df_mul_add(Pd, wd, so.mud[k]);
-    P = df_to_double(Pd);
-    top = h;
-  }
-#pragma unroll 1
-  for (int k = top; k >= 0; --k) P = fma(P, ws, so.mu[k]);   // the warp's leading terms
-  const double S2 = P * P;
-  if (KIND == KIND_I) return fma(0.5, ix_log_call(S2 * w * (8.0 / kTwoPi)), x);
-  return fma(0.5, ix_log_call(S2 * w * (4.0 * kPi)), -x);
-}
-
-template <int KIND, int K>
-__device__ __forceinline__ double u_expr_so(const ScalarOrder& so, double x) {
-  const double v = so.v, inv_v = so.inv_v;
-  const double xp = x * inv_v;
-  double r, t;
-  if (LB_LT(xp, 1e150)) {
-    const double r2 = fma(xp, xp, 1.0);
-    t = ix_rsqrt_call(r2);
-    r = r2 * t;
-  } else {
-    r = xp;
-    t = ix_rcp_call(r);
-  }
-  const double* C = K == 4 ? so.u4 : (K == 6 ? so.u6 : (K == 9 ? so.u9 : so.u13));
-  const dfloat* Cd = K == 4 ? so.u4d : (K == 6 ? so.u6d : (K == 9 ? so.u9d : so.u13d));
-  // S = sum_m C_m t^m.  C_m for m >= 4 holds the parts of u_k, k >= 2 only
-  // (u_k has the powers t^k .. t^3k), at most about 2e-3 of the sum in the
-  // U regions: those terms in double-float, C_3 .. C_0 in FP64.
-  const dfloat td = df_from_double(t);
-  dfloat Sd = Cd[3 * K];
-#pragma unroll 1
-  for (int m = 3 * K - 1; m >= 4; --m) Sd = df_mul_add(Sd, td, Cd[m]);
-  double S = df_to_double(Sd);
-#pragma unroll
-  for (int m = 3; m >= 0; --m) S = fma(S, t, C[m]);
-  const double eta = r + (ix_log_call(xp) - ix_log_call(1.0 + r));
-  const double w = S * S * (t * inv_v);          // as in u_expr
-  if (KIND == KIND_I) return fma(0.5, ix_log_call(w), fma(v, eta, -kHalfLog2Pi));
-  return fma(0.5, ix_log_call(w), fma(-v, eta, kHalfLogHalfPi));
+  for (int k = n - 1; k >= 0; --k) acc = so.mu[k] + ix_mulhi(acc, W);
+  const double S = (double)acc;
+  return fma(0x1p-54, log_q53_plus(S * S * rx, so.muc), KIND == KIND_I ? x : -x);
 }
 
 __device__ __forceinline__ double series_so(const ScalarOrder& so, double x, int packed) {
@@ -670,30 +582,15 @@ __device__ __forceinline__ double series_so(const ScalarOrder& so, double x, int
 // (Sec. 7), and these follow directly from its Eqs.
 // ---------------------------------------------------------------------------
 
+// 1/k and (2k-1)^2/k for k = 1..20 (entry 0 unused).
+static __constant__ double kMuInvK[21] = {0.0, 1.0 / 1.0, 1.0 / 2.0, 1.0 / 3.0, 1.0 / 4.0, 1.0 / 5.0, 1.0 / 6.0, 1.0 / 7.0, 1.0 / 8.0, 1.0 / 9.0, 1.0 / 10.0, 1.0 / 11.0, 1.0 / 12.0, 1.0 / 13.0, 1.0 / 14.0, 1.0 / 15.0, 1.0 / 16.0, 1.0 / 17.0, 1.0 / 18.0, 1.0 / 19.0, 1.0 / 20.0};
+static __constant__ double kMuOddK[21] = {0.0, 1.0 / 1.0, 9.0 / 2.0, 25.0 / 3.0, 49.0 / 4.0, 81.0 / 5.0, 121.0 / 6.0, 169.0 / 7.0, 225.0 / 8.0, 289.0 / 9.0, 361.0 / 10.0, 441.0 / 11.0, 529.0 / 12.0, 625.0 / 13.0, 729.0 / 14.0, 841.0 / 15.0, 961.0 / 16.0, 1089.0 / 17.0, 1225.0 / 18.0, 1369.0 / 19.0, 1521.0 / 20.0};
+
 // mu_K: log f = +-x - log(2 pi x)/2 + log S (I: +x, K: -x and +log(pi/2)/2),
 // S = 1 + sum_k c_k x^-k, so d/dx log f = +-1 - 1/(2x) - (sum_k k c_k x^-k) / (x S).
-template <int KIND, int K>
-__device__ __forceinline__ double mu_dx(double v, double x) {
-  const double mu = 4.0 * v * v;
-  const double inv8x = ix_rcp(8.0 * x);             // the reciprocals on the integer pipe
-  double term = 1.0, S = 1.0, D = 0.0;
-#pragma unroll
-  for (int k = 1; k <= K; ++k) {
-    const double odd = (double)((2 * k - 1) * (2 * k - 1));
-    double r = (mu - odd) * (inv8x * (1.0 / (double)k));
-    if (KIND == KIND_I) r = -r;
-    term *= r;
-    S += term;
-    D = fma((double)k, term, D);
-  }
-  const double inv_x = 8.0 * inv8x;                 // exact scaling
-  const double base = (KIND == KIND_I) ? 1.0 : -1.0;
-  return base - inv_x * fma(D, ix_rcp(S), 0.5);
-}
-
-// The same for the first n terms only (n: the pair's term count, made
-// warp-uniform), as a rolled loop: the terms past n are below 2^-56 of S.
-template <int KIND, int K>
+// Over the first n terms only (n: the pair's term count, made warp-uniform),
+// as a rolled loop: the terms past n are below 2^-56 of S.
+template <int KIND>
 __device__ __forceinline__ double mu_dx_n(double v, double x, int n) {
   n = __reduce_max_sync(0xffffffffu, n);
   const double mu = 4.0 * v * v;
@@ -716,8 +613,9 @@ __device__ __forceinline__ double mu_dx_n(double v, double x, int n) {
 // d/dt u_k(t) = t^(k-1) Q_k(t^2):
 //   d/dx log f = +-1/(t x') - (x' t^2 / v) (1/2 + SQ / S),
 //   S = 1 + sum q^k P_k(t^2), SQ = sum q^k Q_k(t^2), q = +-t/v.
-template <int KIND, int K>
-__device__ __forceinline__ double u_dx(double v, double x) {
+// K: the pair's own terms (its region's).
+template <int KIND>
+__device__ __forceinline__ double u_dx(double v, double x, int K) {
   const double inv_v = ix_rcp(v);                  // reciprocals and 1/sqrt on the integer pipe
   const double xp = x * inv_v;
   double r, t;

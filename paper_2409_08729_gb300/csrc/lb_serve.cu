@@ -124,7 +124,7 @@ __device__ __forceinline__ void serve_tile(TileShared<T, LB_THREADS>& S, ServeAu
   const int64_t t0 = tile * LB_TILE;
   const int tid = threadIdx.x;
   tile_bin<KIND, false, T>(S, v, d.v_stride, x, t0, d.n, d.mode, -1);
-  tile_eval<KIND, false, T>(S, out, t0, d.n);
+  tile_eval<KIND, false, T, false>(S, out, t0, d.n);
   if (KIND == KIND_K && sizeof(T) == 8) {
     const int c = S.rcount(R_FALLBACK), f0 = S.rbeg(R_FALLBACK);
     if (c > 0) {                                   // block-uniform

@@ -52,32 +52,31 @@ static __device__ unsigned int lb_check_status;
 #define LB_CHECK(cond, bit) true
 #endif
 
-// List keys.  mu_20 (FP64 values) takes one key per term count n = 1..20,
-// found while binning (an unrolled single-precision pass); the power series
-// one key per band of x, log-spaced, 3 log2(1 + x) (its term count grows with
-// x: rank correlation 0.98), because its exact count is a loop of up to 90
-// steps that is cheaper once per 32-pair chunk than once per item round.  So
-// each region's pairs come ordered by the number of terms their lanes sum.
-// Keys of a region are adjacent; regions come in the order of their list
-// ranges.
+// List keys.  mu_20 (FP64) takes one key per term count n = 1..20 (mu_counts);
+// the uniform expansions U_13 .. U_4 share one range of ten keys, by the
+// pair's number of terms, largest first (for FP64 values at most the
+// region's, uni_terms); the power series one key per band of x, log-spaced,
+// 2 log2(1 + x) (its term count grows with x: rank correlation 0.98), because
+// its exact count is a loop of up to 90 steps that is cheaper once per
+// 32-pair chunk than once per item round.  So each region's pairs come
+// ordered by the number of terms their lanes sum.  Keys of a region are
+// adjacent; regions come in the order of their list ranges.
 enum TileKey {
   KEY_MU20 = 0,                  // .. KEY_MU20 + 19
-  KEY_U13 = 20,
-  KEY_FB = 21,                   // .. KEY_FB + 14: power series (I), K integral (K)
-  KEY_MU3 = 36,
-  KEY_U4 = 37,
-  KEY_U6 = 38,
-  KEY_U9 = 39,
+  KEY_U = 20,                    // .. KEY_U + 9: 13 .. 4 terms
+  KEY_FB = 30,                   // .. KEY_FB + 8: power series (I), K integral (K)
+  KEY_MU3 = 39,
   NKEYS = 40
 };
 
 __host__ __device__ constexpr int region_key_first(int r) {
-  return r == R_MU20 ? KEY_MU20 : r == R_U13 ? KEY_U13 : r == R_FALLBACK ? KEY_FB : r == R_MU3 ? KEY_MU3
-       : r == R_U4 ? KEY_U4 : r == R_U6 ? KEY_U6 : KEY_U9;
+  return r == R_MU20 ? KEY_MU20 : r == R_FALLBACK ? KEY_FB : r == R_MU3 ? KEY_MU3 : KEY_U;
 }
 __host__ __device__ constexpr int region_key_end(int r) {
-  return r == R_MU20 ? KEY_MU20 + 20 : r == R_FALLBACK ? KEY_FB + 15 : region_key_first(r) + 1;
+  return r == R_MU20 ? KEY_MU20 + 20 : r == R_FALLBACK ? KEY_FB + 9 : r == R_MU3 ? KEY_MU3 + 1 : KEY_U + 10;
 }
+// Terms of a uniform expansion region.
+__host__ __device__ constexpr int region_terms(int r) { return r == R_U4 ? 4 : r == R_U6 ? 6 : r == R_U9 ? 9 : 13; }
 
 // One tile of NT * LB_ITEMS pairs in the shared memory of a block of NT threads.
 template <typename T, int NT>
@@ -90,7 +89,7 @@ struct TileShared {
     T sres[kTile];                                 // results, stored coalesced at the end of the tile
   };
   uint16_t list[kTile];                            // tile offsets of the pairs to evaluate, sorted by key
-  uint8_t nt[kTile];                               // estimated term count (mu_20; FP64 values)
+  uint8_t nt[kTile];                               // term count (uniform expansions)
   uint8_t keep[kTile];                             // 1: sres holds this pair's result
   uint16_t wcount[LB_ITEMS][NT / 32][NKEYS];       // pairs per (item round, warp, key), then offsets
   int kbeg[NKEYS + 1];                             // start of each key's range in list
@@ -117,56 +116,66 @@ __device__ __forceinline__ int tile_classify(T v, T x, int mode) {
   else return classify32(v, x, mode, DX ? WIDE_NONE : (KIND == KIND_K ? WIDE_K : WIDE_I));
 }
 
-// FP64 values with the lane's term count n (mu_20, series) given.
-template <int KIND, bool DX, typename T>
-__device__ __forceinline__ T tile_expr(int r, T v, T x, int n) {
+// One pair per lane of region r (R_U13 stands for every U_K): n is the lane's
+// term count (mu_counts, U_K's terms, series_terms).  so (FP64 values only):
+// the constants of a call whose pairs all have one order, or NULL.
+template <int KIND, bool DX, typename T, bool SO>
+__device__ __forceinline__ T tile_expr(int r, T v, T x, int n, const ScalarOrder* so) {
   if constexpr (sizeof(T) == 4) {
     switch (r) {
       case R_MU20: return mu_expr32<KIND, 20>(v, x);
-      case R_U13: return u_expr32<KIND, 13>(v, x);
       case R_MU3: return mu_expr32<KIND, 3>(v, x);
-      case R_U4: return u_expr32<KIND, 4>(v, x);
-      case R_U6: return u_expr32<KIND, 6>(v, x);
-      case R_U9: return u_expr32<KIND, 9>(v, x);
-      default: return (KIND == KIND_I) ? series_log_i32(v, x) : kt_log_k32(v, x);
+      case R_FALLBACK: return (KIND == KIND_I) ? series_log_i32(v, x) : kt_log_k32(v, x);
+      default:
+        return n == 4 ? u_expr32<KIND, 4>(v, x) : n == 6 ? u_expr32<KIND, 6>(v, x)
+             : n == 9 ? u_expr32<KIND, 9>(v, x) : u_expr32<KIND, 13>(v, x);
     }
   } else if constexpr (DX) {
     switch (r) {
-      case R_MU20: return mu_dx_n<KIND, 20>(v, x, n);
-      case R_U13: return u_dx<KIND, 13>(v, x);
-      case R_MU3: return mu_dx<KIND, 3>(v, x);
-      case R_U4: return u_dx<KIND, 4>(v, x);
-      case R_U6: return u_dx<KIND, 6>(v, x);
-      case R_U9: return u_dx<KIND, 9>(v, x);
-      default: return (KIND == KIND_I) ? series_dx_n(v, x, n) : __longlong_as_double(0x7ff8000000000000LL);
+      case R_MU20: return mu_dx_n<KIND>(v, x, n & 255);
+      case R_MU3: return mu_dx_n<KIND>(v, x, 3);
+      case R_FALLBACK: return (KIND == KIND_I) ? series_dx_n(v, x, n) : __longlong_as_double(0x7ff8000000000000LL);
+      default: return u_dx<KIND>(v, x, n);
     }
   } else {
     switch (r) {
-      case R_MU20: return mu_expr_n<KIND, 20>(v, x, n);
-      case R_U13: return u_expr<KIND, 13>(v, x);
-      case R_MU3: return mu_expr<KIND, 3>(v, x);
-      case R_U4: return u_expr<KIND, 4>(v, x);
-      case R_U6: return u_expr<KIND, 6>(v, x);
-      case R_U9: return u_expr<KIND, 9>(v, x);
-      default: return (KIND == KIND_I) ? series_log_i_n(v, x, n) : __longlong_as_double(0x7ff8000000000000LL);
+      case R_MU20:
+        if constexpr (SO) return mu_expr_so<KIND>(*so, x, n);
+        else return mu_expr_n<KIND>(v, x, n, 20);
+      case R_MU3: return mu_expr_n<KIND>(v, x, n, 3);
+      case R_FALLBACK:
+        if constexpr (KIND == KIND_K) return __longlong_as_double(0x7ff8000000000000LL);
+        else if constexpr (SO) return series_so(*so, x, n);
+        else return series_log_i_n(v, x, n);
+      default: {
+        const int Kmax = __reduce_max_sync(0xffffffffu, n);
+        const double s = fma(v, v, x * x);
+        return uni_ok(s, x) ? u_fx(KIND, v, x, s, n, Kmax) : u_expr<KIND>(v, x, n);
+      }
     }
   }
 }
 
-// List key of a classified pair, and the term count of mu_20 in *n (FP64
-// values and x-derivatives; 0 otherwise).
+// List key of a classified pair, and the term count of a uniform expansion
+// in *n (0 otherwise).
 template <int KIND, bool DX, typename T>
 __device__ __forceinline__ int tile_key(int r, T v, T x, int* n) {
   *n = 0;
-  if constexpr (sizeof(T) == 8) {
-    if (r == R_MU20) {
-      *n = mu_terms<20>(f32_cut(v), f32_cut(x));
-      return KEY_MU20 + *n - 1;
-    }
+  if (r == R_MU20) {
+    if constexpr (sizeof(T) == 8) return KEY_MU20 + (mu_counts(f32_cut(v), f32_cut(x)) & 255) - 1;
+    return KEY_MU20;
   }
-  if (KIND == KIND_I && r == R_FALLBACK)
-    return KEY_FB + min(14, (int)(3.0f * __log2f(1.0f + (sizeof(T) == 8 ? f32_cut((double)x) : (float)x))));
-  return region_key_first(r);
+  if (r == R_MU3) return KEY_MU3;
+  if (r == R_FALLBACK)
+    return KIND == KIND_I ? KEY_FB + min(8, (int)(2.0f * __log2f(1.0f + (sizeof(T) == 8 ? f32_cut((double)x) : (float)x))))
+                          : KEY_FB;
+  int K = region_terms(r);
+  if constexpr (sizeof(T) == 8 && !DX) {
+    const float vf = f32_cut(v), xf = f32_cut(x);
+    K = uni_terms(fmaf(vf, vf, xf * xf), K);
+  }
+  *n = K;
+  return KEY_U + 13 - K;
 }
 
 // Tile offset of item round `it` of thread `tid`: each thread handles two
@@ -299,27 +308,13 @@ __device__ __forceinline__ void tile_bin(TileShared<T, NT>& S, const T* __restri
   __syncthreads();
 }
 
-// The FP64 expressions with the order's constants of a ScalarOrder block.
-template <int KIND>
-__device__ __forceinline__ double tile_expr_so(int r, const ScalarOrder& so, double x, int n) {
-  switch (r) {
-    case R_MU20: return mu_expr_so<KIND>(so, x, n);
-    case R_U13: return u_expr_so<KIND, 13>(so, x);
-    case R_MU3: return mu_expr<KIND, 3>(so.v, x);
-    case R_U4: return u_expr_so<KIND, 4>(so, x);
-    case R_U6: return u_expr_so<KIND, 6>(so, x);
-    case R_U9: return u_expr_so<KIND, 9>(so, x);
-    default: return (KIND == KIND_I) ? series_so(so, x, n) : __longlong_as_double(0x7ff8000000000000LL);
-  }
-}
-
 // The chunks (32 pairs, one warp each) of region R's range of the list,
 // handed out from a shared counter: a warp that runs out moves on to the
 // next region while the others finish this one.  Lanes past the end of the
 // range recompute the chunk's first entry and do not keep it.  `so` (FP64
 // values only) holds the constants of a call whose pairs all have one
 // order, or is NULL.
-template <int KIND, bool DX, typename T, int R, int NT>
+template <int KIND, bool DX, typename T, bool SO, int R, int NT>
 __device__ __forceinline__ void tile_eval_region(TileShared<T, NT>& S, int lane, const ScalarOrder* so) {
   const int b0 = S.rbeg(R), c = S.rend(R) - b0;
   const int nch = (c + 31) >> 5;
@@ -336,16 +331,11 @@ __device__ __forceinline__ void tile_eval_region(TileShared<T, NT>& S, int lane,
       ok = false;
     }
     const int li = S.list[jl];
-    int nterm = S.nt[li];
-    if constexpr (sizeof(T) == 8 && KIND == KIND_I && R == R_FALLBACK)
-      nterm = series_terms(f32_cut(so ? so->v : (double)S.sv[li]), f32_cut((double)S.sx[li]));
-    T val;
-    if constexpr (sizeof(T) == 8 && !DX) {
-      if (so) val = tile_expr_so<KIND>(R, *so, S.sx[li], nterm);
-      else val = tile_expr<KIND, DX, T>(R, S.sv[li], S.sx[li], nterm);
-    } else {
-      val = tile_expr<KIND, DX, T>(R, S.sv[li], S.sx[li], nterm);
-    }
+    const T v = SO ? (T)so->v : S.sv[li], x = S.sx[li];
+    int n = S.nt[li];
+    if constexpr (sizeof(T) == 8 && (R == R_MU20 || R == R_MU3)) n = mu_counts(f32_cut(v), f32_cut(x));
+    if constexpr (sizeof(T) == 8 && KIND == KIND_I && R == R_FALLBACK) n = series_terms(f32_cut(v), f32_cut(x));
+    const T val = tile_expr<KIND, DX, T, SO>(R, v, x, n, so);
     __syncwarp();                                  // every lane has read its arguments (sres is sx)
     if (ok) S.sres[li] = val;
   }
@@ -359,18 +349,15 @@ __device__ __forceinline__ void tile_eval_region(TileShared<T, NT>& S, int lane,
 // instruction where both are kept and the buffer is aligned.  The FP64 K fallback
 // pairs are left to the K integral: neither evaluated nor stored (so out may
 // equal x: their arguments stay in place for it).  Ends with a barrier.
-template <int KIND, bool DX, typename T, int NT>
+template <int KIND, bool DX, typename T, bool SO, int NT>
 __device__ __forceinline__ void tile_eval(TileShared<T, NT>& S, T* __restrict__ out, int64_t t0, int64_t n,
                                           const ScalarOrder* so = nullptr) {
   typedef typename Vec2<T>::type T2;
   const int tid = threadIdx.x, lane = tid & 31;
-  if (KIND == KIND_I || sizeof(T) == 4) tile_eval_region<KIND, DX, T, R_FALLBACK, NT>(S, lane, so);
-  tile_eval_region<KIND, DX, T, R_U13, NT>(S, lane, so);
-  tile_eval_region<KIND, DX, T, R_U9, NT>(S, lane, so);
-  tile_eval_region<KIND, DX, T, R_MU20, NT>(S, lane, so);
-  tile_eval_region<KIND, DX, T, R_U6, NT>(S, lane, so);
-  tile_eval_region<KIND, DX, T, R_MU3, NT>(S, lane, so);
-  tile_eval_region<KIND, DX, T, R_U4, NT>(S, lane, so);
+  if (KIND == KIND_I || sizeof(T) == 4) tile_eval_region<KIND, DX, T, SO, R_FALLBACK, NT>(S, lane, so);
+  tile_eval_region<KIND, DX, T, SO, R_U13, NT>(S, lane, so);
+  tile_eval_region<KIND, DX, T, SO, R_MU20, NT>(S, lane, so);
+  tile_eval_region<KIND, DX, T, SO, R_MU3, NT>(S, lane, so);
   __syncthreads();
   const bool vec = (reinterpret_cast<uintptr_t>(out) & (2 * sizeof(T) - 1)) == 0;
 #pragma unroll

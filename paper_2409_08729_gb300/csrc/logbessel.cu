@@ -104,7 +104,7 @@ lb_tiles_kernel(const T* __restrict__ v, int64_t v_stride, const T* __restrict__
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t t0 = tile * kTile;
     tile_bin<KIND, DX, T>(S, v, v_stride, x, t0, n, mode, forced_region);
-    tile_eval<KIND, DX, T>(S, out, t0, n, so);
+    tile_eval<KIND, DX, T, SO>(S, out, t0, n, so);
     if (KIND == KIND_K && sizeof(T) == 8) {
       const int c = S.rcount(R_FALLBACK), f0 = S.rbeg(R_FALLBACK);
       if (c > 0) {
