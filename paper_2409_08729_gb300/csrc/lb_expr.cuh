@@ -511,7 +511,7 @@ struct ScalarOrder {
 };
 
 // All threads of the block call it; ends with a barrier.
-template <int KIND>
+template <int KIND, int NT>
 __device__ __forceinline__ void scalar_order_setup(ScalarOrder& so, double v) {
   const int tid = threadIdx.x;
   if (tid == 0) {
@@ -534,10 +534,12 @@ __device__ __forceinline__ void scalar_order_setup(ScalarOrder& so, double v) {
     for (int k = 0; k <= 20; ++k) so.mu[k] = ix_fix(c[k], 60 - muq);
     so.muj = j;
     so.muc = (KIND == KIND_I ? kMuSoLogI : kMuSoLogK) - 2 * (60 - muq) * kLn2Q53;
-  } else if (tid <= 90) {
-    so.ser[tid] = 1.0 / ((double)tid * ((double)tid + v));
-    so.serd[tid] = df_from_double(so.ser[tid]);
   }
+  if (tid >= 32)
+    for (int k = tid - 31; k <= 90; k += NT - 32) {
+      so.ser[k] = 1.0 / ((double)k * ((double)k + v));
+      so.serd[k] = df_from_double(so.ser[k]);
+    }
   __syncthreads();
 }
 

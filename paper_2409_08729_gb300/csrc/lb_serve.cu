@@ -123,8 +123,8 @@ __device__ __forceinline__ void serve_tile(TileShared<T, LB_THREADS>& S, ServeAu
   T* out = reinterpret_cast<T*>(d.out);
   const int64_t t0 = tile * LB_TILE;
   const int tid = threadIdx.x;
-  tile_bin<KIND, false, T>(S, v, d.v_stride, x, t0, d.n, d.mode, -1);
-  tile_eval<KIND, false, T, false>(S, out, t0, d.n);
+  tile_bin<KIND, false, T, false>(S, v, d.v_stride, d.v_stride ? T(0) : v[0], x, t0, d.n, d.mode, -1);
+  tile_eval<KIND, false, T, false, false>(S, out, t0, d.n);
   if (KIND == KIND_K && sizeof(T) == 8) {
     const int c = S.rcount(R_FALLBACK), f0 = S.rbeg(R_FALLBACK);
     if (c > 0) {                                   // block-uniform

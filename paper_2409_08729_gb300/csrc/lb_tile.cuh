@@ -89,7 +89,7 @@ struct TileShared {
     T sres[kTile];                                 // results, stored coalesced at the end of the tile
   };
   uint16_t list[kTile];                            // tile offsets of the pairs to evaluate, sorted by key
-  uint8_t nt[kTile];                               // term count (uniform expansions)
+  uint8_t nt[kTile];                               // term count (uniform expansions), class (K fallback)
   uint8_t keep[kTile];                             // 1: sres holds this pair's result
   uint16_t wcount[LB_ITEMS][NT / 32][NKEYS];       // pairs per (item round, warp, key), then offsets
   int kbeg[NKEYS + 1];                             // start of each key's range in list
@@ -134,7 +134,7 @@ __device__ __forceinline__ T tile_expr(int r, T v, T x, int n, const ScalarOrder
     switch (r) {
       case R_MU20: return mu_dx_n<KIND>(v, x, n & 255);
       case R_MU3: return mu_dx_n<KIND>(v, x, 3);
-      case R_FALLBACK: return (KIND == KIND_I) ? series_dx_n(v, x, n) : __longlong_as_double(0x7ff8000000000000LL);
+      case R_FALLBACK: return (KIND == KIND_I) ? series_dx_n(v, x, n) : kt_eval<true>(v, x, n, lb_kt_exp2);
       default: return u_dx<KIND>(v, x, n);
     }
   } else {
@@ -144,7 +144,7 @@ __device__ __forceinline__ T tile_expr(int r, T v, T x, int n, const ScalarOrder
         else return mu_expr_n<KIND>(v, x, n, 20);
       case R_MU3: return mu_expr_n<KIND>(v, x, n, 3);
       case R_FALLBACK:
-        if constexpr (KIND == KIND_K) return __longlong_as_double(0x7ff8000000000000LL);
+        if constexpr (KIND == KIND_K) return kt_eval<false>(v, x, n, lb_kt_exp2);
         else if constexpr (SO) return series_so(*so, x, n);
         else return series_log_i_n(v, x, n);
       default: {
@@ -156,9 +156,11 @@ __device__ __forceinline__ T tile_expr(int r, T v, T x, int n, const ScalarOrder
   }
 }
 
-// List key of a classified pair, and the term count of a uniform expansion
-// in *n (0 otherwise).
-template <int KIND, bool DX, typename T>
+// List key of a classified pair, and in *n the term count of a uniform
+// expansion or the class of a K fallback pair (0 otherwise).
+// KIN: FP64 K fallback pairs are evaluated in the tile, by class (kt_class,
+// costliest first).
+template <int KIND, bool DX, typename T, bool KIN>
 __device__ __forceinline__ int tile_key(int r, T v, T x, int* n) {
   *n = 0;
   if (r == R_MU20) {
@@ -166,9 +168,14 @@ __device__ __forceinline__ int tile_key(int r, T v, T x, int* n) {
     return KEY_MU20;
   }
   if (r == R_MU3) return KEY_MU3;
-  if (r == R_FALLBACK)
-    return KIND == KIND_I ? KEY_FB + min(8, (int)(2.0f * __log2f(1.0f + (sizeof(T) == 8 ? f32_cut((double)x) : (float)x))))
-                          : KEY_FB;
+  if (r == R_FALLBACK) {
+    if (KIND == KIND_I) return KEY_FB + min(8, (int)(2.0f * __log2f(1.0f + (sizeof(T) == 8 ? f32_cut((double)x) : (float)x))));
+    if constexpr (KIN) {
+      *n = kt_class(v, x, DX);
+      return KEY_FB + *n;
+    }
+    return KEY_FB;
+  }
   int K = region_terms(r);
   if constexpr (sizeof(T) == 8 && !DX) {
     const float vf = f32_cut(v), xf = f32_cut(x);
@@ -198,8 +205,9 @@ struct Vec2<float> { typedef float2 type; };
 // ordered by (key, item round, warp, lane), from one warp match per item
 // and a per-key prefix over (item round, warp): the order, and so the warp
 // mates of every pair, do not depend on scheduling.
-template <int KIND, bool DX, typename T, int NT>
-__device__ __forceinline__ void tile_bin(TileShared<T, NT>& S, const T* __restrict__ v, int64_t v_stride,
+// v0: the order of every pair when v_stride is 0 (v is not read then).
+template <int KIND, bool DX, typename T, bool KIN, int NT>
+__device__ __forceinline__ void tile_bin(TileShared<T, NT>& S, const T* __restrict__ v, int64_t v_stride, T v0,
                                          const T* __restrict__ x, int64_t t0, int64_t n, int mode,
                                          int forced_region) {
   typedef typename Vec2<T>::type T2;
@@ -208,7 +216,6 @@ __device__ __forceinline__ void tile_bin(TileShared<T, NT>& S, const T* __restri
   // the pair offsets t0 are multiples of the tile size, so aligned bases keep every pair of loads aligned
   const bool vec = ((reinterpret_cast<uintptr_t>(x) | (v_stride ? reinterpret_cast<uintptr_t>(v) : 0)) &
                     (2 * sizeof(T) - 1)) == 0;
-  const T v0 = v_stride ? T(0) : v[0];
   T vv[LB_ITEMS], xx[LB_ITEMS];
 #pragma unroll
   for (int h = 0; h < LB_ITEMS / 2; ++h) {
@@ -256,9 +263,9 @@ __device__ __forceinline__ void tile_bin(TileShared<T, NT>& S, const T* __restri
         S.sx[li] = xi;
         const int r = forced_region >= 0 ? forced_region : tile_classify<KIND, DX, T>(vi, xi, mode);
         int nterm;
-        k = tile_key<KIND, DX, T>(r, vi, xi, &nterm);
+        k = tile_key<KIND, DX, T, KIN>(r, vi, xi, &nterm);
         S.nt[li] = (uint8_t)nterm;
-        keep = (KIND == KIND_K && sizeof(T) == 8 && r == R_FALLBACK) ? 0 : 1;   // FP64 K integral pairs are stored later
+        keep = (KIND == KIND_K && sizeof(T) == 8 && !KIN && r == R_FALLBACK) ? 0 : 1;   // queued pairs are stored later
       }
     }
     S.keep[li] = keep;
@@ -308,6 +315,20 @@ __device__ __forceinline__ void tile_bin(TileShared<T, NT>& S, const T* __restri
   __syncthreads();
 }
 
+// von Mises-Fisher log-normaliser (paper Sec. 6.3):
+//   log C_d(k) = (d/2 - 1) log k - (d/2) log(2 pi) - log I_{d/2-1}(k),
+// from f = log I_{d/2-1}(k) (or, for DX, f = d/dk log I_{d/2-1}, giving
+// d/dk log C_d = (d/2-1)/k - I'/I).
+// At k = 0: log C_d(0) = lgamma(d/2) - log 2 - (d/2) log pi, the limit of
+// I_nu(k) ~ (k/2)^nu / Gamma(nu + 1).
+template <bool DX>
+__device__ __forceinline__ double vmf_form(double d, double k, double f) {
+  const double nu = 0.5 * d - 1.0;
+  if (DX) return (k == 0.0) ? 0.0 : (k < 1e300 ? kt_div(nu, k) : nu / k) - f;
+  if (k == 0.0) return lgamma(0.5 * d) - 0.6931471805599453 - 0.5 * d * 1.1447298858494002;
+  return fma(nu, ix_log_call(k), -0.5 * d * 1.8378770664093453) - f;
+}
+
 // The chunks (32 pairs, one warp each) of region R's range of the list,
 // handed out from a shared counter: a warp that runs out moves on to the
 // next region while the others finish this one.  Lanes past the end of the
@@ -349,12 +370,15 @@ __device__ __forceinline__ void tile_eval_region(TileShared<T, NT>& S, int lane,
 // instruction where both are kept and the buffer is aligned.  The FP64 K fallback
 // pairs are left to the K integral: neither evaluated nor stored (so out may
 // equal x: their arguments stay in place for it).  Ends with a barrier.
-template <int KIND, bool DX, typename T, bool SO, int NT>
+// vmf_d >= 0 (FP64 log I and its derivative only): the von Mises-Fisher form
+// of the result in dimension vmf_d (vmf_form) is stored instead.
+template <int KIND, bool DX, typename T, bool SO, bool KIN, int NT>
 __device__ __forceinline__ void tile_eval(TileShared<T, NT>& S, T* __restrict__ out, int64_t t0, int64_t n,
-                                          const ScalarOrder* so = nullptr) {
+                                          const ScalarOrder* so = nullptr, const T* __restrict__ x = nullptr,
+                                          double vmf_d = -1.0) {
   typedef typename Vec2<T>::type T2;
   const int tid = threadIdx.x, lane = tid & 31;
-  if (KIND == KIND_I || sizeof(T) == 4) tile_eval_region<KIND, DX, T, SO, R_FALLBACK, NT>(S, lane, so);
+  if (KIND == KIND_I || sizeof(T) == 4 || KIN) tile_eval_region<KIND, DX, T, SO, R_FALLBACK, NT>(S, lane, so);
   tile_eval_region<KIND, DX, T, SO, R_U13, NT>(S, lane, so);
   tile_eval_region<KIND, DX, T, SO, R_MU20, NT>(S, lane, so);
   tile_eval_region<KIND, DX, T, SO, R_MU3, NT>(S, lane, so);
@@ -365,6 +389,12 @@ __device__ __forceinline__ void tile_eval(TileShared<T, NT>& S, T* __restrict__ 
     const int li = tile_offset<NT>(2 * h, tid);
     const int64_t i = t0 + li;
     const bool k0 = i < n && S.keep[li], k1 = i + 1 < n && S.keep[li + 1];
+    if constexpr (sizeof(T) == 8 && KIND == KIND_I) {
+      if (vmf_d >= 0.0) {
+        if (k0) S.sres[li] = vmf_form<DX>(vmf_d, x[i], S.sres[li]);
+        if (k1) S.sres[li + 1] = vmf_form<DX>(vmf_d, x[i + 1], S.sres[li + 1]);
+      }
+    }
     if (vec && k0 && k1) {
       T2 r;
       r.x = S.sres[li];
@@ -392,6 +422,45 @@ __device__ __forceinline__ double kint_warp_batch(double vi, double xi, int m, i
     if (lane == e) mine = li;
   }
   return pre + mine;
+}
+
+// One pair per lane, `ppw` pairs per warp, tight mode (FP64): for calls with
+// too few pairs for the tiles to fill the GPU.  The groups of expressions
+// present in the warp run one after another; lanes outside the group run on
+// its first pair's arguments, so that the warp stays together, and drop the
+// result.  One kernel, no queue and no shared memory.
+template <int KIND, bool DX>
+__device__ __forceinline__ void warp_pairs64(const double* __restrict__ v, int64_t v_stride, double v0,
+                                             const double* __restrict__ x, double* __restrict__ out, int64_t i,
+                                             bool valid, double vmf_d) {
+  double vi = valid ? (v_stride ? v[i] : v0) : 1.0;
+  const double xi = valid ? x[i] : 1.0;
+  if constexpr (KIND == KIND_K) vi = fabs(vi);
+  double val = 0.0;
+  const bool edge = tile_special<KIND, DX, double>(vi, xi, &val);
+  int r = R_SPECIAL, n = 0;
+  if (valid && !edge) {
+    r = tile_classify<KIND, DX, double>(vi, xi, MODE_TIGHT);
+    tile_key<KIND, DX, double, true>(r, vi, xi, &n);
+    if (r == R_MU20) n = mu_counts(f32_cut(vi), f32_cut(xi));
+    if (KIND == KIND_I && r == R_FALLBACK) n = series_terms(f32_cut(vi), f32_cut(xi));
+    if (r != R_MU20 && r != R_FALLBACK) r = R_U13;         // every uniform expansion
+  }
+  unsigned todo = __ballot_sync(0xffffffffu, r != R_SPECIAL);
+  while (todo) {
+    const int lead = __ffs(todo) - 1, g = __shfl_sync(0xffffffffu, r, lead);
+    const bool in = r == g;
+    const unsigned members = __ballot_sync(0xffffffffu, in);
+    const double vl = __shfl_sync(0xffffffffu, vi, lead), xl = __shfl_sync(0xffffffffu, xi, lead);
+    const int nl = __shfl_sync(0xffffffffu, n, lead);
+    const double f = tile_expr<KIND, DX, double, false>(g, in ? vi : vl, in ? xi : xl, in ? n : nl, nullptr);
+    if (in) val = f;
+    todo &= ~members;
+  }
+  if constexpr (KIND == KIND_I) {
+    if (valid && vmf_d >= 0.0) val = vmf_form<DX>(vmf_d, xi, val);
+  }
+  if (valid) out[i] = val;
 }
 
 // The 16 KB table of kt_exp2_q58 in shared memory (random lookups cost a few

@@ -58,6 +58,15 @@ namespace {
 #ifndef LB_KINT_CTAS_PER_SM
 #define LB_KINT_CTAS_PER_SM 4
 #endif
+#ifndef LB_MID_CTAS_PER_SM
+#define LB_MID_CTAS_PER_SM 8
+#endif
+#ifndef LB_SMALL_THREADS
+#define LB_SMALL_THREADS 64
+#endif
+#ifndef LB_SMALL_N
+#define LB_SMALL_N 12000
+#endif
 #ifndef LB_TILES32_CTAS_PER_SM
 #define LB_TILES32_CTAS_PER_SM 6
 #endif
@@ -86,32 +95,42 @@ constexpr uint32_t kQueueOffsetMask = (1u << kQueueOffsetBits) - 1u;
 // region): the order's constants once per block, and only the per-order
 // forms of the expressions compiled in (each kernel carries one form's
 // code, half the instruction footprint).
-template <int KIND, bool DX, typename T, bool SO>
-__global__ void __launch_bounds__(kTileThreads, LB_TILES_CTAS_PER_SM)
-lb_tiles_kernel(const T* __restrict__ v, int64_t v_stride, const T* __restrict__ x, T* __restrict__ out,
+// NT: threads per block; the 2048-pair tiles of 512 threads suit calls that
+// fill the GPU several times over, tiles of 512 pairs the smaller ones.
+// KIN: the K fallback pairs are evaluated in the tile instead of queued.
+// v == NULL: the order of every pair is v0 (v_stride 0).
+// vmf_d >= 0: see tile_eval.
+__host__ __device__ constexpr int tiles_ctas(int nt, bool kin) {
+  return nt == kTileThreads ? LB_TILES_CTAS_PER_SM : (kin ? LB_MID_CTAS_PER_SM : LB_TILES_CTAS_PER_SM * kTileThreads / nt);
+}
+template <int KIND, bool DX, typename T, bool SO, int NT, bool KIN>
+__global__ void __launch_bounds__(NT, tiles_ctas(NT, KIN))
+lb_tiles_kernel(const T* __restrict__ v, int64_t v_stride, T v0, const T* __restrict__ x, T* __restrict__ out,
                 int64_t n, int mode, int forced_region, unsigned int* __restrict__ qcount,
-                uint32_t* __restrict__ queue, int64_t qcap) {
+                uint32_t* __restrict__ queue, int64_t qcap, double vmf_d) {
   static_assert(!SO || (sizeof(T) == 8 && !DX), "per-order constants are built for FP64 values");
-  __shared__ TileShared<T, kTileThreads> S;
+  constexpr int kPairs = NT * LB_ITEMS;
+  __shared__ TileShared<T, NT> S;
   const int tid = threadIdx.x;
-  const int64_t ntiles = (n + kTile - 1) / kTile;
+  const int64_t ntiles = (n + kPairs - 1) / kPairs;
+  if (v_stride == 0 && v) v0 = v[0];
   const ScalarOrder* so = nullptr;
   if constexpr (SO) {
     __shared__ ScalarOrder SOC;
-    scalar_order_setup<KIND>(SOC, KIND == KIND_K ? fabs((double)v[0]) : (double)v[0]);
+    scalar_order_setup<KIND, NT>(SOC, KIND == KIND_K ? fabs((double)v0) : (double)v0);
     so = &SOC;
   }
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t t0 = tile * kTile;
-    tile_bin<KIND, DX, T>(S, v, v_stride, x, t0, n, mode, forced_region);
-    tile_eval<KIND, DX, T, SO>(S, out, t0, n, so);
-    if (KIND == KIND_K && sizeof(T) == 8) {
+    const int64_t t0 = tile * kPairs;
+    tile_bin<KIND, DX, T, KIN>(S, v, v_stride, v0, x, t0, n, mode, forced_region);
+    tile_eval<KIND, DX, T, SO, KIN>(S, out, t0, n, so, x, vmf_d);
+    if (KIND == KIND_K && sizeof(T) == 8 && !KIN) {
       const int c = S.rcount(R_FALLBACK), f0 = S.rbeg(R_FALLBACK);
       if (c > 0) {
         if (tid == 0) S.qbase = atomicAdd(qcount, (unsigned int)c);
         __syncthreads();
         const unsigned int b = S.qbase;
-        for (int j = tid; j < c; j += kTileThreads) {
+        for (int j = tid; j < c; j += NT) {
           const int li = S.list[f0 + j];
           uint32_t cl = 0;
           if constexpr (sizeof(T) == 8) {
@@ -128,6 +147,17 @@ lb_tiles_kernel(const T* __restrict__ v, int64_t v_stride, const T* __restrict__
     }
     __syncthreads();
   }
+}
+
+// Calls of few pairs: see warp_pairs64.
+template <int KIND, bool DX>
+__global__ void __launch_bounds__(LB_SMALL_THREADS)
+lb_small_kernel(const double* __restrict__ v, int64_t v_stride, double v0, const double* __restrict__ x,
+                double* __restrict__ out, int64_t n, int ppw, double vmf_d) {
+  if (v_stride == 0 && v) v0 = v[0];
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = ((int64_t)blockIdx.x * LB_SMALL_THREADS + threadIdx.x) >> 5, i = warp * ppw + lane;
+  warp_pairs64<KIND, DX>(v, v_stride, v0, x, out, i, lane < ppw && i < n, vmf_d);
 }
 
 // K integral, tight FP64: one thread per queued pair (lb_ktrap.cuh).  A
@@ -276,30 +306,6 @@ __global__ void lb_classify_kernel(const double* __restrict__ v, int64_t v_strid
     reg[i] = special_value<KIND>(vi, xi, &sp) ? (uint8_t)R_SPECIAL : (uint8_t)classify(vi, xi, mode, KIND == KIND_K ? WIDE_K : WIDE_I);
   }
 }
-
-// von Mises-Fisher log-normaliser (paper Sec. 6.3):
-//   log C_d(k) = (d/2 - 1) log k - (d/2) log(2 pi) - log I_{d/2-1}(k),
-// applied in place to out[i] = log I_{d/2-1}(kappa[i]) (or, for DX, to
-// out[i] = d/dk log I_{d/2-1}, giving d/dk log C_d = (d/2-1)/k - I'/I).
-// At k = 0: log C_d(0) = lgamma(d/2) - log 2 - (d/2) log pi, the limit of
-// I_nu(k) ~ (k/2)^nu / Gamma(nu + 1).
-template <bool DX>
-__global__ void lb_vmf_finish_kernel(const double* __restrict__ kappa, double* __restrict__ out, int64_t n,
-                                     double d) {
-  const double nu = 0.5 * d - 1.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double k = kappa[i];
-    if (DX) {
-      out[i] = (k == 0.0) ? 0.0 : nu / k - out[i];
-    } else if (k == 0.0) {
-      out[i] = lgamma(0.5 * d) - 0.6931471805599453 - 0.5 * d * 1.1447298858494002;
-    } else {
-      out[i] = fma(nu, log(k), -0.5 * d * 1.8378770664093453) - out[i];
-    }
-  }
-}
-
-__global__ void lb_set_scalar_kernel(double* p, double value) { *p = value; }
 
 // Elementwise exp/log for checking the table-driven implementations against
 // the libm ones: which = 0 fm_exp, 1 fm_log, 2 exp, 3 log; and CUDA's
@@ -468,60 +474,100 @@ lb_status run_tiles32(const float* v, int64_t v_stride, const float* x, float* o
 // of 32-bit pair offsets in scratch memory (qcount: the counter, queue:
 // min(n, chunk) entries), processed chunk by chunk; `scratch` supplies it,
 // or, when NULL, it comes from the stream-ordered allocator.
+//
+// FP64 calls of total_n pairs (the caller's n; passes and pieces of one call
+// take the same route, so that their results are those of one pass):
+//   up to LB_SMALL_N     lb_small_kernel alone (tight mode);
+//   below 2^17           tiles of 512 pairs, the K fallback in the tile (tight
+//                        mode): one launch and no scratch;
+//   below 2^20           tiles of 512 pairs, K fallback queued;
+//   from there           tiles of 2048 pairs, K fallback queued.
+constexpr int64_t kMidInTile = (int64_t)1 << 17, kMid = (int64_t)1 << 20;
+constexpr int kMidThreads = 128;
+
+template <int KIND, bool DX, typename T, bool SO, int NT, bool KIN>
+lb_status launch_tiles(int sms, cudaStream_t st, const T* v, int64_t v_stride, T v0, const T* x, T* out, int64_t n,
+                       int mode, int forced_region, unsigned int* qcount, uint32_t* queue, int64_t cap, double vmf_d) {
+  const int64_t ntiles = (n + NT * LB_ITEMS - 1) / (NT * LB_ITEMS), most = (int64_t)sms * tiles_ctas(NT, KIN);
+  const int grid = (int)(ntiles < most ? ntiles : most);
+  return launch(PS_TILES, st, [&] {
+    lb_tiles_kernel<KIND, DX, T, SO, NT, KIN><<<grid, NT, 0, st>>>(v, v_stride, v0, x, out, n, mode, forced_region,
+                                                                  qcount, queue, cap, vmf_d);
+  });
+}
+
+// The tile kernel of a pass of n pairs: one order per call has its constants
+// computed per block, where there are enough pairs to pay for that.
+template <int KIND, bool DX, typename T>
+lb_status run_tiles(int sms, cudaStream_t st, const T* v, int64_t v_stride, T v0, const T* x, T* out, int64_t n,
+                    int mode, int forced_region, unsigned int* qcount, uint32_t* queue, int64_t cap, int64_t total_n,
+                    double vmf_d) {
+  if constexpr (sizeof(T) == 8) {
+    const bool so = !DX && v_stride == 0 && forced_region < 0;
+    if (total_n < kMid && forced_region < 0) {
+      if (so && total_n >= kMidInTile)
+        return launch_tiles<KIND, DX, T, !DX, kMidThreads, false>(sms, st, v, v_stride, v0, x, out, n, mode,
+                                                                  forced_region, qcount, queue, cap, vmf_d);
+      return launch_tiles<KIND, DX, T, false, kMidThreads, false>(sms, st, v, v_stride, v0, x, out, n, mode,
+                                                                  forced_region, qcount, queue, cap, vmf_d);
+    }
+    if (so)
+      return launch_tiles<KIND, DX, T, !DX, kTileThreads, false>(sms, st, v, v_stride, v0, x, out, n, mode,
+                                                                 forced_region, qcount, queue, cap, vmf_d);
+  }
+  return launch_tiles<KIND, DX, T, false, kTileThreads, false>(sms, st, v, v_stride, v0, x, out, n, mode,
+                                                               forced_region, qcount, queue, cap, vmf_d);
+}
+
 template <int KIND, bool DX, typename T>
 lb_status run_impl(const T* v, int64_t v_stride, const T* x, T* out, int64_t n, int mode, int forced_region,
-                   cudaStream_t st, void* scratch, int64_t chunk) {
+                   cudaStream_t st, void* scratch, int64_t chunk, int64_t total_n, T v0 = T(0), double vmf_d = -1.0) {
   const int sms = sm_count();
-  const int64_t ntiles_all = (n + kTile - 1) / kTile;
-  const bool per_order = sizeof(T) == 8 && !DX && v_stride == 0 && forced_region < 0;
   if (KIND == KIND_K && sizeof(T) == 4 && mode != MODE_TIGHT && (forced_region < 0 || forced_region == R_FALLBACK))
     return fail(LB_ENOTSUP, "%sthe FP32 K integral is implemented for LB_TIGHT only", "", 0);
   if constexpr (sizeof(T) == 4) {
     if (mode == MODE_TIGHT && forced_region < 0) return run_tiles32<KIND>(v, v_stride, x, out, n, st);
-  }
-  if (KIND == KIND_I || sizeof(T) == 4 || (forced_region >= 0 && forced_region != R_FALLBACK)) {
-    const int grid = (int)(ntiles_all < (int64_t)sms * LB_TILES_CTAS_PER_SM ? ntiles_all : (int64_t)sms * LB_TILES_CTAS_PER_SM);
-    return launch(PS_TILES, st, [&] {
-      if (per_order)
-        lb_tiles_kernel<KIND, DX, T, !DX && sizeof(T) == 8><<<grid, kTileThreads, 0, st>>>(
-            v, v_stride, x, out, n, mode, forced_region, nullptr, nullptr, 0);
-      else
-        lb_tiles_kernel<KIND, DX, T, false><<<grid, kTileThreads, 0, st>>>(v, v_stride, x, out, n, mode,
-                                                                          forced_region, nullptr, nullptr, 0);
-    });
-  }
-  // queue entries a pass can write: every workspace holds at least this many
-  const int64_t cap = n < chunk ? n : chunk;
-  void* ws = scratch;
-  if (!ws) {
-    const size_t bytes = 256 + (size_t)cap * sizeof(uint32_t);
-    if (cudaMallocAsync(&ws, bytes, st) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(LB_ENOMEM, "cudaMallocAsync of %s%lld bytes failed", "", (long long)bytes);
+  } else if (mode == MODE_TIGHT && forced_region < 0) {
+    if (total_n <= LB_SMALL_N) {
+      // as few pairs per warp as 16 warps per SM allow
+      const int64_t most = (int64_t)sms * 16, want = (n + most - 1) / most;
+      const int ppw = (int)(want < 32 ? want : 32);
+      const int64_t warps = (n + ppw - 1) / ppw;
+      const int grid = (int)((warps * 32 + LB_SMALL_THREADS - 1) / LB_SMALL_THREADS);
+      return launch(PS_TILES, st, [&] {
+        lb_small_kernel<KIND, DX><<<grid, LB_SMALL_THREADS, 0, st>>>(v, v_stride, v0, x, out, n, ppw, vmf_d);
+      });
     }
+    if (KIND == KIND_K && total_n < kMidInTile)
+      return launch_tiles<KIND, DX, T, false, kMidThreads, KIND == KIND_K>(sms, st, v, v_stride, v0, x, out, n, mode,
+                                                                           forced_region, nullptr, nullptr, 0, vmf_d);
   }
-  unsigned int* qcount = (unsigned int*)ws;
-  uint32_t* queue = (uint32_t*)((char*)ws + 256);
-  lb_status status = LB_OK;
-  for (int64_t c0 = 0; c0 < n && status == LB_OK; c0 += chunk) {
-    const int64_t cn = (n - c0) < chunk ? (n - c0) : chunk;
-    if (cudaMemsetAsync(qcount, 0, sizeof(unsigned int), st) != cudaSuccess) { status = check_launch("cudaMemsetAsync"); break; }
-    const T* vc = v + c0 * v_stride;
-    const T* xc = x + c0;
-    T* oc = out + c0;
-    const int64_t ntiles = (cn + kTile - 1) / kTile;
-    const int grid = (int)(ntiles < (int64_t)sms * LB_TILES_CTAS_PER_SM ? ntiles : (int64_t)sms * LB_TILES_CTAS_PER_SM);
-    status = launch(PS_TILES, st, [&] {
-      if (per_order)
-        lb_tiles_kernel<KIND, DX, T, !DX && sizeof(T) == 8><<<grid, kTileThreads, 0, st>>>(
-            vc, v_stride, xc, oc, cn, mode, forced_region, qcount, queue, cap);
-      else
-        lb_tiles_kernel<KIND, DX, T, false><<<grid, kTileThreads, 0, st>>>(vc, v_stride, xc, oc, cn, mode,
-                                                                          forced_region, qcount, queue, cap);
-    });
-    if (status != LB_OK) break;
-    bool done = false;
-    if constexpr (sizeof(T) == 8) {
+  if (KIND == KIND_I || sizeof(T) == 4 || (forced_region >= 0 && forced_region != R_FALLBACK))
+    return run_tiles<KIND, DX, T>(sms, st, v, v_stride, v0, x, out, n, mode, forced_region, nullptr, nullptr, 0,
+                                  total_n, vmf_d);
+  if constexpr (sizeof(T) == 8) {
+    // queue entries a pass can write: every workspace holds at least this many
+    const int64_t cap = n < chunk ? n : chunk;
+    void* ws = scratch;
+    if (!ws) {
+      const size_t bytes = 256 + (size_t)cap * sizeof(uint32_t);
+      if (cudaMallocAsync(&ws, bytes, st) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(LB_ENOMEM, "cudaMallocAsync of %s%lld bytes failed", "", (long long)bytes);
+      }
+    }
+    unsigned int* qcount = (unsigned int*)ws;
+    uint32_t* queue = (uint32_t*)((char*)ws + 256);
+    lb_status status = LB_OK;
+    for (int64_t c0 = 0; c0 < n && status == LB_OK; c0 += chunk) {
+      const int64_t cn = (n - c0) < chunk ? (n - c0) : chunk;
+      if (cudaMemsetAsync(qcount, 0, sizeof(unsigned int), st) != cudaSuccess) { status = check_launch("cudaMemsetAsync"); break; }
+      const T* vc = v + c0 * v_stride;
+      const T* xc = x + c0;
+      T* oc = out + c0;
+      status = run_tiles<KIND, DX, T>(sms, st, vc, v_stride, v0, xc, oc, cn, mode, forced_region, qcount, queue, cap,
+                                      total_n, vmf_d);
+      if (status != LB_OK) break;
       if (mode == MODE_TIGHT) {
         // the queue's length is on the device: a block per 32 pairs it can hold, at most the resident ones
         const int64_t want = (cn + 31) / 32, most = (int64_t)sms * ktrap_ctas(DX);
@@ -529,32 +575,29 @@ lb_status run_impl(const T* v, int64_t v_stride, const T* x, T* out, int64_t n, 
         status = launch(PS_KINT, st, [&] {
           lb_ktrap_kernel<DX><<<kgrid, LB_THREADS, 0, st>>>(vc, v_stride, xc, oc, qcount, queue, cn, cap);
         });
-        done = true;
-      }
-    }
-    if constexpr (sizeof(T) == 8) {
-      if (!done) {
+      } else {
         const int kgrid = sms * 2 * LB_KINT_CTAS_PER_SM;
         status = launch(PS_KINT, st, [&] {
           lb_kint_kernel<<<kgrid, LB_THREADS, 0, st>>>(vc, v_stride, xc, oc, qcount, queue, cn, cap);
         });
       }
     }
+    if (!scratch) cudaFreeAsync(ws, st);
+    return status;
   }
-  if (!scratch) cudaFreeAsync(ws, st);
-  return status;
+  return LB_OK;
 }
 
 template <int KIND, bool DX>
 lb_status run(const double* v, int64_t v_stride, const double* x, double* out, int64_t n, int mode,
               int forced_region, cudaStream_t st) {
-  return run_impl<KIND, DX, double>(v, v_stride, x, out, n, mode, forced_region, st, nullptr, kChunk);
+  return run_impl<KIND, DX, double>(v, v_stride, x, out, n, mode, forced_region, st, nullptr, kChunk, n);
 }
 
 lb_status run32(int kind, const float* v, int64_t v_stride, const float* x, float* out, int64_t n, int mode,
                 int forced_region, cudaStream_t st) {
-  if (kind == KIND_I) return run_impl<KIND_I, false, float>(v, v_stride, x, out, n, mode, forced_region, st, nullptr, kChunk);
-  return run_impl<KIND_K, false, float>(v, v_stride, x, out, n, mode, forced_region, st, nullptr, kChunk);
+  if (kind == KIND_I) return run_impl<KIND_I, false, float>(v, v_stride, x, out, n, mode, forced_region, st, nullptr, kChunk, n);
+  return run_impl<KIND_K, false, float>(v, v_stride, x, out, n, mode, forced_region, st, nullptr, kChunk, n);
 }
 
 // Fixed scratch for logbessel_k_noalloc: the queue counter (first 256
@@ -634,7 +677,7 @@ lb_status logbessel_k_noalloc(lb_dtype dtype, const void* v, int64_t v_stride, c
   void* scratch = noalloc_scratch_address();
   if (!scratch) return LB_ECUDA;
   return run_impl<KIND_K, false, double>((const double*)v, v_stride, (const double*)x, (double*)out, n, (int)mode,
-                                         -1, (cudaStream_t)cuda_stream, scratch, LB_NOALLOC_MAX_PAIRS);
+                                         -1, (cudaStream_t)cuda_stream, scratch, LB_NOALLOC_MAX_PAIRS, n);
 }
 
 int64_t logbessel_workspace_bytes(int64_t n) {
@@ -657,9 +700,9 @@ lb_status logbessel_k_ws(lb_dtype dtype, const void* v, int64_t v_stride, const 
   cudaStream_t st = (cudaStream_t)cuda_stream;
   if (dtype == LB_F32)
     return run_impl<KIND_K, false, float>((const float*)v, v_stride, (const float*)x, (float*)out, n, (int)mode, -1,
-                                          st, workspace, cap);
+                                          st, workspace, cap, n);
   return run_impl<KIND_K, false, double>((const double*)v, v_stride, (const double*)x, (double*)out, n, (int)mode,
-                                         -1, st, workspace, cap);
+                                         -1, st, workspace, cap, n);
 }
 
 lb_status logbessel_k_dx_ws(lb_dtype dtype, const void* v, int64_t v_stride, const void* x, void* out, int64_t n,
@@ -676,7 +719,7 @@ lb_status logbessel_k_dx_ws(lb_dtype dtype, const void* v, int64_t v_stride, con
   const int64_t cap0 = (ws_bytes - 256) / 4;
   const int64_t cap = ((cap0 < kChunk ? cap0 : kChunk) / kTile) * kTile;
   return run_impl<KIND_K, true, double>((const double*)v, v_stride, (const double*)x, (double*)out, n, (int)mode, -1,
-                                        (cudaStream_t)cuda_stream, workspace, cap);
+                                        (cudaStream_t)cuda_stream, workspace, cap, n);
 }
 
 lb_status logbessel_classify(int kind, lb_dtype dtype, const void* v, int64_t v_stride,
@@ -726,26 +769,10 @@ lb_status logbessel_vmf_log_c(lb_dtype dtype, double d, const void* kappa, void*
   if (s != LB_OK || n == 0) return s;
   if (dtype != LB_F64) return fail(LB_ENOTSUP, "%sthe vMF log-normaliser is implemented for LB_F64 only", "", 0);
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  double* nu = nullptr;
-  if (cudaMallocAsync(&nu, sizeof(double), st) != cudaSuccess) {
-    cudaGetLastError();
-    return fail(LB_ENOMEM, "cudaMallocAsync of %s%lld bytes failed", "", 8);
-  }
-  s = launch(PS_AUX, st, [&] { lb_set_scalar_kernel<<<1, 1, 0, st>>>(nu, 0.5 * d - 1.0); });
-  if (s == LB_OK)
-    s = deriv ? run<KIND_I, true>(nu, 0, (const double*)kappa, (double*)out, n, MODE_TIGHT, -1, st)
-              : run<KIND_I, false>(nu, 0, (const double*)kappa, (double*)out, n, MODE_TIGHT, -1, st);
-  if (s == LB_OK) {
-    const int grid = sm_count() * 4;
-    s = launch(PS_AUX, st, [&] {
-      if (deriv)
-        lb_vmf_finish_kernel<true><<<grid, LB_THREADS, 0, st>>>((const double*)kappa, (double*)out, n, d);
-      else
-        lb_vmf_finish_kernel<false><<<grid, LB_THREADS, 0, st>>>((const double*)kappa, (double*)out, n, d);
-    });
-  }
-  cudaFreeAsync(nu, st);
-  return s;
+  const double nu = 0.5 * d - 1.0, *k = (const double*)kappa;
+  if (deriv)
+    return run_impl<KIND_I, true, double>(nullptr, 0, k, (double*)out, n, MODE_TIGHT, -1, st, nullptr, kChunk, n, nu, d);
+  return run_impl<KIND_I, false, double>(nullptr, 0, k, (double*)out, n, MODE_TIGHT, -1, st, nullptr, kChunk, n, nu, d);
 }
 
 lb_status logbessel_math_eval(int which, const double* in, double* out, int64_t n, void* cuda_stream) {
@@ -897,16 +924,16 @@ lb_status logbessel_host(int fn, lb_dtype dtype, const void* v, int64_t v_stride
     if (dtype == LB_F32) {
       const float *fv = (const float*)dv, *fx = (const float*)dx;
       float* fo = (float*)dout;
-      s = fn == 0 ? run_impl<KIND_I, false, float>(fv, v_stride, fx, fo, cn, (int)mode, -1, sc, nullptr, kChunk)
-                  : run_impl<KIND_K, false, float>(fv, v_stride, fx, fo, cn, (int)mode, -1, sc, ws, kChunk);
+      s = fn == 0 ? run_impl<KIND_I, false, float>(fv, v_stride, fx, fo, cn, (int)mode, -1, sc, nullptr, kChunk, n)
+                  : run_impl<KIND_K, false, float>(fv, v_stride, fx, fo, cn, (int)mode, -1, sc, ws, kChunk, n);
     } else {
       const double *dvv = (const double*)dv, *dxx = (const double*)dx;
       double* dd = (double*)dout;
       switch (fn) {
-        case 0: s = run_impl<KIND_I, false, double>(dvv, v_stride, dxx, dd, cn, (int)mode, -1, sc, nullptr, kChunk); break;
-        case 1: s = run_impl<KIND_K, false, double>(dvv, v_stride, dxx, dd, cn, (int)mode, -1, sc, ws, kChunk); break;
-        case 2: s = run_impl<KIND_I, true, double>(dvv, v_stride, dxx, dd, cn, (int)mode, -1, sc, nullptr, kChunk); break;
-        default: s = run_impl<KIND_K, true, double>(dvv, v_stride, dxx, dd, cn, (int)mode, -1, sc, ws, kChunk); break;
+        case 0: s = run_impl<KIND_I, false, double>(dvv, v_stride, dxx, dd, cn, (int)mode, -1, sc, nullptr, kChunk, n); break;
+        case 1: s = run_impl<KIND_K, false, double>(dvv, v_stride, dxx, dd, cn, (int)mode, -1, sc, ws, kChunk, n); break;
+        case 2: s = run_impl<KIND_I, true, double>(dvv, v_stride, dxx, dd, cn, (int)mode, -1, sc, nullptr, kChunk, n); break;
+        default: s = run_impl<KIND_K, true, double>(dvv, v_stride, dxx, dd, cn, (int)mode, -1, sc, ws, kChunk, n); break;
       }
     }
     if (s != LB_OK) break;
