@@ -41,7 +41,7 @@ def _prep(v, x):
         raise ValueError("x must be on a CUDA device (the library has no CPU path)")
     dt = x.dtype if x.dtype in (torch.float32, torch.float64) else torch.float64
     if not isinstance(v, torch.Tensor):
-        v = torch.tensor(float(v), dtype=dt, device=x.device)
+        v = torch.full((1,), float(v), dtype=dt, device=x.device)   # a fill on the stream, no copy from the host
     if v.device != x.device:
         raise ValueError("v and x must be on the same device")
     v = v.to(dt)
@@ -62,17 +62,38 @@ def ctypes_stream(s):
     return s.cuda_stream
 
 
+_CODES = {torch.float64: _binding.LB_F64, torch.float32: _binding.LB_F32}
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_fns = {}
+
+
 def _call(name, v, x, mode, out):
-    vf, vs, xf, shape = _prep(v, x)
-    n = xf.numel()
+    fn = _fns.get(name)
+    if fn is None:
+        fn = _fns[name] = getattr(_binding.lib(), name)
+    code = None
+    if type(x) is torch.Tensor and type(v) is torch.Tensor and x.is_cuda and x.is_contiguous() and v.is_contiguous():
+        # both as the library takes them: nothing to convert or broadcast
+        dt = x.dtype
+        if v.dtype is dt and v.device == x.device:
+            vs = 0 if v.numel() == 1 else 1
+            if vs == 0 or v.shape == x.shape:
+                code, vf, xf, shape = _CODES.get(dt), v, x, x.shape
+    if code is None:
+        vf, vs, xf, shape = _prep(v, x)
+        dt = xf.dtype
+        code = _dtype_code(dt)
     if out is None:
-        out = torch.empty(shape, dtype=xf.dtype, device=xf.device)
-    elif out.shape != shape or out.dtype != xf.dtype or not out.is_contiguous():
-        raise ValueError("out must be a contiguous %s tensor of shape %s" % (xf.dtype, tuple(shape)))
-    with torch.cuda.device(xf.device):
-        fn = getattr(_binding.lib(), name)
-        _binding.check(fn(_dtype_code(xf.dtype), vf.data_ptr(), vs, xf.data_ptr(), out.data_ptr(), n,
-                          MODES[mode], _stream(xf.device)))
+        out = torch.empty(shape, dtype=dt, device=xf.device)
+    elif out.shape != shape or out.dtype != dt or not out.is_contiguous():
+        raise ValueError("out must be a contiguous %s tensor of shape %s" % (dt, tuple(shape)))
+    dev = xf.get_device()
+    args = (code, vf.data_ptr(), vs, xf.data_ptr(), out.data_ptr(), xf.numel(), MODES[mode])
+    if _raw_stream is not None and dev == torch.cuda.current_device():
+        _binding.check(fn(*args, _raw_stream(dev)))
+    else:
+        with torch.cuda.device(dev):
+            _binding.check(fn(*args, _stream(xf.device)))
     return out
 
 

@@ -101,8 +101,8 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // Shared memory of the persistent kernel: one tile, the exponential's
 // table (FP64 K windows) or the node table of an FP32 K window with one order.
 union ServeShared {
-  TileShared<double, LB_THREADS> d;
-  TileShared<float, LB_THREADS> f;
+  TileShared<double, LB_THREADS, LB_ITEMS> d;
+  TileShared<float, LB_THREADS, LB_ITEMS> f;
   __align__(16) unsigned long long kt[2048];
   Warp32 w32[LB_THREADS / 32];
 };
@@ -116,7 +116,7 @@ struct ServeAux {          // per-tile class counts and queue bases of the K pai
 // queue of their rule class (class 0 when the request has one queue); their
 // order within a queue does not change any result.
 template <int KIND, typename T>
-__device__ __forceinline__ void serve_tile(TileShared<T, LB_THREADS>& S, ServeAux& A, const SlotDesc& d, int64_t tile,
+__device__ __forceinline__ void serve_tile(TileShared<T, LB_THREADS, LB_ITEMS>& S, ServeAux& A, const SlotDesc& d, int64_t tile,
                                            unsigned* qc) {
   const T* v = reinterpret_cast<const T*>(d.v);
   const T* x = reinterpret_cast<const T*>(d.x);

@@ -78,11 +78,11 @@ __host__ __device__ constexpr int region_key_end(int r) {
 // Terms of a uniform expansion region.
 __host__ __device__ constexpr int region_terms(int r) { return r == R_U4 ? 4 : r == R_U6 ? 6 : r == R_U9 ? 9 : 13; }
 
-// One tile of NT * LB_ITEMS pairs in the shared memory of a block of NT threads.
-template <typename T, int NT>
+// One tile of NT * IT pairs in the shared memory of a block of NT threads.
+template <typename T, int NT, int IT>
 struct TileShared {
   static constexpr int kThreads = NT;
-  static constexpr int kTile = NT * LB_ITEMS;
+  static constexpr int kTile = NT * IT;
   T sv[kTile];
   union {                                          // a pair's result replaces its argument
     T sx[kTile];
@@ -91,7 +91,7 @@ struct TileShared {
   uint16_t list[kTile];                            // tile offsets of the pairs to evaluate, sorted by key
   uint8_t nt[kTile];                               // term count (uniform expansions), class (K fallback)
   uint8_t keep[kTile];                             // 1: sres holds this pair's result
-  uint16_t wcount[LB_ITEMS][NT / 32][NKEYS];       // pairs per (item round, warp, key), then offsets
+  uint16_t wcount[IT][NT / 32][NKEYS];       // pairs per (item round, warp, key), then offsets
   int kbeg[NKEYS + 1];                             // start of each key's range in list
   int next_chunk[8];                               // per region: next chunk of 32 pairs to hand out (tile_eval)
   unsigned int qbase;
@@ -116,11 +116,22 @@ __device__ __forceinline__ int tile_classify(T v, T x, int mode) {
   else return classify32(v, x, mode, DX ? WIDE_NONE : (KIND == KIND_K ? WIDE_K : WIDE_I));
 }
 
+// The 16 KB table of kt_exp2_q58 in shared memory (random lookups cost a few
+// bank conflicts there, up to 32 cache-line accesses in global memory).  All
+// NT threads of the block call it; the caller synchronizes.
+template <int NT>
+__device__ __forceinline__ void kt_load_table(unsigned long long* tab) {
+  for (int i = 2 * threadIdx.x; i < 2048; i += 2 * NT)
+    *reinterpret_cast<ulonglong2*>(tab + i) = *reinterpret_cast<const ulonglong2*>(lb_kt_exp2 + i);
+}
+
 // One pair per lane of region r (R_U13 stands for every U_K): n is the lane's
 // term count (mu_counts, U_K's terms, series_terms).  so (FP64 values only):
-// the constants of a call whose pairs all have one order, or NULL.
+// the constants of a call whose pairs all have one order, or NULL; tab: the
+// table of kt_exp2_q58 (K integral).
 template <int KIND, bool DX, typename T, bool SO>
-__device__ __forceinline__ T tile_expr(int r, T v, T x, int n, const ScalarOrder* so) {
+__device__ __forceinline__ T tile_expr(int r, T v, T x, int n, const ScalarOrder* so,
+                                       const unsigned long long* tab) {
   if constexpr (sizeof(T) == 4) {
     switch (r) {
       case R_MU20: return mu_expr32<KIND, 20>(v, x);
@@ -134,7 +145,7 @@ __device__ __forceinline__ T tile_expr(int r, T v, T x, int n, const ScalarOrder
     switch (r) {
       case R_MU20: return mu_dx_n<KIND>(v, x, n & 255);
       case R_MU3: return mu_dx_n<KIND>(v, x, 3);
-      case R_FALLBACK: return (KIND == KIND_I) ? series_dx_n(v, x, n) : kt_eval<true>(v, x, n, lb_kt_exp2);
+      case R_FALLBACK: return (KIND == KIND_I) ? series_dx_n(v, x, n) : kt_eval<true>(v, x, n, tab);
       default: return u_dx<KIND>(v, x, n);
     }
   } else {
@@ -144,7 +155,7 @@ __device__ __forceinline__ T tile_expr(int r, T v, T x, int n, const ScalarOrder
         else return mu_expr_n<KIND>(v, x, n, 20);
       case R_MU3: return mu_expr_n<KIND>(v, x, n, 3);
       case R_FALLBACK:
-        if constexpr (KIND == KIND_K) return kt_eval<false>(v, x, n, lb_kt_exp2);
+        if constexpr (KIND == KIND_K) return kt_eval<false>(v, x, n, tab);
         else if constexpr (SO) return series_so(*so, x, n);
         else return series_log_i_n(v, x, n);
       default: {
@@ -188,9 +199,10 @@ __device__ __forceinline__ int tile_key(int r, T v, T x, int* n) {
 // Tile offset of item round `it` of thread `tid`: each thread handles two
 // adjacent pairs per pair of rounds, so it loads and stores them with one
 // 16-byte (FP64) or 8-byte (FP32) instruction.
-template <int NT>
+// IT = 1: one pair per thread.
+template <int NT, int IT>
 __device__ __forceinline__ int tile_offset(int it, int tid) {
-  return (it >> 1) * (2 * NT) + 2 * tid + (it & 1);
+  return IT == 1 ? tid : (it >> 1) * (2 * NT) + 2 * tid + (it & 1);
 }
 
 template <typename T>
@@ -200,14 +212,14 @@ struct Vec2<double> { typedef double2 type; };
 template <>
 struct Vec2<float> { typedef float2 type; };
 
-// Load, edge-handle, classify and sort pairs [t0, min(t0 + NT * LB_ITEMS, n)).
+// Load, edge-handle, classify and sort pairs [t0, min(t0 + NT * IT, n)).
 // All threads of the block call it; it ends with a barrier.  The list is
 // ordered by (key, item round, warp, lane), from one warp match per item
 // and a per-key prefix over (item round, warp): the order, and so the warp
 // mates of every pair, do not depend on scheduling.
 // v0: the order of every pair when v_stride is 0 (v is not read then).
-template <int KIND, bool DX, typename T, bool KIN, int NT>
-__device__ __forceinline__ void tile_bin(TileShared<T, NT>& S, const T* __restrict__ v, int64_t v_stride, T v0,
+template <int KIND, bool DX, typename T, bool KIN, int NT, int IT>
+__device__ __forceinline__ void tile_bin(TileShared<T, NT, IT>& S, const T* __restrict__ v, int64_t v_stride, T v0,
                                          const T* __restrict__ x, int64_t t0, int64_t n, int mode,
                                          int forced_region) {
   typedef typename Vec2<T>::type T2;
@@ -216,34 +228,40 @@ __device__ __forceinline__ void tile_bin(TileShared<T, NT>& S, const T* __restri
   // the pair offsets t0 are multiples of the tile size, so aligned bases keep every pair of loads aligned
   const bool vec = ((reinterpret_cast<uintptr_t>(x) | (v_stride ? reinterpret_cast<uintptr_t>(v) : 0)) &
                     (2 * sizeof(T) - 1)) == 0;
-  T vv[LB_ITEMS], xx[LB_ITEMS];
+  T vv[IT], xx[IT];
+  if constexpr (IT == 1) {
+    const int64_t i = t0 + tid;
+    xx[0] = i < n ? x[i] : T(1);
+    vv[0] = i < n ? (v_stride ? v[i] : v0) : T(0);
+  } else {
 #pragma unroll
-  for (int h = 0; h < LB_ITEMS / 2; ++h) {
-    const int li = tile_offset<NT>(2 * h, tid);
-    const int64_t i = t0 + li;
-    if (vec && i + 1 < n) {
-      const T2 xv = *reinterpret_cast<const T2*>(x + i);
-      xx[2 * h] = xv.x;
-      xx[2 * h + 1] = xv.y;
-      if (v_stride) {
-        const T2 vw = *reinterpret_cast<const T2*>(v + i);
-        vv[2 * h] = vw.x;
-        vv[2 * h + 1] = vw.y;
+    for (int h = 0; h < IT / 2; ++h) {
+      const int li = tile_offset<NT, IT>(2 * h, tid);
+      const int64_t i = t0 + li;
+      if (vec && i + 1 < n) {
+        const T2 xv = *reinterpret_cast<const T2*>(x + i);
+        xx[2 * h] = xv.x;
+        xx[2 * h + 1] = xv.y;
+        if (v_stride) {
+          const T2 vw = *reinterpret_cast<const T2*>(v + i);
+          vv[2 * h] = vw.x;
+          vv[2 * h + 1] = vw.y;
+        } else {
+          vv[2 * h] = vv[2 * h + 1] = v0;
+        }
       } else {
-        vv[2 * h] = vv[2 * h + 1] = v0;
-      }
-    } else {
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        xx[2 * h + e] = (i + e < n) ? x[i + e] : T(1);
-        vv[2 * h + e] = (i + e < n) ? (v_stride ? v[i + e] : v0) : T(0);
+        for (int e = 0; e < 2; ++e) {
+          xx[2 * h + e] = (i + e < n) ? x[i + e] : T(1);
+          vv[2 * h + e] = (i + e < n) ? (v_stride ? v[i + e] : v0) : T(0);
+        }
       }
     }
   }
-  int key[LB_ITEMS], rank[LB_ITEMS];
+  int key[IT], rank[IT];
 #pragma unroll
-  for (int it = 0; it < LB_ITEMS; ++it) {
-    const int li = tile_offset<NT>(it, tid);
+  for (int it = 0; it < IT; ++it) {
+    const int li = tile_offset<NT, IT>(it, tid);
     const int64_t i = t0 + li;
     int k = NKEYS;                                 // NKEYS: no list entry
     uint8_t keep = 0;
@@ -281,7 +299,7 @@ __device__ __forceinline__ void tile_bin(TileShared<T, NT>& S, const T* __restri
   // exclusive prefix per key over (item round, warp); the key's total to kbeg
   if (tid < NKEYS) {
     int acc = 0;
-    for (int it = 0; it < LB_ITEMS; ++it)
+    for (int it = 0; it < IT; ++it)
       for (int w = 0; w < NT / 32; ++w) {
         const int c = S.wcount[it][w][tid];
         S.wcount[it][w][tid] = (uint16_t)acc;
@@ -307,10 +325,10 @@ __device__ __forceinline__ void tile_bin(TileShared<T, NT>& S, const T* __restri
   if (tid < 8) S.next_chunk[tid] = 0;
   __syncthreads();
 #pragma unroll
-  for (int it = 0; it < LB_ITEMS; ++it)
+  for (int it = 0; it < IT; ++it)
     if (key[it] < NKEYS) {
       const int pos = S.kbeg[key[it]] + S.wcount[it][warp][key[it]] + rank[it];
-      if (LB_CHECK(pos >= 0 && pos < (NT * LB_ITEMS), 1u)) S.list[pos] = (uint16_t)tile_offset<NT>(it, tid);
+      if (LB_CHECK(pos >= 0 && pos < (NT * IT), 1u)) S.list[pos] = (uint16_t)tile_offset<NT, IT>(it, tid);
     }
   __syncthreads();
 }
@@ -335,8 +353,8 @@ __device__ __forceinline__ double vmf_form(double d, double k, double f) {
 // range recompute the chunk's first entry and do not keep it.  `so` (FP64
 // values only) holds the constants of a call whose pairs all have one
 // order, or is NULL.
-template <int KIND, bool DX, typename T, bool SO, int R, int NT>
-__device__ __forceinline__ void tile_eval_region(TileShared<T, NT>& S, int lane, const ScalarOrder* so) {
+template <int KIND, bool DX, typename T, bool SO, int R, int NT, int IT>
+__device__ __forceinline__ void tile_eval_region(TileShared<T, NT, IT>& S, int lane, const ScalarOrder* so) {
   const int b0 = S.rbeg(R), c = S.rend(R) - b0;
   const int nch = (c + 31) >> 5;
   for (;;) {
@@ -347,7 +365,7 @@ __device__ __forceinline__ void tile_eval_region(TileShared<T, NT>& S, int lane,
     const int j0 = id << 5, j = j0 + lane;
     bool ok = j < c;
     int jl = b0 + (ok ? j : j0);
-    if (!LB_CHECK(jl >= 0 && jl < (NT * LB_ITEMS), 2u)) {
+    if (!LB_CHECK(jl >= 0 && jl < (NT * IT), 2u)) {
       jl = 0;                                      // clamped: the warp still runs the expression together
       ok = false;
     }
@@ -356,9 +374,37 @@ __device__ __forceinline__ void tile_eval_region(TileShared<T, NT>& S, int lane,
     int n = S.nt[li];
     if constexpr (sizeof(T) == 8 && (R == R_MU20 || R == R_MU3)) n = mu_counts(f32_cut(v), f32_cut(x));
     if constexpr (sizeof(T) == 8 && KIND == KIND_I && R == R_FALLBACK) n = series_terms(f32_cut(v), f32_cut(x));
-    const T val = tile_expr<KIND, DX, T, SO>(R, v, x, n, so);
+    const T val = tile_expr<KIND, DX, T, SO>(R, v, x, n, so, nullptr);
     __syncwarp();                                  // every lane has read its arguments (sres is sx)
     if (ok) S.sres[li] = val;
+  }
+}
+
+// The K fallback pairs of a tile, in chunks of 32 pairs of one class: with
+// few pairs per tile the chunks are not full, but run side by side on the
+// block's warps instead of one class after another in one warp.
+template <bool DX, int NT, int IT>
+__device__ __forceinline__ void tile_eval_kint(TileShared<double, NT, IT>& S, int lane, const unsigned long long* tab) {
+  for (;;) {
+    int id = 0;
+    if (lane == 0) id = atomicAdd(&S.next_chunk[R_FALLBACK], 1);
+    id = __shfl_sync(0xffffffffu, id, 0);
+    int c = 0, b = 0, e = 0;
+#pragma unroll 1
+    for (; c < 6; ++c) {
+      b = S.kbeg[KEY_FB + c];
+      e = S.kbeg[KEY_FB + c + 1];
+      const int nch = (e - b + 31) >> 5;
+      if (id < nch) break;
+      id -= nch;
+    }
+    if (c == 6) break;
+    const int j = b + (id << 5) + lane;
+    if (j < e) {
+      const int li = S.list[j];
+      S.sres[li] = kt_eval<DX>(S.sv[li], S.sx[li], c, tab);   // sres is sx: read before written, by this lane alone
+    }
+    __syncwarp();
   }
 }
 
@@ -372,23 +418,24 @@ __device__ __forceinline__ void tile_eval_region(TileShared<T, NT>& S, int lane,
 // equal x: their arguments stay in place for it).  Ends with a barrier.
 // vmf_d >= 0 (FP64 log I and its derivative only): the von Mises-Fisher form
 // of the result in dimension vmf_d (vmf_form) is stored instead.
-template <int KIND, bool DX, typename T, bool SO, bool KIN, int NT>
-__device__ __forceinline__ void tile_eval(TileShared<T, NT>& S, T* __restrict__ out, int64_t t0, int64_t n,
+template <int KIND, bool DX, typename T, bool SO, bool KIN, int NT, int IT>
+__device__ __forceinline__ void tile_eval(TileShared<T, NT, IT>& S, T* __restrict__ out, int64_t t0, int64_t n,
                                           const ScalarOrder* so = nullptr, const T* __restrict__ x = nullptr,
-                                          double vmf_d = -1.0) {
+                                          double vmf_d = -1.0, const unsigned long long* tab = nullptr) {
   typedef typename Vec2<T>::type T2;
   const int tid = threadIdx.x, lane = tid & 31;
-  if (KIND == KIND_I || sizeof(T) == 4 || KIN) tile_eval_region<KIND, DX, T, SO, R_FALLBACK, NT>(S, lane, so);
-  tile_eval_region<KIND, DX, T, SO, R_U13, NT>(S, lane, so);
-  tile_eval_region<KIND, DX, T, SO, R_MU20, NT>(S, lane, so);
-  tile_eval_region<KIND, DX, T, SO, R_MU3, NT>(S, lane, so);
+  if constexpr (KIN) tile_eval_kint<DX>(S, lane, tab);
+  else if (KIND == KIND_I || sizeof(T) == 4) tile_eval_region<KIND, DX, T, SO, R_FALLBACK>(S, lane, so);
+  tile_eval_region<KIND, DX, T, SO, R_U13>(S, lane, so);
+  tile_eval_region<KIND, DX, T, SO, R_MU20>(S, lane, so);
+  tile_eval_region<KIND, DX, T, SO, R_MU3>(S, lane, so);
   __syncthreads();
   const bool vec = (reinterpret_cast<uintptr_t>(out) & (2 * sizeof(T) - 1)) == 0;
 #pragma unroll
-  for (int h = 0; h < LB_ITEMS / 2; ++h) {
-    const int li = tile_offset<NT>(2 * h, tid);
+  for (int h = 0; h < (IT + 1) / 2; ++h) {
+    const int li = tile_offset<NT, IT>(2 * h, tid);
     const int64_t i = t0 + li;
-    const bool k0 = i < n && S.keep[li], k1 = i + 1 < n && S.keep[li + 1];
+    const bool k0 = i < n && S.keep[li], k1 = IT > 1 && i + 1 < n && S.keep[li + (IT > 1)];
     if constexpr (sizeof(T) == 8 && KIND == KIND_I) {
       if (vmf_d >= 0.0) {
         if (k0) S.sres[li] = vmf_form<DX>(vmf_d, x[i], S.sres[li]);
@@ -428,11 +475,12 @@ __device__ __forceinline__ double kint_warp_batch(double vi, double xi, int m, i
 // too few pairs for the tiles to fill the GPU.  The groups of expressions
 // present in the warp run one after another; lanes outside the group run on
 // its first pair's arguments, so that the warp stays together, and drop the
-// result.  One kernel, no queue and no shared memory.
-template <int KIND, bool DX>
+// result.  One kernel and no queue; tab: 16 KB of shared memory for the K
+// integral's table (filled if a pair of the block needs it).
+template <int KIND, bool DX, int NT>
 __device__ __forceinline__ void warp_pairs64(const double* __restrict__ v, int64_t v_stride, double v0,
                                              const double* __restrict__ x, double* __restrict__ out, int64_t i,
-                                             bool valid, double vmf_d) {
+                                             bool valid, double vmf_d, unsigned long long* tab) {
   double vi = valid ? (v_stride ? v[i] : v0) : 1.0;
   const double xi = valid ? x[i] : 1.0;
   if constexpr (KIND == KIND_K) vi = fabs(vi);
@@ -446,6 +494,12 @@ __device__ __forceinline__ void warp_pairs64(const double* __restrict__ v, int64
     if (KIND == KIND_I && r == R_FALLBACK) n = series_terms(f32_cut(vi), f32_cut(xi));
     if (r != R_MU20 && r != R_FALLBACK) r = R_U13;         // every uniform expansion
   }
+  if constexpr (KIND == KIND_K) {
+    if (__syncthreads_or(r == R_FALLBACK)) {
+      kt_load_table<NT>(tab);
+      __syncthreads();
+    }
+  }
   unsigned todo = __ballot_sync(0xffffffffu, r != R_SPECIAL);
   while (todo) {
     const int lead = __ffs(todo) - 1, g = __shfl_sync(0xffffffffu, r, lead);
@@ -453,7 +507,7 @@ __device__ __forceinline__ void warp_pairs64(const double* __restrict__ v, int64
     const unsigned members = __ballot_sync(0xffffffffu, in);
     const double vl = __shfl_sync(0xffffffffu, vi, lead), xl = __shfl_sync(0xffffffffu, xi, lead);
     const int nl = __shfl_sync(0xffffffffu, n, lead);
-    const double f = tile_expr<KIND, DX, double, false>(g, in ? vi : vl, in ? xi : xl, in ? n : nl, nullptr);
+    const double f = tile_expr<KIND, DX, double, false>(g, in ? vi : vl, in ? xi : xl, in ? n : nl, nullptr, tab);
     if (in) val = f;
     todo &= ~members;
   }
@@ -461,15 +515,6 @@ __device__ __forceinline__ void warp_pairs64(const double* __restrict__ v, int64
     if (valid && vmf_d >= 0.0) val = vmf_form<DX>(vmf_d, xi, val);
   }
   if (valid) out[i] = val;
-}
-
-// The 16 KB table of kt_exp2_q58 in shared memory (random lookups cost a few
-// bank conflicts there, up to 32 cache-line accesses in global memory).  All
-// NT threads of the block call it; the caller synchronizes.
-template <int NT>
-__device__ __forceinline__ void kt_load_table(unsigned long long* tab) {
-  for (int i = 2 * threadIdx.x; i < 2048; i += 2 * NT)
-    *reinterpret_cast<ulonglong2*>(tab + i) = *reinterpret_cast<const ulonglong2*>(lb_kt_exp2 + i);
 }
 
 // FP32 pairs in tight mode (log I or log K).  Each warp works by itself, with

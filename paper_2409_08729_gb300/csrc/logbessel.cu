@@ -58,14 +58,26 @@ namespace {
 #ifndef LB_KINT_CTAS_PER_SM
 #define LB_KINT_CTAS_PER_SM 4
 #endif
-#ifndef LB_MID_CTAS_PER_SM
-#define LB_MID_CTAS_PER_SM 8
+#ifndef LB_IN_TILE_THREADS_PER_SM
+#define LB_IN_TILE_THREADS_PER_SM 768
+#endif
+#ifndef LB_LOW_THREADS
+#define LB_LOW_THREADS 256
+#endif
+#ifndef LB_LOW_ITEMS
+#define LB_LOW_ITEMS 1
+#endif
+#ifndef LB_MID_THREADS
+#define LB_MID_THREADS 256
+#endif
+#ifndef LB_MID_ITEMS
+#define LB_MID_ITEMS 2
 #endif
 #ifndef LB_SMALL_THREADS
 #define LB_SMALL_THREADS 64
 #endif
 #ifndef LB_SMALL_N
-#define LB_SMALL_N 12000
+#define LB_SMALL_N 2000
 #endif
 #ifndef LB_TILES32_CTAS_PER_SM
 #define LB_TILES32_CTAS_PER_SM 6
@@ -101,19 +113,25 @@ constexpr uint32_t kQueueOffsetMask = (1u << kQueueOffsetBits) - 1u;
 // v == NULL: the order of every pair is v0 (v_stride 0).
 // vmf_d >= 0: see tile_eval.
 __host__ __device__ constexpr int tiles_ctas(int nt, bool kin) {
-  return nt == kTileThreads ? LB_TILES_CTAS_PER_SM : (kin ? LB_MID_CTAS_PER_SM : LB_TILES_CTAS_PER_SM * kTileThreads / nt);
+  return (kin ? LB_IN_TILE_THREADS_PER_SM : LB_TILES_CTAS_PER_SM * kTileThreads) / nt;
 }
-template <int KIND, bool DX, typename T, bool SO, int NT, bool KIN>
+template <int KIND, bool DX, typename T, bool SO, int NT, int IT, bool KIN>
 __global__ void __launch_bounds__(NT, tiles_ctas(NT, KIN))
 lb_tiles_kernel(const T* __restrict__ v, int64_t v_stride, T v0, const T* __restrict__ x, T* __restrict__ out,
                 int64_t n, int mode, int forced_region, unsigned int* __restrict__ qcount,
                 uint32_t* __restrict__ queue, int64_t qcap, double vmf_d) {
   static_assert(!SO || (sizeof(T) == 8 && !DX), "per-order constants are built for FP64 values");
-  constexpr int kPairs = NT * LB_ITEMS;
-  __shared__ TileShared<T, NT> S;
+  constexpr int kPairs = NT * IT;
+  __shared__ TileShared<T, NT, IT> S;
   const int tid = threadIdx.x;
   const int64_t ntiles = (n + kPairs - 1) / kPairs;
   if (v_stride == 0 && v) v0 = v[0];
+  const unsigned long long* tab = nullptr;
+  if constexpr (KIN) {
+    __shared__ __align__(16) unsigned long long T2[2048];
+    kt_load_table<NT>(T2);                          // a barrier of tile_bin stands between this and its use
+    tab = T2;
+  }
   const ScalarOrder* so = nullptr;
   if constexpr (SO) {
     __shared__ ScalarOrder SOC;
@@ -123,7 +141,7 @@ lb_tiles_kernel(const T* __restrict__ v, int64_t v_stride, T v0, const T* __rest
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t t0 = tile * kPairs;
     tile_bin<KIND, DX, T, KIN>(S, v, v_stride, v0, x, t0, n, mode, forced_region);
-    tile_eval<KIND, DX, T, SO, KIN>(S, out, t0, n, so, x, vmf_d);
+    tile_eval<KIND, DX, T, SO, KIN>(S, out, t0, n, so, x, vmf_d, tab);
     if (KIND == KIND_K && sizeof(T) == 8 && !KIN) {
       const int c = S.rcount(R_FALLBACK), f0 = S.rbeg(R_FALLBACK);
       if (c > 0) {
@@ -157,7 +175,8 @@ lb_small_kernel(const double* __restrict__ v, int64_t v_stride, double v0, const
   if (v_stride == 0 && v) v0 = v[0];
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * LB_SMALL_THREADS + threadIdx.x) >> 5, i = warp * ppw + lane;
-  warp_pairs64<KIND, DX>(v, v_stride, v0, x, out, i, lane < ppw && i < n, vmf_d);
+  __shared__ __align__(16) unsigned long long tab[KIND == KIND_K ? 2048 : 2];
+  warp_pairs64<KIND, DX, LB_SMALL_THREADS>(v, v_stride, v0, x, out, i, lane < ppw && i < n, vmf_d, tab);
 }
 
 // K integral, tight FP64: one thread per queued pair (lb_ktrap.cuh).  A
@@ -477,21 +496,25 @@ lb_status run_tiles32(const float* v, int64_t v_stride, const float* x, float* o
 //
 // FP64 calls of total_n pairs (the caller's n; passes and pieces of one call
 // take the same route, so that their results are those of one pass):
-//   up to LB_SMALL_N     lb_small_kernel alone (tight mode);
-//   below 2^17           tiles of 512 pairs, the K fallback in the tile (tight
-//                        mode): one launch and no scratch;
-//   below 2^20           tiles of 512 pairs, K fallback queued;
-//   from there           tiles of 2048 pairs, K fallback queued.
+//   up to LB_SMALL_N  lb_small_kernel alone (tight mode);
+//   below 2^17        tiles of 256 pairs, one per thread, the K fallback in the
+//                     tile (tight mode): one launch and no scratch;
+//   below 2^20        tiles of 512 pairs, two per thread, K fallback queued;
+//   from there        tiles of 2048 pairs, four per thread, K fallback queued.
+// Device time of a call on the mixed-order sweep, log I / log K, us: 1000
+// pairs 12 / 14 (small kernel) against 18 / 16 (256-pair tiles) and 29 / 37
+// (2048-pair tiles, queued); 24000 pairs 19 / 17 against 29 / 41 (small
+// kernel 29 / 35); 100000 pairs 25 / 26 against 31 / 43; 1M pairs 105 / 115
+// against 119 / 129.
 constexpr int64_t kMidInTile = (int64_t)1 << 17, kMid = (int64_t)1 << 20;
-constexpr int kMidThreads = 128;
 
-template <int KIND, bool DX, typename T, bool SO, int NT, bool KIN>
+template <int KIND, bool DX, typename T, bool SO, int NT, int IT, bool KIN>
 lb_status launch_tiles(int sms, cudaStream_t st, const T* v, int64_t v_stride, T v0, const T* x, T* out, int64_t n,
                        int mode, int forced_region, unsigned int* qcount, uint32_t* queue, int64_t cap, double vmf_d) {
-  const int64_t ntiles = (n + NT * LB_ITEMS - 1) / (NT * LB_ITEMS), most = (int64_t)sms * tiles_ctas(NT, KIN);
+  const int64_t ntiles = (n + NT * IT - 1) / (NT * IT), most = (int64_t)sms * tiles_ctas(NT, KIN);
   const int grid = (int)(ntiles < most ? ntiles : most);
   return launch(PS_TILES, st, [&] {
-    lb_tiles_kernel<KIND, DX, T, SO, NT, KIN><<<grid, NT, 0, st>>>(v, v_stride, v0, x, out, n, mode, forced_region,
+    lb_tiles_kernel<KIND, DX, T, SO, NT, IT, KIN><<<grid, NT, 0, st>>>(v, v_stride, v0, x, out, n, mode, forced_region,
                                                                   qcount, queue, cap, vmf_d);
   });
 }
@@ -506,16 +529,19 @@ lb_status run_tiles(int sms, cudaStream_t st, const T* v, int64_t v_stride, T v0
     const bool so = !DX && v_stride == 0 && forced_region < 0;
     if (total_n < kMid && forced_region < 0) {
       if (so && total_n >= kMidInTile)
-        return launch_tiles<KIND, DX, T, !DX, kMidThreads, false>(sms, st, v, v_stride, v0, x, out, n, mode,
+        return launch_tiles<KIND, DX, T, !DX, LB_MID_THREADS, LB_MID_ITEMS, false>(sms, st, v, v_stride, v0, x, out, n, mode,
                                                                   forced_region, qcount, queue, cap, vmf_d);
-      return launch_tiles<KIND, DX, T, false, kMidThreads, false>(sms, st, v, v_stride, v0, x, out, n, mode,
-                                                                  forced_region, qcount, queue, cap, vmf_d);
+      if (total_n < kMidInTile)
+        return launch_tiles<KIND, DX, T, false, LB_LOW_THREADS, LB_LOW_ITEMS, false>(
+            sms, st, v, v_stride, v0, x, out, n, mode, forced_region, qcount, queue, cap, vmf_d);
+      return launch_tiles<KIND, DX, T, false, LB_MID_THREADS, LB_MID_ITEMS, false>(
+          sms, st, v, v_stride, v0, x, out, n, mode, forced_region, qcount, queue, cap, vmf_d);
     }
     if (so)
-      return launch_tiles<KIND, DX, T, !DX, kTileThreads, false>(sms, st, v, v_stride, v0, x, out, n, mode,
+      return launch_tiles<KIND, DX, T, !DX, kTileThreads, LB_ITEMS, false>(sms, st, v, v_stride, v0, x, out, n, mode,
                                                                  forced_region, qcount, queue, cap, vmf_d);
   }
-  return launch_tiles<KIND, DX, T, false, kTileThreads, false>(sms, st, v, v_stride, v0, x, out, n, mode,
+  return launch_tiles<KIND, DX, T, false, kTileThreads, LB_ITEMS, false>(sms, st, v, v_stride, v0, x, out, n, mode,
                                                                forced_region, qcount, queue, cap, vmf_d);
 }
 
@@ -539,7 +565,7 @@ lb_status run_impl(const T* v, int64_t v_stride, const T* x, T* out, int64_t n, 
       });
     }
     if (KIND == KIND_K && total_n < kMidInTile)
-      return launch_tiles<KIND, DX, T, false, kMidThreads, KIND == KIND_K>(sms, st, v, v_stride, v0, x, out, n, mode,
+      return launch_tiles<KIND, DX, T, false, LB_LOW_THREADS, LB_LOW_ITEMS, KIND == KIND_K>(sms, st, v, v_stride, v0, x, out, n, mode,
                                                                            forced_region, nullptr, nullptr, 0, vmf_d);
   }
   if (KIND == KIND_I || sizeof(T) == 4 || (forced_region >= 0 && forced_region != R_FALLBACK))
