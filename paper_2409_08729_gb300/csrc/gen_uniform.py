@@ -9,14 +9,16 @@ E, O of positive coefficients.  With y = p^2/2, g = p/2 and 8/r as variables
 
     E: |c_2i| 2^i / 8^k,   O: |c_(2i+1)| 2^(i+1) / 8^k      (Q56)
 
-as pairs (E_i, O_i), i = 0 .. k // 2, for k = 1 .. 13 in turn.
+as pairs (E_i, O_i), i = 0 .. k // 2, for k = 1 .. 13 in turn.  The second
+table holds Q_k = k P_k + 2 p P_k', for the x-derivative: the same entries
+times k + 2 (2i) and k + 2 (2i + 1), in Q50.
 """
 from gen_debye import debye_polys
 
 
 def main():
     u = debye_polys(13)
-    rows, offs = [], [0, 0]
+    rows, drows, offs = [], [], [0, 0]
     for k in range(1, 14):
         c = [u[k].get(k + 2 * i, 0) for i in range(k + 1)]
         assert all((a > 0) == (i % 2 == 0) for i, a in enumerate(c))
@@ -24,6 +26,7 @@ def main():
             e = abs(c[2 * i]) * 2 ** i / 8 ** k
             o = abs(c[2 * i + 1]) * 2 ** (i + 1) / 8 ** k if 2 * i + 1 <= k else 0
             rows.append(tuple(int(round(a * 2 ** 56)) for a in (e, o)))
+            drows.append(tuple(int(round(a * 2 ** 50)) for a in ((k + 4 * i) * e, (k + 4 * i + 2) * o)))
         offs.append(len(rows))
     print("// Generated by gen_uniform.py: do not edit.")
     print("#pragma once")
@@ -33,10 +36,11 @@ def main():
     print("#define LB_UNI_TABLE static const")
     print("#endif")
     print("LB_UNI_TABLE int lb_uni_off[15] = {%s};" % ", ".join(map(str, offs)))
-    print("LB_UNI_TABLE unsigned long long lb_uni[%d][2] = {" % len(rows))
-    for e, o in rows:
-        print("    {0x%016xull, 0x%016xull}," % (e, o))
-    print("};")
+    for name, t in (("lb_uni", rows), ("lb_uniq", drows)):
+        print("LB_UNI_TABLE unsigned long long %s[%d][2] = {" % (name, len(t)))
+        for e, o in t:
+            print("    {0x%016xull, 0x%016xull}," % (e, o))
+        print("};")
 
 
 if __name__ == "__main__":

@@ -584,30 +584,40 @@ __device__ __forceinline__ double series_so(const ScalarOrder& so, double x, int
 // (Sec. 7), and these follow directly from its Eqs.
 // ---------------------------------------------------------------------------
 
-// 1/k and (2k-1)^2/k for k = 1..20 (entry 0 unused).
-static __constant__ double kMuInvK[21] = {0.0, 1.0 / 1.0, 1.0 / 2.0, 1.0 / 3.0, 1.0 / 4.0, 1.0 / 5.0, 1.0 / 6.0, 1.0 / 7.0, 1.0 / 8.0, 1.0 / 9.0, 1.0 / 10.0, 1.0 / 11.0, 1.0 / 12.0, 1.0 / 13.0, 1.0 / 14.0, 1.0 / 15.0, 1.0 / 16.0, 1.0 / 17.0, 1.0 / 18.0, 1.0 / 19.0, 1.0 / 20.0};
-static __constant__ double kMuOddK[21] = {0.0, 1.0 / 1.0, 9.0 / 2.0, 25.0 / 3.0, 49.0 / 4.0, 81.0 / 5.0, 121.0 / 6.0, 169.0 / 7.0, 225.0 / 8.0, 289.0 / 9.0, 361.0 / 10.0, 441.0 / 11.0, 529.0 / 12.0, 625.0 / 13.0, 729.0 / 14.0, 841.0 / 15.0, 961.0 / 16.0, 1089.0 / 17.0, 1225.0 / 18.0, 1369.0 / 19.0, 1521.0 / 20.0};
-
 // mu_K: log f = +-x - log(2 pi x)/2 + log S (I: +x, K: -x and +log(pi/2)/2),
-// S = 1 + sum_k c_k x^-k, so d/dx log f = +-1 - 1/(2x) - (sum_k k c_k x^-k) / (x S).
-// Over the first n terms only (n: the pair's term count, made warp-uniform),
-// as a rolled loop: the terms past n are below 2^-56 of S.
+// S = 1 + sum_k c_k w^k, w = 1/(8x), so with E = w dS/dw
+//   d/dx log f = +-1 - (1/x) (1/2 + E/S).
+// The sums as mu_expr_n's: Q <- D_k Q + 20!/(k-1)! and, D_k being
+// proportional to w, R <- D_k (Q + R) beside it; the terms past the leading
+// h in double-float, at most cap terms.
 template <int KIND>
-__device__ __forceinline__ double mu_dx_n(double v, double x, int n) {
-  n = __reduce_max_sync(0xffffffffu, n);
-  const double mu = 4.0 * v * v;
-  const double rx = ix_rcp(8.0 * x);                // on the integer pipe
-  const double inv8x = (KIND == KIND_I) ? -rx : rx;  // the sign folded in
-  double term = 1.0, S = 1.0, D = 0.0, kd = 0.0;
+__device__ __forceinline__ double mu_dx_n(double v, double x, int counts, int cap) {
+  const int n = __reduce_max_sync(0xffffffffu, min(cap, counts & 255));
+  const int h = min(n, __reduce_max_sync(0xffffffffu, counts >> 8));
+  const double rx = ix_rcp_call(8.0 * x);           // on the integer pipe
+  const double w = (KIND == KIND_I) ? -rx : rx;      // the sign folded in
+  const double A = (4.0 * v * v) * w;
+  double Q = kMuF[n + 1], R = 0.0;
+  if (n > h) {
+    const dfloat wd = df_from_double(w), Ad = df_from_double(A);
+    dfloat Qd = df_make(kMuFd[n + 1][0], kMuFd[n + 1][1]), Rd = df_make(0.0f, 0.0f);
 #pragma unroll 1
-  for (int k = 1; k <= n; ++k) {
-    kd += 1.0;
-    term *= fma(mu, kMuInvK[k], -kMuOddK[k]) * inv8x;
-    S += term;
-    D = fma(kd, term, D);
+    for (int k = n; k > h; --k) {
+      const dfloat D = df_mulf_add(wd, -kMuOdd[k], Ad);
+      Rd = df_mul(D, df_add(Qd, Rd));
+      Qd = df_mul_add(D, Qd, df_make(kMuFd[k][0], kMuFd[k][1]));
+    }
+    Q = df_to_double(Qd);
+    R = df_to_double(Rd);
+  }
+#pragma unroll 1
+  for (int k = h; k >= 1; --k) {
+    const double D = fma(-kMuOddD[k], w, A);
+    R = D * (Q + R);
+    Q = fma(D, Q, kMuF[k]);
   }
   const double base = (KIND == KIND_I) ? 1.0 : -1.0;
-  return base - (8.0 * rx) * fma(D, ix_rcp(S), 0.5);
+  return base - (8.0 * rx) * fma(R, ix_rcp_call(Q), 0.5);
 }
 
 // U_K: with x' = x/v, t = (1 + x'^2)^-1/2, d(v eta)/dx = 1/(t x'),
@@ -615,9 +625,10 @@ __device__ __forceinline__ double mu_dx_n(double v, double x, int n) {
 // d/dt u_k(t) = t^(k-1) Q_k(t^2):
 //   d/dx log f = +-1/(t x') - (x' t^2 / v) (1/2 + SQ / S),
 //   S = 1 + sum q^k P_k(t^2), SQ = sum q^k Q_k(t^2), q = +-t/v.
-// K: the pair's own terms (its region's).
+// Evaluated by u_dx_fx (lb_uniform.cuh) wherever u_fx serves the values; this
+// form for the rest.  K: the pair's own terms.
 template <int KIND>
-__device__ __forceinline__ double u_dx(double v, double x, int K) {
+static __device__ __noinline__ double u_dx(double v, double x, int K) {
   const double inv_v = ix_rcp(v);                  // reciprocals and 1/sqrt on the integer pipe
   const double xp = x * inv_v;
   double r, t;

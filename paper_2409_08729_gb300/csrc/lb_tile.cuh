@@ -54,8 +54,8 @@ static __device__ unsigned int lb_check_status;
 
 // List keys.  mu_20 (FP64) takes one key per term count n = 1..20 (mu_counts);
 // the uniform expansions U_13 .. U_4 share one range of ten keys, by the
-// pair's number of terms, largest first (for FP64 values at most the
-// region's, uni_terms); the power series one key per band of x, log-spaced,
+// pair's number of terms, largest first (in FP64 at most the region's,
+// uni_terms); the power series one key per band of x, log-spaced,
 // 2 log2(1 + x) (its term count grows with x: rank correlation 0.98), because
 // its exact count is a loop of up to 90 steps that is cheaper once per
 // 32-pair chunk than once per item round.  So each region's pairs come
@@ -143,10 +143,14 @@ __device__ __forceinline__ T tile_expr(int r, T v, T x, int n, const ScalarOrder
     }
   } else if constexpr (DX) {
     switch (r) {
-      case R_MU20: return mu_dx_n<KIND>(v, x, n & 255);
-      case R_MU3: return mu_dx_n<KIND>(v, x, 3);
+      case R_MU20: return mu_dx_n<KIND>(v, x, n, 20);
+      case R_MU3: return mu_dx_n<KIND>(v, x, n, 3);
       case R_FALLBACK: return (KIND == KIND_I) ? series_dx_n(v, x, n) : kt_eval<true>(v, x, n, tab);
-      default: return u_dx<KIND>(v, x, n);
+      default: {
+        const int Kmax = __reduce_max_sync(0xffffffffu, n);
+        const double s = fma(v, v, x * x);
+        return uni_ok(s, x) ? u_dx_fx(KIND, v, x, s, n, Kmax) : u_dx<KIND>(v, x, n);
+      }
     }
   } else {
     switch (r) {
@@ -188,9 +192,9 @@ __device__ __forceinline__ int tile_key(int r, T v, T x, int* n) {
     return KEY_FB;
   }
   int K = region_terms(r);
-  if constexpr (sizeof(T) == 8 && !DX) {
-    const float vf = f32_cut(v), xf = f32_cut(x);
-    K = uni_terms(fmaf(vf, vf, xf * xf), K);
+  if constexpr (sizeof(T) == 8) {
+    const float vf = f32_cut(v), xf = f32_cut(x), s = fmaf(vf, vf, xf * xf);
+    K = DX ? uni_terms_dx(s, K) : uni_terms(s, K);
   }
   *n = K;
   return KEY_U + 13 - K;

@@ -85,4 +85,43 @@ LB_IX_FN double u_fx(int kind, double v, double x, double s, int K, int Kmax) {
   return -fma(w, a, fma(-0x1p-54, (double)(lw + kLogHalfPiQ53), r));
 }
 
+// Terms for the x-derivative, whose sum's term k is k times the value's: the
+// value's rule at r/1.31 (1.31 = 5^(1/6), the most that (K + 1)^(1/(K + 2)) is).
+LB_IX_FN int uni_terms_dx(float f, int cap) { return uni_terms(f * 0.58f, cap); }
+
+// d/dx log I or log K of one pair, arguments as u_fx (K: uni_terms_dx).  r
+// alone depends on x:
+//   d/dx log f = +-r/x - (x/r^2) (1/2 + SQ/S),  SQ = sum_k (+-1/r)^k Q_k(p),
+// Q_k = k P_k + 2 p P_k'.  SQ is below 0.3/r of a factor that is below 1/r of
+// the result: its 2^-50 and S's 2^-56 are far below the result's last place.
+LB_IX_FN double u_dx_fx(int kind, double v, double x, double s, int K, int Kmax) {
+  const double q = kt_rsqrt(s), r = s * q;
+  const uint64_t t = (uint64_t)ix_fix(v * q, 63);
+  const uint64_t g = ix_umulhi(t, t) << 1;
+  const uint64_t y = ix_umulhi(g, g) << 1;
+  const int64_t h = kind ? -ix_fix(q, 67) : ix_fix(q, 67);
+  int64_t acc = 0, dcc = 0;
+#pragma unroll 1
+  for (int k = Kmax; k >= 1; --k) {
+    const int b = lb_uni_off[k];
+    int i = lb_uni_off[k + 1] - 1;
+    uint64_t e = lb_uni[i][0], o = lb_uni[i][1], de = lb_uniq[i][0], dd = lb_uniq[i][1];
+#pragma unroll 1
+    for (--i; i >= b; --i) {
+      e = lb_uni[i][0] + kt_mulhi(e, y);
+      o = lb_uni[i][1] + kt_mulhi(o, y);
+      de = lb_uniq[i][0] + kt_mulhi(de, y);
+      dd = lb_uniq[i][1] + kt_mulhi(dd, y);
+    }
+    acc = ix_mulhi(acc, h) + (int64_t)(e - kt_mulhi(o, g));
+    dcc = ix_mulhi(dcc, h) + (int64_t)(de - kt_mulhi(dd, g));
+    if (k > K) acc = dcc = 0;
+  }
+  const double S = (double)((1ll << 56) + ix_mulhi(acc, h));          // Q56
+  const double SQ = (double)ix_mulhi(dcc, h) * 64.0;                  // Q50 to Q56
+  const double corr = (x * q) * q * fma(SQ, kt_rcp(S), 0.5);
+  const double lead = r * kt_rcp(x);
+  return kind ? -lead - corr : lead - corr;
+}
+
 }  // namespace lb
