@@ -459,6 +459,25 @@ __device__ __forceinline__ dfloat series_ratio_df(dfloat y, dfloat v, int k) {
   return r;
 }
 
+// 1/Gamma(v + 1) = g / p for 2 <= v <= 30 (g below 2, p a product of at most 30
+// factors): 1/Gamma(1 + mu) from Temme's Gamma_1 and Gamma_2 in fixed point
+// (kt_small), v = n + mu, and p = v (v - 1) ... (mu + 1).
+__device__ __forceinline__ void series_rgamma(double v, double& g, double& p) {
+  const int n = (int)(f32_cut(v) + 0.5f);
+  const double mu = v - (double)n;
+  int64_t q1, q2;
+  const int64_t mq = ix_fix(mu, 62);
+  kt_gammas(mq, q1, q2);
+  g = (double)(q2 - (ix_mulhi(mq, q1) << 2)) * 0x1p-62;
+  p = 1.0;
+  double u = v;
+#pragma unroll 1
+  for (int j = 0; j < n; ++j) {
+    p *= u;
+    u -= 1.0;
+  }
+}
+
 __device__ __forceinline__ double series_log_i_n(double v, double x, int packed) {
   const int n = __reduce_max_sync(0xffffffffu, series_count(packed));
   const int h = __reduce_max_sync(0xffffffffu, series_head(packed));
@@ -481,7 +500,17 @@ __device__ __forceinline__ double series_log_i_n(double v, double x, int packed)
     A = fma(d, B, y * A);
     B *= d;
   }
-  double res = ix_log_call(A * ix_rcp_call(B)) - lgamma(v + 1.0);
+  double res;
+  // from v = 2 on the result is of the size of v log(2v/x) or larger, where the
+  // product's roundings do not show; below, the library's lgamma keeps the
+  // last bits (8.3e-16 against 6.7e-16 at v = 0.5)
+  if (LB_GE(v, 2.0) && LB_LE(v, 30.0)) {
+    double g, p;
+    series_rgamma(v, g, p);
+    res = ix_log_call(kt_div(A * g, B * p));
+  } else {
+    res = ix_log_call(A * ix_rcp_call(B)) - lgamma(v + 1.0);
+  }
   if ((__double_as_longlong(v) << 1) != 0) res = fma(v, ix_log_call(0.5 * x), res);   // v != 0, on the bits
   return res;
 }
@@ -505,7 +534,7 @@ struct ScalarOrder {
   double v, lg1;                        // v, lgamma(v + 1)
   int muj;                              // W = 2^muj w <= 1/2 wherever the dispatch takes mu_20
   long long muc;                        // log constant of mu_K, Q53, the scale of mu[] included
-  long long mu[21];                     // a_0..a_20 / 2^(k muj) (sign s of the kind folded in), Q(60 - muq)
+  long long mu[21];                     // a_0..a_20 / 2^(k muj) (sign s of the kind folded in), Q(59 - muq), + 2^62
   double ser[91];                       // 1 / (k (k + v)), k = 1..90
   dfloat serd[91];                      // ser[] in double-float
 };
@@ -529,11 +558,11 @@ __device__ __forceinline__ void scalar_order_setup(ScalarOrder& so, double v) {
       c[k] = a;
       big = fmax(big, fabs(a));
     }
-    // |c_k| 2^(60 - muq) < 2^61: with W <= 1/2 every Horner step stays below 2^62
+    // |c_k| 2^(59 - muq) < 2^60: with W <= 1/2 every Horner sum stays within +-2^61
     const int muq = big < 1e15 ? ilogb(big) : 50;
-    for (int k = 0; k <= 20; ++k) so.mu[k] = ix_fix(c[k], 60 - muq);
+    for (int k = 0; k <= 20; ++k) so.mu[k] = ix_fix(c[k], 59 - muq) + (1ll << 62);
     so.muj = j;
-    so.muc = (KIND == KIND_I ? kMuSoLogI : kMuSoLogK) - 2 * (60 - muq) * kLn2Q53;
+    so.muc = (KIND == KIND_I ? kMuSoLogI : kMuSoLogK) - 2 * (59 - muq) * kLn2Q53;
   }
   if (tid >= 32)
     for (int k = tid - 31; k <= 90; k += NT - 32) {
@@ -547,11 +576,14 @@ template <int KIND>
 __device__ __forceinline__ double mu_expr_so(const ScalarOrder& so, double x, int counts) {
   const int n = __reduce_max_sync(0xffffffffu, counts & 255);
   const double rx = ix_rcp_call(8.0 * x);
-  const long long W = ix_fix(rx, 64 + so.muj);    // below 2^63
-  long long acc = so.mu[n];
-#pragma unroll 1
-  for (int k = n - 1; k >= 0; --k) acc = so.mu[k] + ix_mulhi(acc, W);
-  const double S = (double)acc;
+  const uint64_t W = (uint64_t)ix_fix(rx, 64 + so.muj);   // below 2^63
+  // Horner on the sums plus 2^62 (positive: the short unsigned product), the
+  // bias's product taken off again
+  const uint64_t bias = W >> 2;
+  uint64_t acc = (uint64_t)so.mu[n];
+#pragma unroll 2
+  for (int k = n - 1; k >= 0; --k) acc = (uint64_t)so.mu[k] + kt_mulhi(acc, W) - bias;
+  const double S = (double)(long long)(acc - (1ull << 62));
   return fma(0x1p-54, log_q53_plus(S * S * rx, so.muc), KIND == KIND_I ? x : -x);
 }
 

@@ -170,17 +170,9 @@ LB_IX_FN double kt_div(double n, double d) {
   return fma(r, fma(-q, d, n), q);
 }
 
-// Small arguments, x < 2^-9, v <= 16.5: Temme's series for K_mu and
-// K_(mu+1), v = n + mu, |mu| <= 1/2 (J. Comput. Phys. 19, 1975; y = x^2/4 <
-// 2^-20, so two terms past the leading one), then n steps of
-// K_(u+1) = K_(u-1) + (2u/x) K_u, on (x/2)^(u - mu) K_u, which neither
-// overflows nor divides.  Gamma_1 and Gamma_2 are summed in integers.
-template <bool DX>
-LB_IX_FN double kt_small(double v, double x) {
-  const int n = (int)(v + 0.5);
-  double mu = v - (double)n;
-  const double L = kKtLn2 - kt_log(x);                      // log(2/x) >= 6.9
-  const int64_t mq = ix_fix(mu, 62);
+// Temme's Gamma_1(mu) and Gamma_2(mu) in Q62 (1/Gamma(1 +- mu) = Gamma_2 -+ mu
+// Gamma_1), |mu| <= 1/2 in Q62, by their Taylor series in mu^2.
+LB_IX_FN void kt_gammas(int64_t mq, int64_t& g1, int64_t& g2) {
   const int64_t m2 = ix_mulhi(mq, mq) << 4;                 // mu^2, Q64
   int64_t q1 = LB_KT_G1_8, q2 = LB_KT_G2_8;
   q1 = LB_KT_G1_7 + ix_mulhi(q1, m2);
@@ -199,6 +191,22 @@ LB_IX_FN double kt_small(double v, double x) {
   q2 = LB_KT_G2_1 + ix_mulhi(q2, m2);
   q1 = LB_KT_G1_0 + ix_mulhi(q1, m2);
   q2 = LB_KT_G2_0 + ix_mulhi(q2, m2);
+  g1 = q1;
+  g2 = q2;
+}
+
+// Small arguments, x < 2^-9, v <= 16.5: Temme's series for K_mu and
+// K_(mu+1), v = n + mu, |mu| <= 1/2 (J. Comput. Phys. 19, 1975; y = x^2/4 <
+// 2^-20, so two terms past the leading one), then n steps of
+// K_(u+1) = K_(u-1) + (2u/x) K_u, on (x/2)^(u - mu) K_u, which neither
+// overflows nor divides.  Gamma_1 and Gamma_2 are summed in integers.
+template <bool DX>
+LB_IX_FN double kt_small(double v, double x) {
+  const int n = (int)(v + 0.5);
+  double mu = v - (double)n;
+  const double L = kKtLn2 - kt_log(x);                      // log(2/x) >= 6.9
+  int64_t q1, q2;
+  kt_gammas(ix_fix(mu, 62), q1, q2);
   const double G1 = (double)q1 * 0x1p-62, G2 = (double)q2 * 0x1p-62;
   const double mg = mu * G1;
   const double gp = kt_rcp(G2 - mg), gm = kt_rcp(G2 + mg);   // Gamma(1 + mu), Gamma(1 - mu)

@@ -873,11 +873,11 @@ lb_status logbessel_host(int fn, lb_dtype dtype, const void* v, int64_t v_stride
   if (fn < 0 || fn > 3) return fail(LB_EINVAL, "fn must be 0..3 (got %s%lld)", "", (long long)fn);
   lb_status s = validate(dtype, v, v_stride, x, out, n, (int)mode);
   if (s != LB_OK || n == 0) return s;
-  // default pieces of up to 16M pairs: on the sweep's 24 calls per step 2^24
-  // measured 7.35 Gevals/s end to end against 7.17 (2^23), 6.88 (2^25) and
-  // 6.62 (2^26): smaller pieces cost more kernel ends, larger ones longer
-  // unoverlapped first and last copies
-  if (chunk <= 0) chunk = (int64_t)1 << 24;
+  // default pieces of up to 2M pairs: log K on 8M pairs takes 1.00 ms end to
+  // end against 0.98 (2^20), 1.20 (2^22) and 1.11 ms (2^24), on 20M pairs 2.12
+  // against 2.10, 2.16 and 2.37: larger ones leave longer first and last copies
+  // unoverlapped, smaller ones cost more kernel ends
+  if (chunk <= 0) chunk = (int64_t)1 << 21;
   if (chunk > kChunk) chunk = kChunk;
   if ((fn >= 2 && dtype != LB_F64) || (fn == 3 && mode != LB_TIGHT))
     return fail(LB_ENOTSUP, "%sthe derivatives are implemented for LB_F64 (and LB_TIGHT for K) only", "", 0);
