@@ -459,25 +459,6 @@ __device__ __forceinline__ dfloat series_ratio_df(dfloat y, dfloat v, int k) {
   return r;
 }
 
-// 1/Gamma(v + 1) = g / p for 2 <= v <= 30 (g below 2, p a product of at most 30
-// factors): 1/Gamma(1 + mu) from Temme's Gamma_1 and Gamma_2 in fixed point
-// (kt_small), v = n + mu, and p = v (v - 1) ... (mu + 1).
-__device__ __forceinline__ void series_rgamma(double v, double& g, double& p) {
-  const int n = (int)(f32_cut(v) + 0.5f);
-  const double mu = v - (double)n;
-  int64_t q1, q2;
-  const int64_t mq = ix_fix(mu, 62);
-  kt_gammas(mq, q1, q2);
-  g = (double)(q2 - (ix_mulhi(mq, q1) << 2)) * 0x1p-62;
-  p = 1.0;
-  double u = v;
-#pragma unroll 1
-  for (int j = 0; j < n; ++j) {
-    p *= u;
-    u -= 1.0;
-  }
-}
-
 __device__ __forceinline__ double series_log_i_n(double v, double x, int packed) {
   const int n = __reduce_max_sync(0xffffffffu, series_count(packed));
   const int h = __reduce_max_sync(0xffffffffu, series_head(packed));
@@ -500,17 +481,7 @@ __device__ __forceinline__ double series_log_i_n(double v, double x, int packed)
     A = fma(d, B, y * A);
     B *= d;
   }
-  double res;
-  // from v = 2 on the result is of the size of v log(2v/x) or larger, where the
-  // product's roundings do not show; below, the library's lgamma keeps the
-  // last bits (8.3e-16 against 6.7e-16 at v = 0.5)
-  if (LB_GE(v, 2.0) && LB_LE(v, 30.0)) {
-    double g, p;
-    series_rgamma(v, g, p);
-    res = ix_log_call(kt_div(A * g, B * p));
-  } else {
-    res = ix_log_call(A * ix_rcp_call(B)) - lgamma(v + 1.0);
-  }
+  double res = ix_log_call(A * ix_rcp_call(B)) - lgamma(v + 1.0);
   if ((__double_as_longlong(v) << 1) != 0) res = fma(v, ix_log_call(0.5 * x), res);   // v != 0, on the bits
   return res;
 }
