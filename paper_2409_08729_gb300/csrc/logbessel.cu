@@ -82,11 +82,17 @@ namespace {
 #ifndef LB_TILES32_CTAS_PER_SM
 #define LB_TILES32_CTAS_PER_SM 6
 #endif
+#ifndef LB_KTRAP_THREADS
+#define LB_KTRAP_THREADS 512
+#endif
+#ifndef LB_KTRAP_WINDOW
+#define LB_KTRAP_WINDOW 15872
+#endif
 #ifndef LB_KTRAP_CTAS_PER_SM
-#define LB_KTRAP_CTAS_PER_SM 6
+#define LB_KTRAP_CTAS_PER_SM 3
 #endif
 #ifndef LB_KTRAP_CTAS_PER_SM_DX
-#define LB_KTRAP_CTAS_PER_SM_DX 4
+#define LB_KTRAP_CTAS_PER_SM_DX 2
 #endif
 __host__ __device__ constexpr int ktrap_ctas(bool dx) { return dx ? LB_KTRAP_CTAS_PER_SM_DX : LB_KTRAP_CTAS_PER_SM; }
 
@@ -181,65 +187,78 @@ lb_small_kernel(const double* __restrict__ v, int64_t v_stride, double v0, const
 
 // K integral, tight FP64: one thread per queued pair (lb_ktrap.cuh).  A
 // block takes windows of the queue, sorts each by the pairs' classes and
-// bands in shared memory (a counting sort of 48 keys) and hands out chunks of
-// 32 pairs of one class to its warps, costliest class first, so that a warp
-// runs one class's code on lanes that need about as many nodes.  The order of
-// a key's pairs varies from run to run; a pair's result depends on the pair
-// alone.  A window is the queue's share of a block, at most 2048.
-constexpr int kKtWindow = 2048;
+// bands in shared memory (a counting sort of 48 keys, two passes over the
+// window) and hands out chunks of 32 pairs of one class to its warps,
+// costliest class first, so that a warp runs one class's code on lanes that
+// need about as many nodes.  The order of a key's pairs varies from run to
+// run; a pair's result depends on the pair alone.
+// What bounds it once the lanes are even is instruction fetch: the classes'
+// code is larger than the instruction cache, so the warps of an SM should be
+// in the same class.  Hence large blocks and windows of up to 15872 pairs (what
+// 48 KB of shared memory hold beside the table), equal ones, as few per block
+// as the queue needs: on the whole domain (6.9M queued pairs) 1.69 ms with
+// 128-thread blocks and 1024-pair windows, 1.28 with 256 and 2048, 1.18 with
+// 512 and 4096, 1.13 with 512 and 16384.
+constexpr int kKtThreads = LB_KTRAP_THREADS;
+constexpr int kKtWindow = LB_KTRAP_WINDOW;
+static_assert(kKtWindow <= 65536, "16-bit offsets within a window");
 template <bool DX>
-__global__ void __launch_bounds__(LB_THREADS, ktrap_ctas(DX))
+__global__ void __launch_bounds__(kKtThreads, ktrap_ctas(DX))
 lb_ktrap_kernel(const double* __restrict__ v, int64_t v_stride, const double* __restrict__ x,
                 double* __restrict__ out, const unsigned int* __restrict__ qcount,
                 const uint32_t* __restrict__ queue, int64_t n, int64_t qcap) {
-  constexpr int kPer = kKtWindow / LB_THREADS;
-  __shared__ __align__(16) unsigned long long tab[2048];
-  __shared__ uint32_t list[kKtWindow];
+  extern __shared__ __align__(16) unsigned char kt_shared[];
+  unsigned long long* tab = reinterpret_cast<unsigned long long*>(kt_shared);
+  uint16_t* list = reinterpret_cast<uint16_t*>(kt_shared + 2048 * sizeof(unsigned long long));
   __shared__ int count[64], beg[64], next_chunk;
   unsigned int cnt = *qcount;
   if (!LB_CHECK(cnt <= qcap, 8u)) cnt = (unsigned int)qcap;
   const int tid = threadIdx.x, lane = tid & 31;
-  // equal windows: as many per block as the queue needs, so that no block's last one is short
   const int64_t share = ((int64_t)cnt + gridDim.x - 1) / gridDim.x;
   const int64_t rounds = (share + kKtWindow - 1) / kKtWindow;
   const int W = rounds ? (int)(((share + rounds - 1) / rounds + 31) & ~(int64_t)31) : 32;
   if ((int64_t)blockIdx.x * W >= (int64_t)cnt) return;     // the same for every thread of the block
-  kt_load_table<LB_THREADS>(tab);
+  kt_load_table<kKtThreads>(tab);
   for (int64_t w0 = (int64_t)blockIdx.x * W; w0 < (int64_t)cnt; w0 += (int64_t)gridDim.x * W) {
     const int m = (int)min((int64_t)W, (int64_t)cnt - w0);
     if (tid < 64) count[tid] = 0;
     if (tid == 0) next_chunk = 0;
     __syncthreads();
-    uint32_t ent[kPer];
-    int rank[kPer];
+    // pass 0 counts the keys, pass 1 places the entries; one atomic per key and warp
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int j0 = tid - lane; j0 < m; j0 += kKtThreads) {
+        const int j = j0 + lane;
+        int key = -1;
+        if (j < m) {
+          const uint32_t e = queue[w0 + j];
+          key = (int)(e >> kQueueOffsetBits);
+          if (!LB_CHECK(key < 48, 32u)) key = 0;
+          if (!LB_CHECK((int64_t)(e & kQueueOffsetMask) < n, 16u)) key = -1;
+        }
+        const unsigned peers = __match_any_sync(0xffffffffu, key);
+        const int leader = __ffs(peers) - 1;
+        int pos = 0;
+        if (key >= 0 && lane == leader) pos = atomicAdd(pass ? &beg[key] : &count[key], __popc(peers));
+        pos = __shfl_sync(0xffffffffu, pos, leader) + __popc(peers & ((1u << lane) - 1u));
+        if (pass && key >= 0 && LB_CHECK(pos < kKtWindow, 1u)) list[pos] = (uint16_t)j;
+      }
+      __syncthreads();
+      if (pass == 0) {
+        if (tid < 32) {                            // exclusive prefix over the 64 key slots
+          const int a = count[2 * lane], b = count[2 * lane + 1];
+          int p = a + b;
 #pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-      const int j = tid + q * LB_THREADS;
-      rank[q] = -1;
-      if (j < m) {
-        uint32_t e = queue[w0 + j];
-        if (!LB_CHECK((e >> kQueueOffsetBits) < 48u, 32u)) e &= kQueueOffsetMask;
-        ent[q] = e;
-        if (LB_CHECK((int64_t)(e & kQueueOffsetMask) < n, 16u)) rank[q] = atomicAdd(&count[e >> kQueueOffsetBits], 1);
+          for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, p, o);
+            if (lane >= o) p += u;
+          }
+          beg[2 * lane] = p - a - b;
+          beg[2 * lane + 1] = p - b;
+        }
+        __syncthreads();
       }
     }
-    __syncthreads();
-    if (tid < 32) {                                // exclusive prefix over the 64 key slots
-      const int a = count[2 * lane], b = count[2 * lane + 1];
-      int p = a + b;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, p, o);
-        if (lane >= o) p += u;
-      }
-      beg[2 * lane] = p - a - b;
-      beg[2 * lane + 1] = p - b;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < kPer; ++q)
-      if (rank[q] >= 0) list[beg[ent[q] >> kQueueOffsetBits] + rank[q]] = ent[q] & kQueueOffsetMask;
-    __syncthreads();
+    // beg[k] is now the end of key k's entries
     for (;;) {
       int ch = 0;
       if (lane == 0) ch = atomicAdd(&next_chunk, 1);
@@ -248,8 +267,8 @@ lb_ktrap_kernel(const double* __restrict__ v, int64_t v_stride, const double* __
       int c = 0, b = 0, e = 0;
 #pragma unroll 1
       for (; c < 6; ++c) {
-        b = beg[8 * c];
-        e = beg[8 * c + 8];                        // 8 * 6 = 48: the end of the last class
+        b = c ? beg[8 * c - 1] : 0;
+        e = beg[8 * c + 7];
         const int nc = (e - b + 31) >> 5;
         if (ch < nc) break;
         ch -= nc;
@@ -257,7 +276,7 @@ lb_ktrap_kernel(const double* __restrict__ v, int64_t v_stride, const double* __
       if (c == 6) break;
       const int j = b + (ch << 5) + lane;
       if (j < e) {
-        const int64_t idx = (int64_t)list[j];
+        const int64_t idx = (int64_t)(queue[w0 + list[j]] & kQueueOffsetMask);
         out[idx] = kt_eval<DX>(fabs(v[idx * v_stride]), x[idx], c, tab);
       }
       __syncwarp();
@@ -598,8 +617,9 @@ lb_status run_impl(const T* v, int64_t v_stride, const T* x, T* out, int64_t n, 
         // the queue's length is on the device: a block per 32 pairs it can hold, at most the resident ones
         const int64_t want = (cn + 31) / 32, most = (int64_t)sms * ktrap_ctas(DX);
         const int kgrid = (int)(want < most ? want : most);
+        constexpr int kShared = 2048 * 8 + 2 * kKtWindow;   // with the static arrays below 48 KB: no opt-in
         status = launch(PS_KINT, st, [&] {
-          lb_ktrap_kernel<DX><<<kgrid, LB_THREADS, 0, st>>>(vc, v_stride, xc, oc, qcount, queue, cn, cap);
+          lb_ktrap_kernel<DX><<<kgrid, kKtThreads, kShared, st>>>(vc, v_stride, xc, oc, qcount, queue, cn, cap);
         });
       } else {
         const int kgrid = sms * 2 * LB_KINT_CTAS_PER_SM;
