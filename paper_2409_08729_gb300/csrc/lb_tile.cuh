@@ -535,7 +535,7 @@ __device__ __forceinline__ void warp_pairs64(const double* __restrict__ v, int64
 constexpr int kList32 = 256 + 128;                         // entries before a flush, and one slice's
 struct Warp32 {
   uint32_t raw[kList32], list[kList32];                    // offsets from the base of v, x and out
-  uint8_t rkey[kList32], lkey[kList32];
+  uint8_t rkey[kList32];
   int count[16];
 };
 
@@ -556,6 +556,15 @@ template <int KIND>
 __device__ __forceinline__ int flush32(Warp32& W, int cnt, bool last, const float* __restrict__ v, int64_t v_stride,
                                        const float* __restrict__ x, float* __restrict__ out) {
   const int lane = threadIdx.x & 31;
+  if (lane < 16) W.count[lane] = 0;
+  __syncwarp();
+  for (int j = lane; j < cnt; j += 32) {
+    const int64_t i = W.raw[j];
+    const float vi = v[i * v_stride];
+    const int k = key32<KIND>(KIND == KIND_K ? fabsf(vi) : vi, x[i]);
+    W.rkey[j] = (uint8_t)k;
+    atomicAdd(&W.count[k], 1);
+  }
   __syncwarp();
   const int c = lane < 16 ? W.count[lane] : 0;
   int p = c;
@@ -568,10 +577,7 @@ __device__ __forceinline__ int flush32(Warp32& W, int cnt, bool last, const floa
   __syncwarp();
   for (int j = lane; j < cnt; j += 32) {
     const int k = W.rkey[j], pos = atomicAdd(&W.count[k], 1);
-    if (LB_CHECK(pos < kList32, 1u)) {
-      W.list[pos] = W.raw[j];
-      W.lkey[pos] = (uint8_t)k;
-    }
+    if (LB_CHECK(pos < kList32, 1u)) W.list[pos] = W.raw[j];
   }
   __syncwarp();
   const int m = last ? cnt : cnt & ~31;
@@ -581,14 +587,7 @@ __device__ __forceinline__ int flush32(Warp32& W, int cnt, bool last, const floa
     out[i] = KIND == KIND_I ? series_all32(vi, xi) : kt_log_k32(fabsf(vi), xi);
   }
   __syncwarp();
-  if (lane < 16) W.count[lane] = 0;
-  __syncwarp();
-  if (lane < cnt - m) {
-    const int k = W.lkey[m + lane];
-    W.raw[lane] = W.list[m + lane];
-    W.rkey[lane] = (uint8_t)k;
-    atomicAdd(&W.count[k], 1);
-  }
+  if (lane < cnt - m) W.raw[lane] = W.list[m + lane];
   __syncwarp();
   return cnt - m;
 }
@@ -602,9 +601,8 @@ __device__ __forceinline__ void warp_pairs32(Warp32& W, const float* __restrict_
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const float v0 = v_stride ? 0.0f : v[0];
+  const bool in_place = out == x;
   int cnt = 0;                                             // entries in the list (warp-uniform)
-  if (lane < 16) W.count[lane] = 0;
-  __syncwarp();
   for (int64_t s = begin + warp * (32 * VEC); s < end; s += nwarps * (32 * VEC)) {
     const int64_t i = s + lane * VEC;
     float vv[VEC], xx[VEC], rr[VEC];
@@ -647,7 +645,9 @@ __device__ __forceinline__ void warp_pairs32(Warp32& W, const float* __restrict_
         rr[e] = u_all32(KIND, vi, xi, s2);
       }
     }
-    if (whole && fb == 0) {
+    // a listed pair's result is written after this by the same warp; its slot
+    // may hold anything until then, except its argument when out is x
+    if (whole && (fb == 0 || !in_place)) {
       if (VEC == 4) *reinterpret_cast<float4*>(out + i) = make_float4(rr[0], rr[1 % VEC], rr[2 % VEC], rr[3 % VEC]);
     } else {
 #pragma unroll
@@ -658,14 +658,8 @@ __device__ __forceinline__ void warp_pairs32(Warp32& W, const float* __restrict_
     for (int e = 0; e < VEC; ++e) {
       const bool f = ((fb >> e) & 1u) && i + e < end;
       const unsigned m = __ballot_sync(0xffffffffu, f);
-      if (f) {
-        const int b = cnt + __popc(m & lt), k = key32<KIND>(KIND == KIND_K ? fabsf(vv[e]) : vv[e], xx[e]);
-        if (LB_CHECK(b < kList32, 1u)) {
-          W.raw[b] = (uint32_t)(i + e);
-          W.rkey[b] = (uint8_t)k;
-          atomicAdd(&W.count[k], 1);
-        }
-      }
+      const int b = cnt + __popc(m & lt);
+      if (f && LB_CHECK(b < kList32, 1u)) W.raw[b] = (uint32_t)(i + e);
       cnt += __popc(m);
     }
     if (cnt >= 256) cnt = flush32<KIND>(W, cnt, false, v, v_stride, x, out);
