@@ -53,15 +53,36 @@ LB_IX_FN bool uni_ok(double s, double x) {
   return hs >= 0x40701000u && hs < 0x7e37e43cu && hx >= 0x00100000u;
 }
 
+// The sums' variables from v/r <= 1 and 1/r: g = p/2, y = p^2/2, h = 8/r
+// (below 1/2), all in Q64.  The outer sums run over +-h and are kept with
+// kUniBias added, so that they stay positive and take the short unsigned
+// product; hb is the bias's product with h.
+struct UniVars {
+  uint64_t g, y, h, hb;
+};
+constexpr uint64_t kUniBias = 1ull << 57;
+LB_IX_FN UniVars uni_vars(double vr, double q) {
+  UniVars u;
+  const uint64_t t = (uint64_t)ix_fix(vr, 62);
+  u.g = kt_mulhi(t, t) << 3;
+  u.y = kt_mulhi(u.g >> 1, u.g >> 1) << 3;
+  u.h = (uint64_t)ix_fix(q, 67);
+  u.hb = u.h >> 7;                                          // 2^57 h / 2^64
+  return u;
+}
+// kUniBias +- h (acc - kUniBias), c0 = kUniBias -+ hb.
+LB_IX_FN uint64_t uni_step(int kind, uint64_t acc, uint64_t h, uint64_t c0) {
+  const uint64_t m = kt_mulhi(acc, h);
+  return kind ? c0 - m : c0 + m;
+}
+
 // log I (kind 0) or log K of one pair with s = v^2 + x^2, uni_ok; K: the
 // pair's terms, Kmax: the warp's largest.
 LB_IX_FN double u_fx(int kind, double v, double x, double s, int K, int Kmax) {
   const double q = kt_rsqrt(s), r = s * q;                  // 1/r, r
-  const uint64_t t = (uint64_t)ix_fix(v * q, 63);           // v/r <= 1
-  const uint64_t g = ix_umulhi(t, t) << 1;                  // p/2 in Q64
-  const uint64_t y = ix_umulhi(g, g) << 1;                  // p^2/2 in Q64
-  const int64_t h = kind ? -ix_fix(q, 67) : ix_fix(q, 67);  // +-8/r in Q64, below 1/2
-  int64_t acc = 0;
+  const UniVars u = uni_vars(v * q, q);
+  const uint64_t c0 = kind ? kUniBias + u.hb : kUniBias - u.hb;
+  uint64_t acc = kUniBias;
 #pragma unroll 1
   for (int k = Kmax; k >= 1; --k) {
     const int b = lb_uni_off[k];
@@ -69,17 +90,17 @@ LB_IX_FN double u_fx(int kind, double v, double x, double s, int K, int Kmax) {
     uint64_t e = lb_uni[i][0], o = lb_uni[i][1];
 #pragma unroll 1
     for (--i; i >= b; --i) {
-      e = lb_uni[i][0] + kt_mulhi(e, y);
-      o = lb_uni[i][1] + kt_mulhi(o, y);
+      e = lb_uni[i][0] + kt_mulhi(e, u.y);
+      o = lb_uni[i][1] + kt_mulhi(o, u.y);
     }
-    acc = ix_mulhi(acc, h) + (int64_t)(e - kt_mulhi(o, g));
-    if (k > K) acc = 0;
+    acc = uni_step(kind, acc, u.h, c0) + e - kt_mulhi(o, u.g);
+    if (k > K) acc = kUniBias;
   }
-  const uint64_t S = (uint64_t)((1ll << 56) + ix_mulhi(acc, h));      // Q56
-  // S^2 / r: Q63 x Q63, then the 53 bits of 1/r
+  const uint64_t S = uni_step(kind, acc, u.h, c0) + (1ull << 56) - kUniBias;   // Q56
+  // S^2 / r: Q62 x Q62, then the 53 bits of 1/r
   const uint64_t bq = ix_bits(q);
-  const uint64_t W = ix_umulhi(ix_umulhi(S << 7, S << 7), ((bq & 0x000fffffffffffffull) | 0x0010000000000000ull) << 11);   // Q61
-  const long long lw = kt_logq(ix_pack(W, 1022 - (int)(bq >> 52)));
+  const uint64_t W = kt_mulhi(kt_mulhi(S << 6, S << 6) << 2, ((bq & 0x000fffffffffffffull) | 0x0010000000000000ull) << 10);   // Q60
+  const long long lw = kt_logq(ix_pack(W, 1021 - (int)(bq >> 52)));
   const double a = (double)(kt_logq(x) - kt_logq(v + r)), w = v * 0x1p-53;
   if (kind == 0) return fma(w, a, fma(0x1p-54, (double)(lw - kHalfLog2PiQ53x2), r));
   return -fma(w, a, fma(-0x1p-54, (double)(lw + kLogHalfPiQ53), r));
@@ -96,11 +117,9 @@ LB_IX_FN int uni_terms_dx(float f, int cap) { return uni_terms(f * 0.58f, cap); 
 // the result: its 2^-50 and S's 2^-56 are far below the result's last place.
 LB_IX_FN double u_dx_fx(int kind, double v, double x, double s, int K, int Kmax) {
   const double q = kt_rsqrt(s), r = s * q;
-  const uint64_t t = (uint64_t)ix_fix(v * q, 63);
-  const uint64_t g = ix_umulhi(t, t) << 1;
-  const uint64_t y = ix_umulhi(g, g) << 1;
-  const int64_t h = kind ? -ix_fix(q, 67) : ix_fix(q, 67);
-  int64_t acc = 0, dcc = 0;
+  const UniVars u = uni_vars(v * q, q);
+  const uint64_t c0 = kind ? kUniBias + u.hb : kUniBias - u.hb;
+  uint64_t acc = kUniBias, dcc = kUniBias;
 #pragma unroll 1
   for (int k = Kmax; k >= 1; --k) {
     const int b = lb_uni_off[k];
@@ -108,17 +127,17 @@ LB_IX_FN double u_dx_fx(int kind, double v, double x, double s, int K, int Kmax)
     uint64_t e = lb_uni[i][0], o = lb_uni[i][1], de = lb_uniq[i][0], dd = lb_uniq[i][1];
 #pragma unroll 1
     for (--i; i >= b; --i) {
-      e = lb_uni[i][0] + kt_mulhi(e, y);
-      o = lb_uni[i][1] + kt_mulhi(o, y);
-      de = lb_uniq[i][0] + kt_mulhi(de, y);
-      dd = lb_uniq[i][1] + kt_mulhi(dd, y);
+      e = lb_uni[i][0] + kt_mulhi(e, u.y);
+      o = lb_uni[i][1] + kt_mulhi(o, u.y);
+      de = lb_uniq[i][0] + kt_mulhi(de, u.y);
+      dd = lb_uniq[i][1] + kt_mulhi(dd, u.y);
     }
-    acc = ix_mulhi(acc, h) + (int64_t)(e - kt_mulhi(o, g));
-    dcc = ix_mulhi(dcc, h) + (int64_t)(de - kt_mulhi(dd, g));
-    if (k > K) acc = dcc = 0;
+    acc = uni_step(kind, acc, u.h, c0) + e - kt_mulhi(o, u.g);
+    dcc = uni_step(kind, dcc, u.h, c0) + de - kt_mulhi(dd, u.g);
+    if (k > K) acc = dcc = kUniBias;
   }
-  const double S = (double)((1ll << 56) + ix_mulhi(acc, h));          // Q56
-  const double SQ = (double)ix_mulhi(dcc, h) * 64.0;                  // Q50 to Q56
+  const double S = (double)(int64_t)(uni_step(kind, acc, u.h, c0) + (1ull << 56) - kUniBias);   // Q56
+  const double SQ = (double)(int64_t)(uni_step(kind, dcc, u.h, c0) - kUniBias) * 64.0;           // Q50 to Q56
   const double corr = (x * q) * q * fma(SQ, kt_rcp(S), 0.5);
   const double lead = r * kt_rcp(x);
   return kind ? -lead - corr : lead - corr;
