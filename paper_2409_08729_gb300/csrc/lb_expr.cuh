@@ -343,25 +343,6 @@ __device__ __forceinline__ dfloat debye_Q_df(int k, dfloat p) {
   return r;
 }
 
-template <typename T>
-__device__ __forceinline__ T debye_Q(int k, T p) {
-  switch (k) {
-    case 1: return lb_debye_Q1(p);
-    case 2: return lb_debye_Q2(p);
-    case 3: return lb_debye_Q3(p);
-    case 4: return lb_debye_Q4(p);
-    case 5: return lb_debye_Q5(p);
-    case 6: return lb_debye_Q6(p);
-    case 7: return lb_debye_Q7(p);
-    case 8: return lb_debye_Q8(p);
-    case 9: return lb_debye_Q9(p);
-    case 10: return lb_debye_Q10(p);
-    case 11: return lb_debye_Q11(p);
-    case 12: return lb_debye_Q12(p);
-    default: return lb_debye_Q13(p);
-  }
-}
-
 // ---------------------------------------------------------------------------
 // U_K expression (paper Eqs. "log Iv u k", "log Kv u k"):
 //   x' = x/v, r = sqrt(1 + x'^2), t = 1/r, eta = r + log(x' / (1 + r)),
@@ -510,33 +491,47 @@ struct ScalarOrder {
   dfloat serd[91];                      // ser[] in double-float
 };
 
-// All threads of the block call it; ends with a barrier.
+// All threads of the block (at least 64) call it; ends with a barrier.  The
+// chains are kept short, as every block runs this before its first tile: the
+// 20 ratios of mu_K on 20 lanes and their products by a warp scan, lgamma on
+// another warp, the series' reciprocals on the rest.
 template <int KIND, int NT>
 __device__ __forceinline__ void scalar_order_setup(ScalarOrder& so, double v) {
   const int tid = threadIdx.x;
-  if (tid == 0) {
-    so.v = v;
-    so.lg1 = lgamma(v + 1.0);
-    // the smallest x at which a dispatch takes mu_20 for this order (tight:
-    // 18.5, or v^2 < 3.24 x; paper: 0.5113 log x + 0.7939 > log v)
-    const double xmin = v < 15.4 ? 18.4 : fmax(59.0, 0.98 * fmin(v * v / 3.24, pow(v / 2.212, 1.9558)));
-    const int j = ilogb(4.0 * xmin);                // 2^j / (8 x) <= 1/2
-    const double mu = 4.0 * v * v, s = KIND == KIND_I ? -1.0 : 1.0;
-    double c[21], a = 1.0, big = 1.0;
-    c[0] = 1.0;
-    for (int k = 1; k <= 20; ++k) {
-      a = ldexp(a * (s * (mu - (double)((2 * k - 1) * (2 * k - 1)))) / (double)k, -j);
-      c[k] = a;
-      big = fmax(big, fabs(a));
+  if (tid < 32) {
+    // 2^j = the power of two at most 4 xmin, xmin the smallest x at which a
+    // dispatch takes mu_20 for this order (tight: 18.5, or v^2 < 3.24 x;
+    // paper: 0.5113 log x + 0.7939 > log v): then 2^j / (8 x) <= 1/2
+    int j = 6;                                      // 4 x 18.4
+    if (!(v < 15.4)) {
+      const int e = ilogb(v);
+      const float lv = (float)e + log2f((float)scalbn(v, -e));
+      const float l = fminf(2.0f * lv - 1.6961f, 1.9558f * (lv - 1.1454f));   // log2 of v^2/3.24, (v/2.212)^1.9558
+      j = (int)floorf(2.0f + fmaxf(5.88f, l - 0.05f - 2e-6f * fabsf(l)));      // log2 59 at least
     }
-    // |c_k| 2^(59 - muq) < 2^60: with W <= 1/2 every Horner sum stays within +-2^61
-    const int muq = big < 1e15 ? ilogb(big) : 50;
-    for (int k = 0; k <= 20; ++k) so.mu[k] = ix_fix(c[k], 59 - muq) + (1ll << 62);
-    so.muj = j;
-    so.muc = (KIND == KIND_I ? kMuSoLogI : kMuSoLogK) - 2 * (59 - muq) * kLn2Q53;
+    const int k = tid < 1 ? 1 : (tid > 20 ? 20 : tid);
+    const double mu = 4.0 * v * v, s = KIND == KIND_I ? -1.0 : 1.0;
+    double a = ldexp(s * (mu - (double)((2 * k - 1) * (2 * k - 1))) / (double)k, -j);
+    if (tid == 0 || tid > 20) a = tid == 0 ? 1.0 : 0.0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {              // a_0 .. a_tid
+      const double u = __shfl_up_sync(0xffffffffu, a, o);
+      if (tid >= o) a *= u;
+    }
+    // |a_k| 2^(59 - muq) < 2^60: with W <= 1/2 every Horner sum stays within +-2^61
+    int muq = tid <= 20 && a != 0.0 ? max(ilogb(fabs(a)), 0) : 0;
+    muq = min(__reduce_max_sync(0xffffffffu, muq), 50);
+    if (tid <= 20) so.mu[tid] = ix_fix(a, 59 - muq) + (1ll << 62);
+    if (tid == 0) {
+      so.v = v;
+      so.muj = j;
+      so.muc = (KIND == KIND_I ? kMuSoLogI : kMuSoLogK) - 2 * (59 - muq) * kLn2Q53;
+    }
+  } else if (tid < 64) {
+    if (tid == 32) so.lg1 = lgamma(v + 1.0);
   }
-  if (tid >= 32)
-    for (int k = tid - 31; k <= 90; k += NT - 32) {
+  if (NT > 64 ? tid >= 64 : tid >= 32)
+    for (int k = tid - (NT > 64 ? 63 : 31); k <= 90; k += NT - (NT > 64 ? 64 : 32)) {
       so.ser[k] = 1.0 / ((double)k * ((double)k + v));
       so.serd[k] = df_from_double(so.ser[k]);
     }

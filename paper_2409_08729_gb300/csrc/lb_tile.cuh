@@ -81,7 +81,6 @@ __host__ __device__ constexpr int region_terms(int r) { return r == R_U4 ? 4 : r
 // One tile of NT * IT pairs in the shared memory of a block of NT threads.
 template <typename T, int NT, int IT>
 struct TileShared {
-  static constexpr int kThreads = NT;
   static constexpr int kTile = NT * IT;
   T sv[kTile];
   union {                                          // a pair's result replaces its argument

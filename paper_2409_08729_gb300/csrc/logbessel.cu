@@ -545,7 +545,10 @@ lb_status run_tiles(int sms, cudaStream_t st, const T* v, int64_t v_stride, T v0
                     int mode, int forced_region, unsigned int* qcount, uint32_t* queue, int64_t cap, int64_t total_n,
                     double vmf_d) {
   if constexpr (sizeof(T) == 8) {
-    const bool so = !DX && v_stride == 0 && forced_region < 0;
+    // (an order known here to be past 16 -- the vMF form's d/2 - 1 usually is --
+    // takes the general kernel: mostly U_K then, which the one-order kernel has
+    // no faster form of.  log C_2048, 1M values: 97 -> 72 us)
+    const bool so = !DX && v_stride == 0 && forced_region < 0 && (v || (double)v0 <= 16.0);
     if (total_n < kMid && forced_region < 0) {
       if (so && total_n >= kMidInTile)
         return launch_tiles<KIND, DX, T, !DX, LB_MID_THREADS, LB_MID_ITEMS, false>(sms, st, v, v_stride, v0, x, out, n, mode,

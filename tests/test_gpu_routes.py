@@ -49,3 +49,18 @@ def test_vmf_routes(cuda, n):
     assert abs(e[0] - lim) <= TOL * abs(lim) and np.isnan(e[1]) and np.isnan(e[2])
     e = vmf.log_c(d, torch.tensor([0.0, float("inf")], dtype=torch.float64, device=cuda), deriv=True).cpu().numpy()
     assert e[0] == 0.0 and e[1] == -1.0
+
+
+@pytest.mark.parametrize("d", [2, 3, 33, 34, 35, 300])
+def test_vmf_order_in_either_kernel(cuda, d):
+    """Orders d/2 - 1 up to 16 take the one-order kernel, larger ones the
+    general kernel: log C_d of both against the oracle, over each expansion."""
+    x = np.concatenate([np.geomspace(1e-3, 2e3, 2400), [18.49, 18.5, 18.51, 58.9, 59.0]])
+    nu = 0.5 * d - 1.0
+    li = oracle.log_i(np.full(x.size, nu), x)
+    want = nu * np.log(x) - 0.5 * d * np.log(2 * np.pi) - li
+    got = vmf.log_c(d, torch.tensor(x, device=cuda)).cpu().numpy()
+    # each of the three terms correct to TOL of its size, and the roundings of the sum
+    scale = np.abs(nu * np.log(x)) + 0.5 * d * np.log(2 * np.pi) + np.maximum(
+        np.abs(li), oracle.error_scale("i", np.full(x.size, nu), x))
+    assert np.max(np.abs(got - want) / scale) <= TOL
