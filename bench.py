@@ -29,29 +29,25 @@ import numpy as np  # noqa: E402
 METRIC = "Gevals/s (log I_v and log K_v, FP64)"
 
 # DRAM bytes (read + write) per benchmark step of each kernel, from one ncu
-# capture of every launch of one full-size step (the launch list of
-# profiles/launches_paper_sweep_fp64.md, with dram__bytes_read.sum and
-# dram__bytes_write.sum); empty when the kernels changed since.
-NCU_DRAM_BYTES_PER_STEP = {"lb_tiles_kernel": (17.417e9, 27), "lb_kint_kernel": (9.431e9, 90)}
-# Pipe utilisation of each kernel from ncu --set full on a small case of the
-# same workload (profiles/lb_tiles_kernel_sweep_small.md,
-# profiles/lb_kint_kernel_sweep_small.md, profiles/fp32_mixed_sweep_small.md):
-# share of peak issue of the FP64 pipe, the ALU pipe, the FP32 (FMA) pipe and
+# capture of every launch of one full-size step; empty when the kernels
+# changed since.
+NCU_DRAM_BYTES_PER_STEP = {}
+# Pipe utilisation of each kernel from ncu on 6M pairs of the same workload
+# (profiles/kernels_6m_pairs.md): share of peak issue of the FP64 pipe, the
+# ALU pipe, the FMA-heavy pipe (integer multiplies), the FP32 (FMA) pipe and
 # the XU (special-function) pipe while active, and the share of cycles that
 # issue; empty when stale.
 NCU_PIPES = {
-    "lb_tiles_kernel": {"fp64": 0.618, "alu": 0.460, "fma": 0.300, "xu": 0.025, "issue_active": 0.675,
-                        "launch": "log I, mixed orders, 11M pairs"},
-    "lb_kint_kernel": {"fp64": 0.355, "alu": 0.635, "fma": 0.193, "xu": 0.015, "issue_active": 0.662,
-                       "launch": "one-slot class kernel of a mixed-order log K call (class 4: fp64 0.257, "
-                                 "alu 0.611, issue 0.634); FMA-heavy pipe (integer multiplies) 0.48; captured "
-                                 "before the one-slot rule for orders 0.9-2 was added"},
+    "lb_tiles_kernel": {"fp64": 0.477, "alu": 0.472, "fma_heavy": 0.429, "fma": 0.252, "xu": 0.019,
+                        "issue_active": 0.661, "launch": "log K, mixed orders, 6M pairs"},
+    "lb_kint_kernel": {"fp64": 0.105, "alu": 0.478, "fma_heavy": 0.420, "fma": 0.210, "xu": 0.011,
+                       "issue_active": 0.539, "launch": "lb_ktrap_kernel after the same call's tiles (one pair in "
+                                                        "seven; all classes of the whole domain: alu 0.56, "
+                                                        "issue 0.60)"},
 }
 NCU_PIPES_FP32 = {
-    "lb_tiles_kernel": {"fp64": 0.0, "alu": 0.450, "fma": 0.235, "xu": 0.111, "issue_active": 0.760,
-                        "launch": "log I, mixed orders, 11M pairs"},
-    "lb_kint_kernel": {"fp64": 0.0, "alu": 0.518, "fma": 0.312, "xu": 0.054, "issue_active": 0.798,
-                       "launch": "log K integral, mixed orders"},
+    "lb_tiles_kernel": {"fp64": 0.0, "alu": 0.514, "fma_heavy": 0.228, "fma": 0.350, "xu": 0.118,
+                        "issue_active": 0.747, "launch": "lb_tiles32_kernel, log I, mixed orders, 6M pairs"},
 }
 UNIT = "Gevals/s"
 WORKLOAD = "paper-shaped sweep: v=2^0..2^10 x 20M x~U[1,100] per order, log I + log K, per-order + mixed-order calls"
@@ -518,9 +514,10 @@ def main():
             "algorithmic_bytes": kd["algorithmic_bytes_per_launch"], "launches": kd["launches"],
             "avg_launch_ms": kd["avg_launch_ms"],
             "work": "FP64 operations of the method (benchmarks/optable.py) at per-pair term and node counts; "
-                    "library calls (log, exp, rcp, rsqrt, lgamma) not priced; the high-order terms of the "
-                    "mu_20 and U_K sums execute as double-float FP32 instructions, so the rate counts the "
-                    "method's operations, not the FP64 instructions issued",
+                    "library calls (log, exp, rcp, rsqrt, lgamma) not priced; the U_K and one-order mu_20 sums "
+                    "and the K integral run in 64-bit fixed point on the integer pipes, the other sums' "
+                    "high-order terms in double-float: the rate counts the method's operations, not the FP64 "
+                    "instructions issued, and may pass the FP64 pipe's peak",
             "peak_source": "152 SMs x 2 FP64 op/clk x 2.07 GHz; live DFMA microbenchmark %.1f G/s"
                            % (rates["dfma"] / 1e9),
             "ncu": kd["ncu"]}

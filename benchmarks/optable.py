@@ -14,34 +14,34 @@ pipe's capacity that did the method's own arithmetic.
 Per pair, in tight mode, with n the pair's own term count (not the warp's):
 
   region          general pair                  one order for the whole call
-  mu_K (n terms)  3n + 7     rcp, log           n + 6     rcp, log
-  U_K             K(K+1)/2 + K + 14             3K + 12
-                  rcp, rsqrt, 3 log             rsqrt, 3 log
+  mu_K (n terms)  2n + 8     rcp, log           n + 6     rcp, log
+  U_K             K(K+1)/2 + K + 14             the same
+                  rsqrt, 3 log
   series (n)      4n + 7     rcp, 2 log, lgamma 2n + 5    2 log
-  K integral      8 per g node, 6 per h node,   7 per g node, 6 per h node,
-                  11 per pair                   10 per pair
-                  exp: 2 per g node + 1 per h node (1 + 1 for one order),
-                  log: 1 per node + 3 per pair, rcp, lgamma (per pair)
+  K integral      7 per node, 14 per pair       the same
+                  exp: 1 per node, rsqrt, 2 rcp, 2 log per pair
+  (x < 2^-9)      64 per pair + 2 per step of the recurrence
+                  log, exp, 6 rcp, log
 
-mu_K: per term a_k = (mu - (2k-1)^2)/k (one fma with constants), times
-+-1/(8x), Horner step (fma); per pair mu = 4v^2, 8x, S^2 and two scalings,
-the final fma.  With one order the coefficients a_k (s/8)^k are the call's:
-one fma per term.
-U_K: x' = x/v, 1 + x'^2, r = r^2 t, t^2, +-t/v, the Debye polynomial P_k of
-degree k in t^2 by Horner (k fmas, k = 1..K), Horner over k in q (K fmas),
-eta (3), w = S^2 t / v (3), scaling, halving, final fma.  With one order the
-sum is one polynomial of degree 3K in t (3K fmas).
+mu_K: per term D_k = mu w - (2k-1)^2 w (fma) and Q <- D_k Q + const (fma);
+per pair mu w (3), 8x, S^2 w (2), scaling, the final fma.  With one order the
+sum is a polynomial in w: one fma per term.
+U_K: v^2 + x^2, r = (v^2 + x^2) / sqrt, v/r, its square, v + r, the Debye
+polynomial P_k of degree k by Horner (k fmas, k = 1..K), Horner over k in 1/r
+(K fmas), S^2/r (2), the difference of the logarithms, final fmas.  K is the
+pair's own: its region's, or less at large r.
 Series (the linear fraction of the reading of Eq. "log Iv" with a_0 as
 shift): per term d_k = k(k+v) (fma), A <- d B + y A (mul, fma), B <- d B;
 per pair y = x^2/4, A/B, v+1, x/2, two combining operations.  With one
 order the ratios 1/(k(k+v)) are the call's: per term y r_k and one fma.
-K integral (Eq. "log Kv integral", Gauss nodes): a g node forms s = u^beta
-(beta log u, exp), 2x + s, log, c + log beta, fma, - s; an h node s + 2x,
-log, y + ., fma; every node then takes part in the log-sum-exp of Eq. "log
-sum trick" (compare for the maximum, L - m, exp, add).  Per pair: v - 1/2,
-2x, beta (2v + 1 and a scaling, a reciprocal), v + 1/2 for lgamma, the
-prefactor (fma and two subtractions), the final logarithm and two additions.
-With one order u^beta and lgamma(v + 1/2) are the call's.
+K integral (trapezoid rule about the maximum): a node forms a e^(kh) and
+b e^(-kh) (two multiplications by constants), their sum, the linear term,
+their difference from the maximum, the exponential, and its addition to the
+sum; per pair v^2 + x^2 (2), r, r + v, x^2/(r + v) (2), v h, x^2, (r + v)/x,
+the two logarithms' combination (5).  Below x = 2^-9 Temme's series: 64
+operations and two per step from order mu to v.
+FP32-mixed form (FP32 operations): one expansion of five terms for
+r >= 14 (45), the series 5n + 30, the integral 5 per node + 14.
 """
 import numpy as np
 
@@ -94,26 +94,41 @@ def series_terms(v, x, eps=1.4e-17):
     return n
 
 
-def kint_nodes(v, x, one_slot=True, low_slot=True):
-    """g and h nodes of the tight K-integral rule of each pair (values; |v|
-    given).  The split g rule (v < 0.4, x < 1e-3) has 64 + 32 + 32 nodes,
-    plus 32 more below x ~ 4e-21; 1.2 < v <= 5 takes 24 g + 40 h nodes;
-    2 <= v <= 16.5 the one-slot rules, 22 + 10 (v < 7) or 12 + 20, and
-    0.9 <= v < 2 with x >= 0.8 the one-slot rule of 24 + 8 nodes (FP64 only:
-    low_slot False for the FP32 form)."""
+def uni_terms(v, x, cap):
+    """Terms of the uniform expansion (FP64 values): the region's cap, or the
+    smallest K with max|P_(K+1)| / r^(K+1) <= 3e-17 r, by half octaves."""
+    s = (np.asarray(v, dtype=np.float32) ** 2 + np.asarray(x, dtype=np.float32) ** 2).astype(np.float32)
+    i = (s.view(np.uint32) >> 22).astype(np.int64) - (2 * (127 + 9) + 1)
+    tab = np.array([13, 12, 11, 10, 9, 8, 8, 7, 7, 6, 6, 6, 5, 5, 5, 5, 4])
+    return np.minimum(np.where(i < 0, 13, tab[np.clip(i, 0, 16)]), cap)
+
+
+def kint_nodes(v, x, fp32=False):
+    """Nodes of the tight K-integral rule of each pair (|v| given): both sides
+    of the maximum in groups of m (h = ln2/m) to the first group whose last
+    term is below 2^-54 (FP32: node by node to 2^-26), and the maximum; 0 for
+    x < 2^-9 (Temme's series)."""
     v = np.asarray(v, dtype=np.float64)
     x = np.asarray(x, dtype=np.float64)
-    split = np.where(np.log(128 * np.maximum(x, 1e-320)) + 40 < -4, 160, 128)
-    ng = np.where((v >= 0.9) | (x >= 0.25), 32, np.where((v >= 0.4) | (x >= 1e-3), 64, split))
-    nh = np.where(v <= 1.2, 32, np.where(v <= 5.0, 48, 32))
-    packed = (v > 1.2) & (v <= 5.0)
-    ng, nh = np.where(packed, 24, ng), np.where(packed, 40, nh)
-    one = (v >= 2.0) & (v <= 16.5) & one_slot
-    ng = np.where(one, np.where(v < 7.0, 22, 12), ng)
-    nh = np.where(one, np.where(v < 7.0, 10, 20), nh)
-    low = (v >= 0.9) & (v < 2.0) & (x >= 0.8) & one_slot & low_slot
-    ng, nh = np.where(low, 24, ng), np.where(low, 8, nh)
-    return ng, nh
+    if fp32:
+        m = np.where(x <= 6.8 - 1.8 * v, 2, np.where(x <= 19.5 - 0.115 * v * v, 3, 4))
+    else:
+        m = np.where(x <= 4.5 - 1.5 * v * v, 3, np.where(x <= 17.8 - 0.28 * v * v, 4,
+                                                        np.where(x <= 31 - 0.09 * v * v, 5, 6)))
+    r = np.hypot(v, x)
+    a = (r + v) / 2 / np.log(2)
+    b = x * x / (2 * (r + v)) / np.log(2)
+    cut, step = (26, 1.0 / m) if fp32 else (54, 1.0)
+    total = np.ones(v.shape, dtype=np.int64)
+    for p, q, sgn in ((a, b, 1.0), (b, a, -1.0)):
+        live = x >= 2.0 ** -9
+        for k in range(1, 400):
+            if not live.any():
+                break
+            total += np.where(live, 1 if fp32 else m, 0)
+            d = np.minimum(k * step, 500.0)
+            live = live & (p * 2.0 ** d + q * 2.0 ** -d - (a + b) - sgn * v * d <= cut)
+    return np.where(x >= 2.0 ** -9, total, 0)
 
 
 def region_ops(region, v, x, shared=False, fp32=False):
@@ -122,21 +137,22 @@ def region_ops(region, v, x, shared=False, fp32=False):
     calls pass no order constants, so shared does not apply)."""
     shape = np.shape(x)
     shared = shared and not fp32
+    if fp32:
+        return 5 * series_terms(v, x, eps=1.5e-8) + 30 if region == 2 else np.full(shape, 45, dtype=np.int64)
     if region in (0, 4):
-        n = mu_terms(v, x, REGION_K[region], eps=6e-8 if fp32 else 1.4e-17)
-        return (n + 6) if (shared and region == 0) else (3 * n + 7)
+        n = mu_terms(v, x, REGION_K[region])
+        return (n + 6) if (shared and region == 0) else (2 * n + 8)
     if region in REGION_K:
-        K = REGION_K[region]
-        return np.full(shape, 3 * K + 12 if shared else K * (K + 1) // 2 + K + 14, dtype=np.int64)
-    n = series_terms(v, x, eps=1.5e-8 if fp32 else 1.4e-17)
+        K = uni_terms(v, x, REGION_K[region])
+        return K * (K + 1) // 2 + K + 14
+    n = series_terms(v, x)
     return (2 * n + 5) if shared else (4 * n + 7)
 
 
 def kint_ops(v, x, shared=False, fp32=False):
-    """Operations per pair of the K integral (Gauss rules; the FP32 form takes
-    the same rules, in single precision)."""
-    ng, nh = kint_nodes(v, x, low_slot=not fp32)
-    return ng * (7 if shared else 8) + nh * 6 + (10 if shared else 11)
+    """Operations per pair of the K integral."""
+    n = kint_nodes(v, x, fp32)
+    return np.where(n > 0, (5 if fp32 else 7) * n + 14, 64 + 2 * np.floor(np.asarray(v) + 0.5).astype(np.int64))
 
 
 def region_calls(region, shared=False):
@@ -144,12 +160,5 @@ def region_calls(region, shared=False):
     if region in (0, 4):
         return {"rcp": 1, "log": 1}
     if region in REGION_K:
-        return {"rsqrt": 1, "log": 3} if shared else {"rcp": 1, "rsqrt": 1, "log": 3}
+        return {"rsqrt": 1, "log": 3}
     return {"log": 2} if shared else {"rcp": 1, "log": 2, "lgamma": 1}
-
-
-def kint_calls(ng, nh, shared=False):
-    calls = {"exp": (1 if shared else 2) * ng + nh, "log": ng + nh + 3}
-    if not shared:
-        calls.update(rcp=1, lgamma=1)
-    return calls
