@@ -53,8 +53,9 @@ typedef enum {
 typedef enum {
   /* Default.  The paper's GPU expressions (mu_20, U_13, power series or
    * integral) with region thresholds moved so that the truncation error of
-   * each expression stays below 3e-16 of the error scale, and Gauss
-   * quadrature in place of Simpson's rule for the K integral. */
+   * each expression stays below 3e-16 of the error scale, and the
+   * trapezoid rule on int exp(-x cosh t) cosh(vt) dt in place of Simpson's
+   * rule on the paper's integral for K. */
   LB_TIGHT = 0,
   /* The paper's GPU algorithm as printed: Algorithm 1 without the mu_3, U_4,
    * U_6, U_9 branches (Sec. 4.3), Table "input ranges" thresholds, composite
@@ -99,10 +100,10 @@ lb_status logbessel_k(lb_dtype dtype, const void* v, int64_t v_stride, const voi
 /*
  * Caller-supplied workspace.  The K entry points queue the pairs that take
  * the integral (the fallback region) in device scratch: 256 bytes for a
- * counter and the mask of the quadrature rules queued, plus 4 bytes per pair
- * of a pass.  logbessel_k and logbessel_k_dx
- * take it from the stream-ordered allocator; these variants take it from the
- * caller and allocate nothing.
+ * counter, plus 4 bytes per pair of a pass.  (LB_TIGHT calls in FP32 or of
+ * fewer than 2^17 pairs evaluate the integral in place and use no scratch.)
+ * logbessel_k and logbessel_k_dx take it from the stream-ordered allocator;
+ * these variants take it from the caller and allocate nothing.
  *
  * logbessel_workspace_bytes(n): the bytes that evaluate n pairs in one pass,
  * 256 + 4 min(m, 2^26) with m = n rounded up to a multiple of 2048 (the
@@ -139,7 +140,7 @@ lb_status logbessel_k_dx_ws(lb_dtype dtype, const void* v, int64_t v_stride, con
  * point stays valid after cudaDeviceReset; the first call on a device may
  * load the library's module, so make it before any stream capture on that
  * device.  Every call shares the one
- * array and clears its counter and mask on the stream: calls whose work overlaps on
+ * array and clears its counter on the stream: calls whose work overlaps on
  * the GPU (different streams, or concurrent host threads) race and must be
  * serialized by the caller.  Other arguments, results and errors as in
  * logbessel_k; LB_ENOTSUP for LB_F32.
@@ -151,8 +152,8 @@ lb_status logbessel_k_noalloc(lb_dtype dtype, const void* v, int64_t v_stride, c
  * d/dx log I_v(x) = I'_v(x) / I_v(x) and d/dx log K_v(x) = K'_v(x) / K_v(x):
  * the adjoint of logbessel_i / logbessel_k, computed by differentiating each
  * region's expression term by term with the same dispatch (the paper lists
- * derivatives as future work, Sec. 7; the integrand derivative of the K
- * integral is dF/dx = F (2v - 1)/(s + 2x)).  Same arguments as logbessel_i.
+ * derivatives as future work, Sec. 7; the integrand of the K integral gains
+ * the factor -cosh t).  Same arguments as logbessel_i.
  * Domain edges: x = 0 gives 0 (I, v = 0), +inf (I, v > 0), -inf (K);
  * x = +inf gives +1 (I) and -1 (K); infinite or NaN order gives NaN.
  * logbessel_k_dx supports LB_TIGHT only (LB_ENOTSUP otherwise).
@@ -218,7 +219,7 @@ lb_status logbessel_classify(int kind, lb_dtype dtype, const void* v, int64_t v_
  * an lb_region value (MU20, U13, FALLBACK, or with LB_PAPER_CPU_ORDER also
  * MU3, U4, U6, U9).  For checking each expression on both sides of a region
  * boundary.  Domain edges still give the values listed above.  `mode` selects
- * the quadrature of the K integral (Gauss for LB_TIGHT, Simpson otherwise).
+ * the quadrature of the K integral (trapezoid for LB_TIGHT, Simpson otherwise).
  */
 lb_status logbessel_eval_region(int kind, lb_dtype dtype, const void* v, int64_t v_stride,
                                 const void* x, void* out, int64_t n, int region, lb_mode mode,
@@ -230,7 +231,8 @@ lb_status logbessel_eval_region(int kind, lb_dtype dtype, const void* v, int64_t
  * events recorded on its stream, and logbessel_profile_get sums the elapsed
  * times per kernel.  Enabling resets the timers.  logbessel_profile_get waits
  * for the recorded events (it synchronizes with the timed launches).
- * slot: 0 = lb_tiles_kernel, 1 = lb_kint_kernel, 2 = lb_classify_kernel,
+ * slot: 0 = lb_tiles_kernel (with lb_tiles32_kernel and lb_small_kernel),
+ * 1 = lb_kint_kernel (with lb_ktrap_kernel), 2 = lb_classify_kernel,
  * 3 = small auxiliary kernels (logbessel_profile_slots() gives the count).  *name points to a static
  * string.  Returns LB_EINVAL for a slot out of range.
  */
@@ -263,8 +265,7 @@ lb_status logbessel_measure_fp64(double* rates, void* cuda_stream);
  * 7 exp, 8 log, 9 reciprocal and 10 1/sqrt in fixed-point integer
  * arithmetic (exp: y <= 708), 11 the Q53 log (out holds the int64 result's
  * bits) and 12 the Q58 exponential of a Q53 shift d <= 0 (in holds d's
- * int64 bits, out the uint64 result's bits), the K integral's node
- * functions.  in/out are device arrays of n doubles (8-byte words).
+ * int64 bits, out the uint64 result's bits).  in/out are device arrays of n doubles (8-byte words).
  * LB_EINVAL for a bad which, size or pointer.
  */
 lb_status logbessel_math_eval(int which, const double* in, double* out, int64_t n, void* cuda_stream);
@@ -277,7 +278,7 @@ lb_status logbessel_math_eval(int which, const double* in, double* out, int64_t 
  * interleaves the work of all resident requests, so requests that arrive
  * while others run overlap on the device.  A request runs the two stages of
  * a direct call: tiles (classify, bin, expressions), then for log K the
- * integral of the fallback pairs, queued per quadrature rule class and
+ * integral of the fallback pairs (FP64), queued per class of the rule and
  * evaluated in windows of one class each (paper Sec. 3.2; Sec. 4.3 groups
  * pairs by expression for the same reason: one code path per warp).
  * Results of host requests are copied back into the caller's buffer.
@@ -342,9 +343,9 @@ lb_status lb_server_stats(lb_server* server, long long* completed, long long* ev
  * (a CTA with nothing to do counts here until it exits).  busy_ns[f] and
  * items[f], f < LB_SERVER_FAMILIES: the summed time CTAs spent running the
  * items of family f, and how many ran; the families are 0 FP64 log I tiles,
- * 1 FP64 log K tiles, 2 FP32 log I tiles, 3 FP32 log K tiles, 4 + c the
- * windows of the FP64 K-integral queue of rule class c (c < 6; the paper
- * modes' single queue counts as class 0), 10 FP32 K-integral windows.  Times
+ * 1 FP64 log K tiles, 2 FP32 log I tiles, 3 FP32 log K tiles (integrals
+ * included), 4 + c the windows of the FP64 K-integral queue of class c (c < 6;
+ * the paper modes' single queue counts as class 0), 10 unused (0).  Times
  * are ns of the device's global timer.  The counters are read by a copy on a
  * stream of the server's own while the kernel runs; the call blocks until
  * that copy is done.  Any pointer may be NULL.  LB_ECUDA if the copy fails.
@@ -362,7 +363,7 @@ const char* lb_server_last_error(void);
  * into the K-integral queue, and every pair offset read back from the queue
  * is checked against its bound before use; a failed check sets a bit of a
  * device status word (1 list write, 2 list read, 4 queue write, 8 queue
- * count above the capacity, 16 pair offset beyond the chunk, 32 rule class
+ * count above the capacity, 16 pair offset beyond the chunk, 32 queue key
  * out of range) and the access is skipped, so an index error is recorded
  * instead of faulting.  Results are identical to the release build's when
  * no check fails.  logbessel_check_status stores the word in *bits (host

@@ -7,8 +7,9 @@
 //   U_K   : uniform large-order expansion (Eqs. "log Iv u k", "log Kv u k")
 //   series: power series of I_v summed in log scale (Eqs. "Iv infinite series",
 //           "ak recurrence", "log Iv")
-// The K integral (Eq. "log Kv integral") is warp-cooperative and lives in
-// lb_kint.cuh.
+// U_K values and derivatives in tight mode run in fixed point (lb_uniform.cuh).
+// The K integral (Eq. "log Kv integral") is in lb_ktrap.cuh (tight mode, one
+// pair per thread) and lb_kint.cuh (the paper's Simpson rule, warp-cooperative).
 #pragma once
 
 #include <math.h>

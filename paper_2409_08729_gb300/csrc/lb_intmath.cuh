@@ -275,12 +275,10 @@ LB_IX_FN double ix_log(double z) {
 }
 
 // ---------------------------------------------------------------------------
-// Fixed point for sums of terms e^(c + a log z - m): the K-integral nodes
-// (lb_kint.cuh) keep each node's logarithm term in Q53 (an int64 holding
-// value 2^53; |value| < 2^10), form it, its warp maximum and the shift by
-// that maximum with integer instructions, and exponentiate the shifted
-// term from Q53 straight into the Q58 sum.  No double is packed or unpacked
-// between the steps, and no FP64 instruction runs.
+// Fixed point: logarithms in Q53 (an int64 holding value 2^53; |value| <
+// 2^10), which the uniform expansions (lb_uniform.cuh) add to their sums
+// without packing a double, conversions to fixed point, and the exponential
+// of a Q53 shift as a Q58 term.  No FP64 instruction runs.
 // ---------------------------------------------------------------------------
 
 // round(d 2^q) for |d| < 2^(62 - q), from the bit fields (ties away from 0;

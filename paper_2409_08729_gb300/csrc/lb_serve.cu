@@ -15,8 +15,9 @@
 //   stage A, tile items: each tile goes through classify, bin and the
 //     per-thread expressions (lb_tile.cuh); the K pairs of the fallback
 //     region are appended to per-class queues in the arena, one queue per
-//     quadrature rule class of the K integral (the six code paths of
-//     lb_kint.cuh for the FP64 Gauss rules; one queue otherwise);
+//     class of the FP64 tight K integral (kt_class of lb_ktrap.cuh: the number
+//     of nodes per octave, Temme's series, the general form; one queue in the
+//     paper's modes; FP32 items evaluate their integrals in the tile);
 //   stage B, K-window items: when a request's last tile is done, the device
 //     posts the per-class queue lengths to mapped host memory and the
 //     scheduler publishes windows of each class's queue, costliest class
@@ -61,8 +62,8 @@ constexpr int kKItemsPerClass = 64;    // stage B: at most this many windows per
 constexpr int kKWindowMin = 512;       // smallest window of a class queue (pairs)
 // Item families of the device time accounts (lb_server_device_stats): FP64
 // tiles of log I and log K, FP32 tiles of log I and log K, FP64 K windows of
-// each rule class (or the one queue of the paper modes, as class 0), FP32 K
-// windows.
+// each class (or the one queue of the paper modes, as class 0), and one
+// that nothing runs any more (FP32 K windows).
 constexpr int kFamilies = LB_SERVER_FAMILIES;
 static_assert(kFamilies == 4 + kKClasses + 1, "item families");
 
@@ -113,7 +114,7 @@ struct ServeAux {          // per-tile class counts and queue bases of the K pai
 };
 
 // Stage A: one tile of a request.  K pairs of the fallback region go to the
-// queue of their rule class (class 0 when the request has one queue); their
+// queue of their class (class 0 when the request has one queue); their
 // order within a queue does not change any result.
 template <int KIND, typename T>
 __device__ __forceinline__ void serve_tile(TileShared<T, LB_THREADS, LB_ITEMS>& S, ServeAux& A, const SlotDesc& d, int64_t tile,

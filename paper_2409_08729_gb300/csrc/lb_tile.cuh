@@ -42,7 +42,7 @@ namespace lb {
 // back from the queue is checked against its bound before use; a failed
 // check sets a bit of lb_check_status (1 list write, 2 list read, 4 queue
 // write, 8 queue count above the capacity, 16 pair offset beyond the chunk,
-// 32 rule class out of range) and the access is skipped or clamped.  It
+// 32 queue key out of range) and the access is skipped or clamped.  It
 // stands in for a memory checker: the kernels record where an index left
 // its buffer instead of faulting.  Release builds compile the checks out.
 #ifdef LB_CHECKS

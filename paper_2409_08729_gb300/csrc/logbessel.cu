@@ -3,20 +3,22 @@
 // Pipeline for one call (paper Sec. 4.3 sorts the pairs by expression before
 // launch so that warps do not diverge; here the grouping is done on chip):
 //
-//   1. lb_tiles_kernel: persistent CTAs walk tiles of kTile pairs.  Each
-//      thread loads LB_ITEMS pairs (coalesced), handles domain edges, and
-//      classifies the rest (Table "input ranges").  The tile's pairs are
-//      binned per region into shared-memory index lists; the warps take
-//      32-pair chunks of the lists from shared counters, so every warp runs
-//      one expression (mu_20, U_K, power series) at a time.  K pairs of the
-//      fallback region are appended to a global queue instead.
+//   1. lb_tiles_kernel: persistent CTAs walk tiles of 256 to 2048 pairs (by
+//      the size of the call).  Each thread loads its pairs (coalesced),
+//      handles domain edges, and classifies the rest (Table "input ranges").
+//      The tile's pairs are binned per region into shared-memory index lists;
+//      the warps take 32-pair chunks of the lists from shared counters, so
+//      every warp runs one expression (mu_20, U_K, power series) at a time.
+//      K pairs of the fallback region are evaluated in the tile (calls below
+//      2^17 pairs) or appended to a global queue.
 //   2. lb_ktrap_kernel (tight FP64): one thread per queued K pair evaluates the
 //      integral by the trapezoid rule (lb_ktrap.cuh); lb_kint_kernel (the
 //      paper's dispatches): one warp per pair with the nodes spread over the
 //      lanes (lb_kint.cuh).
 // An FP64 call with one order for all pairs (v_stride 0) has its order's
-// constants computed once per block (ScalarOrder).  FP32 calls in tight mode
-// run lb_tiles32_kernel alone.
+// constants computed once per block (ScalarOrder).  FP64 calls of up to
+// LB_SMALL_N pairs run lb_small_kernel alone, FP32 calls in tight mode
+// lb_tiles32_kernel alone.
 //
 // The plain form computes in FP64; its exps and logs are evaluated in
 // integer arithmetic where that is faster (lb_intmath.cuh).
@@ -108,7 +110,14 @@ constexpr uint32_t kQueueOffsetMask = (1u << kQueueOffsetBits) - 1u;
 
 // Tile kernel: classify, bin per region in shared memory, evaluate the
 // per-thread expressions (lb_tile.cuh); K fallback pairs go to a global queue
-// for lb_kint_kernel.  T = double (FP64) or float (FP32-mixed).
+// for lb_ktrap_kernel (lb_kint_kernel in the paper's modes).  T = double
+// (FP64) or float (FP32-mixed, the paper's modes).
+// What bounds it: issue, spread over the pipes.  The mixed-order log K call
+// at 6M pairs runs in 367 us (470 with the sums in FP64 and double-float),
+// issue 66 % of cycles, FP64 pipe 48 %, ALU 47 %, integer multiplies 43 %,
+// 1454 thread instructions per pair at 27 of 32 lanes, DRAM 4 %; the rest
+// is waits at the tile's barriers and on fixed latencies, which more warps do
+// not cover (registers allow 48 an SM).
 // SO: one order for every argument (FP64 values, v_stride 0, no forced
 // region): the order's constants once per block, and only the per-order
 // forms of the expressions compiled in (each kernel carries one form's
@@ -198,7 +207,9 @@ lb_small_kernel(const double* __restrict__ v, int64_t v_stride, double v0, const
 // 48 KB of shared memory hold beside the table), equal ones, as few per block
 // as the queue needs: on the whole domain (6.9M queued pairs) 1.69 ms with
 // 128-thread blocks and 1024-pair windows, 1.28 with 256 and 2048, 1.18 with
-// 512 and 4096, 1.13 with 512 and 16384.
+// 512 and 4096, 1.13 with 512 and 16384.  (The warp-per-pair Gauss rules it
+// replaces took 19.1 ms on the same queue.)  There issue is at 60 %, the ALU
+// at 56 %, integer multiplies at 47 %.
 constexpr int kKtThreads = LB_KTRAP_THREADS;
 constexpr int kKtWindow = LB_KTRAP_WINDOW;
 static_assert(kKtWindow <= 65536, "16-bit offsets within a window");
@@ -306,7 +317,11 @@ lb_kint_kernel(const double* __restrict__ v, int64_t v_stride, const double* __r
   }
 }
 
-// FP32, tight mode: see warp_pairs32.
+// FP32, tight mode: see warp_pairs32.  Bound by issue: log I over mixed
+// orders, 24M pairs, 131 us (387 with the binned tiles), 155 thread
+// instructions per pair, issue 75 %, ALU 51 %, DRAM 17 % at 6M pairs; log K
+// over the whole domain, 16M pairs, 219 us (2670 with a warp per integral),
+// issue 69 % and instruction fetch, as its warps are in different loops.
 template <int KIND, int VEC>
 __global__ void __launch_bounds__(LB_THREADS, LB_TILES32_CTAS_PER_SM)
 lb_tiles32_kernel(const float* __restrict__ v, int64_t v_stride, const float* __restrict__ x,
@@ -897,9 +912,10 @@ lb_status logbessel_host(int fn, lb_dtype dtype, const void* v, int64_t v_stride
   lb_status s = validate(dtype, v, v_stride, x, out, n, (int)mode);
   if (s != LB_OK || n == 0) return s;
   // default pieces of up to 2M pairs: log K on 8M pairs takes 1.00 ms end to
-  // end against 0.98 (2^20), 1.20 (2^22) and 1.11 ms (2^24), on 20M pairs 2.12
-  // against 2.10, 2.16 and 2.37: larger ones leave longer first and last copies
-  // unoverlapped, smaller ones cost more kernel ends
+  // end against 0.98 (2^20), 1.20 (2^22) and 1.11 ms (2^24), one order and 20M
+  // pairs 1.36 against 1.41, 1.48 and 1.65, per-pair orders and 220M pairs
+  // 19.8 against 20.9, 19.5 and 20.2: larger ones leave longer first and last
+  // copies unoverlapped, smaller ones cost more kernel ends
   if (chunk <= 0) chunk = (int64_t)1 << 21;
   if (chunk > kChunk) chunk = kChunk;
   if ((fn >= 2 && dtype != LB_F64) || (fn == 3 && mode != LB_TIGHT))
@@ -962,8 +978,8 @@ lb_status logbessel_host(int fn, lb_dtype dtype, const void* v, int64_t v_stride
     }
     // one pass per chunk (cn <= cap <= kChunk), the K queue in ws.  Even and
     // odd pieces run on two compute streams with a queue each, so a piece's
-    // kernels start while the previous piece's last kernels drain (the K
-    // integral's class kernels leave the GPU partly idle at their ends).
+    // kernels start while the previous piece's last kernels drain (the
+    // blocks of the tile and K-integral kernels end at different times).
     cudaStream_t sc = st[(i & 1) ? 3 : 1];
     void* ws = P.dbuf + slot * nbuf + (size_t)(i & 1) * qbytes;
     if (cudaStreamWaitEvent(sc, P.ev_in[b], 0) != cudaSuccess) {
