@@ -24,6 +24,7 @@ template <> __host__ __device__ __forceinline__ float lb_fma<float>(float a, flo
 #include "lb_fastmath.cuh"
 #include "lb_intmath.cuh"
 #include "lb_uniform.cuh"
+#include "lb_lgamma.cuh"
 
 namespace lb {
 
@@ -441,6 +442,10 @@ __device__ __forceinline__ dfloat series_ratio_df(dfloat y, dfloat v, int k) {
   return r;
 }
 
+// lgamma(v + 1): lg_lgamma1p, or (orders past 17, as forced evaluations have)
+// the library's.
+static __device__ __noinline__ double lgamma1p(double v) { return lg_ok(v) ? lg_lgamma1p(v) : lgamma(v + 1.0); }
+
 __device__ __forceinline__ double series_log_i_n(double v, double x, int packed) {
   const int n = __reduce_max_sync(0xffffffffu, series_count(packed));
   const int h = __reduce_max_sync(0xffffffffu, series_head(packed));
@@ -463,7 +468,7 @@ __device__ __forceinline__ double series_log_i_n(double v, double x, int packed)
     A = fma(d, B, y * A);
     B *= d;
   }
-  double res = ix_log_call(A * ix_rcp_call(B)) - lgamma(v + 1.0);
+  double res = ix_log_call(A * ix_rcp_call(B)) - lgamma1p(v);
   if ((__double_as_longlong(v) << 1) != 0) res = fma(v, ix_log_call(0.5 * x), res);   // v != 0, on the bits
   return res;
 }
@@ -529,7 +534,7 @@ __device__ __forceinline__ void scalar_order_setup(ScalarOrder& so, double v) {
       so.muc = (KIND == KIND_I ? kMuSoLogI : kMuSoLogK) - 2 * (59 - muq) * kLn2Q53;
     }
   } else if (tid < 64) {
-    if (tid == 32) so.lg1 = lgamma(v + 1.0);
+    if (tid == 32) so.lg1 = lgamma1p(v);
   }
   if (NT > 64 ? tid >= 64 : tid >= 32)
     for (int k = tid - (NT > 64 ? 63 : 31); k <= 90; k += NT - (NT > 64 ? 64 : 32)) {
