@@ -536,10 +536,12 @@ lb_status run_tiles32(const float* v, int64_t v_stride, const float* x, float* o
 //   below 2^20        tiles of 512 pairs, two per thread, K fallback queued;
 //   from there        tiles of 2048 pairs, four per thread, K fallback queued.
 // Device time of a call on the mixed-order sweep, log I / log K, us: 1000
-// pairs 12 / 14 (small kernel) against 18 / 16 (256-pair tiles) and 29 / 37
-// (2048-pair tiles, queued); 24000 pairs 19 / 17 against 29 / 41 (small
-// kernel 29 / 35); 100000 pairs 25 / 26 against 31 / 43; 1M pairs 105 / 115
-// against 119 / 129.
+// pairs 12 / 12 (small kernel) against 16 / 15 (256-pair tiles); 4000 pairs 17
+// / 16 (256-pair tiles) against 19 / 21 (small kernel); 24000 pairs 17 / 17
+// against 25 / 33 (small kernel), 19 / 36 (512-pair tiles, queued) and 32 / 49
+// (2048-pair tiles); 100000 pairs 22 / 27 against 23 / 43 and 33 / 53; 200000
+// pairs 27 / 49 against 33 / 55 (2048-pair tiles); 1M pairs 91 / 108 against 86
+// / 110, log C_2048 72 against 79.
 constexpr int64_t kMidInTile = (int64_t)1 << 17, kMid = (int64_t)1 << 20;
 
 template <int KIND, bool DX, typename T, bool SO, int NT, int IT, bool KIN>
