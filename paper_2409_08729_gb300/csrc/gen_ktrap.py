@@ -31,7 +31,8 @@ def f32(v):
 
 
 def table(name, vals, per=4):
-    print("LB_IX_TABLE unsigned long long %s[%d] = {" % (name, len(vals)))
+    # the kernels copy it to shared memory 16 bytes at a time
+    print("alignas(16) LB_IX_TABLE unsigned long long %s[%d] = {" % (name, len(vals)))
     for i in range(0, len(vals), per):
         print("    " + ", ".join("0x%016xull" % v for v in vals[i:i + per]) + ",")
     print("};")

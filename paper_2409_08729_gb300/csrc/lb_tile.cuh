@@ -117,7 +117,8 @@ __device__ __forceinline__ int tile_classify(T v, T x, int mode) {
 
 // The 16 KB table of kt_exp2_q58 in shared memory (random lookups cost a few
 // bank conflicts there, up to 32 cache-line accesses in global memory).  All
-// NT threads of the block call it; the caller synchronizes.
+// NT threads of the block call it; the caller synchronizes.  16 bytes at a
+// time: both arrays are declared with that alignment.
 template <int NT>
 __device__ __forceinline__ void kt_load_table(unsigned long long* tab) {
   for (int i = 2 * threadIdx.x; i < 2048; i += 2 * NT)
