@@ -25,6 +25,7 @@ template <> __host__ __device__ __forceinline__ float lb_fma<float>(float a, flo
 #include "lb_intmath.cuh"
 #include "lb_uniform.cuh"
 #include "lb_lgamma.cuh"
+#include "lb_order.cuh"
 
 namespace lb {
 
@@ -259,8 +260,6 @@ static __constant__ float kMuOdd[21] = {0.0f, 1.0f, 9.0f, 25.0f, 49.0f, 81.0f, 1
 static __constant__ double kMuOddD[21] = {0.0, 1.0, 9.0, 25.0, 49.0, 81.0, 121.0, 169.0, 225.0, 289.0, 361.0, 441.0, 529.0, 625.0, 729.0, 841.0, 961.0, 1089.0, 1225.0, 1369.0, 1521.0};
 static __constant__ double kMuF[22] = {0.0, 2432902008176640000.0, 2432902008176640000.0, 1216451004088320000.0, 405483668029440000.0, 101370917007360000.0, 20274183401472000.0, 3379030566912000.0, 482718652416000.0, 60339831552000.0, 6704425728000.0, 670442572800.0, 60949324800.0, 5079110400.0, 390700800.0, 27907200.0, 1860480.0, 116280.0, 6840.0, 380.0, 20.0, 1.0};
 static __constant__ float kMuFd[22][2] = {{0.0f, 0.0f}, {2.4329020231636746e+18f, -14987034624.0f}, {2.4329020231636746e+18f, -14987034624.0f}, {1.2164510115818373e+18f, -7493517312.0f}, {4.054836705272791e+17f, -2497839104.0f}, {1.0137091763181978e+17f, -624459776.0f}, {2.0274182667370496e+16f, 734101504.0f}, {3379030623518720.0f, -56606720.0f}, {482718655709184.0f, -3293184.0f}, {60339831963648.0f, -411648.0f}, {6704425598976.0f, 129024.0f}, {670442586112.0f, -13312.0f}, {60949323776.0f, 1024.0f}, {5079110656.0f, -256.0f}, {390700800.0f, 0.0f}, {27907200.0f, 0.0f}, {1860480.0f, 0.0f}, {116280.0f, 0.0f}, {6840.0f, 0.0f}, {380.0f, 0.0f}, {20.0f, 0.0f}, {1.0f, 0.0f}};
-constexpr long long kMuSoLogI = 2175819361628260ll, kMuSoLogK = 22797439711033177ll;   // log(8/(2 pi)), log(4 pi), Q53
-constexpr long long kLn2Q53 = 6243314768165359ll;
 constexpr long long kMuLogI = -760474846706970267ll;   // log(8/(2 pi)) - 2 log 20!, Q53
 constexpr long long kMuLogK = -739853226357565351ll;   // log(4 pi) - 2 log 20!, Q53
 
@@ -482,7 +481,8 @@ __device__ __forceinline__ double series_log_i(double v, double x) {
 // the expressions are then the same for every pair, and a block computes
 // them once (scalar_order_setup):
 //   mu_K:   S = sum_k a_k w^k, w = 1/(8x), a_k = s^k prod_{j<=k} (mu - (2j-1)^2) / k!
-//           -- one fixed-point multiply-add per term, no FP64;
+//           -- one fixed-point multiply-add per term, no FP64, where that
+//           keeps enough of S (lb_order.cuh);
 //   series: P <- 1 + (y / (k (k + v))) P with the reciprocals 1/(k (k + v))
 //           tabulated -- two operations per term instead of six, and
 //           lgamma(v + 1) once.
@@ -490,9 +490,10 @@ __device__ __forceinline__ double series_log_i(double v, double x) {
 // ---------------------------------------------------------------------------
 struct ScalarOrder {
   double v, lg1;                        // v, lgamma(v + 1)
-  int muj;                              // W = 2^muj w <= 1/2 wherever the dispatch takes mu_20
-  long long muc;                        // log constant of mu_K, Q53, the scale of mu[] included
-  long long mu[21];                     // a_0..a_20 / 2^(k muj) (sign s of the kind folded in), Q(59 - muq), + 2^62
+  double scale;                         // so_scale
+  bool mu_general;                      // so_general
+  long long muc;                        // so_log_const
+  long long mu[21];                     // so_coef of b_0 .. b_20
   double ser[91];                       // 1 / (k (k + v)), k = 1..90
   dfloat serd[91];                      // ser[] in double-float
 };
@@ -502,36 +503,37 @@ struct ScalarOrder {
 // 20 ratios of mu_K on 20 lanes and their products by a warp scan, lgamma on
 // another warp, the series' reciprocals on the rest.
 template <int KIND, int NT>
-__device__ __forceinline__ void scalar_order_setup(ScalarOrder& so, double v) {
+__device__ __forceinline__ void scalar_order_setup(ScalarOrder& so, double v, int mode) {
   const int tid = threadIdx.x;
   if (tid < 32) {
-    // 2^j = the power of two at most 4 xmin, xmin the smallest x at which a
-    // dispatch takes mu_20 for this order (tight: 18.5, or v^2 < 3.24 x;
-    // paper: 0.5113 log x + 0.7939 > log v): then 2^j / (8 x) <= 1/2
-    int j = 6;                                      // 4 x 18.4
-    if (!(v < 15.4)) {
-      const int e = ilogb(v);
-      const float lv = (float)e + log2f((float)scalbn(v, -e));
-      const float l = fminf(2.0f * lv - 1.6961f, 1.9558f * (lv - 1.1454f));   // log2 of v^2/3.24, (v/2.212)^1.9558
-      j = (int)floorf(2.0f + fmaxf(5.88f, l - 0.05f - 2e-6f * fabsf(l)));      // log2 59 at least
-    }
-    const int k = tid < 1 ? 1 : (tid > 20 ? 20 : tid);
-    const double mu = 4.0 * v * v, s = KIND == KIND_I ? -1.0 : 1.0;
-    double a = ldexp(s * (mu - (double)((2 * k - 1) * (2 * k - 1))) / (double)k, -j);
-    if (tid == 0 || tid > 20) a = tid == 0 ? 1.0 : 0.0;
+    const int k = tid < 20 ? tid : 20;
+    const double rf = __ldg(&lb_rfact[k][0]), rfl = __ldg(&lb_rfact[k][1]);
+    const double scale = so_scale(KIND, mode == MODE_TIGHT, v);
+    double bl, b = so_ratio(KIND, v, k < 1 ? 1 : k, scale, bl);
+    if (tid == 0) { b = 1.0; bl = 0.0; }
+    if (so_pairs(v)) {
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {              // a_0 .. a_tid
-      const double u = __shfl_up_sync(0xffffffffu, a, o);
-      if (tid >= o) a *= u;
+      for (int o = 1; o < 32; o <<= 1) {            // k! b_k, k = tid
+        const double u = __shfl_up_sync(0xffffffffu, b, o), ul = __shfl_up_sync(0xffffffffu, bl, o);
+        if (tid >= o) so_mul(b, bl, u, ul);
+      }
+      so_mul(b, bl, rf, rfl);
+    } else {
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const double u = __shfl_up_sync(0xffffffffu, b, o);
+        if (tid >= o) b *= u;
+      }
+      b *= rf;
+      bl = 0.0;
     }
-    // |a_k| 2^(59 - muq) < 2^60: with W <= 1/2 every Horner sum stays within +-2^61
-    int muq = tid <= 20 && a != 0.0 ? max(ilogb(fabs(a)), 0) : 0;
-    muq = min(__reduce_max_sync(0xffffffffu, muq), 50);
-    if (tid <= 20) so.mu[tid] = ix_fix(a, 59 - muq) + (1ll << 62);
+    const int muq = __reduce_max_sync(0xffffffffu, tid <= 20 ? so_size(b) : 0);
+    if (tid <= 20) so.mu[tid] = so_coef(b, bl, muq);
     if (tid == 0) {
       so.v = v;
-      so.muj = j;
-      so.muc = (KIND == KIND_I ? kMuSoLogI : kMuSoLogK) - 2 * (59 - muq) * kLn2Q53;
+      so.scale = scale;
+      so.mu_general = so_general(KIND, muq, scale);
+      so.muc = so_log_const(KIND, muq, scale);
     }
   } else if (tid < 64) {
     if (tid == 32) so.lg1 = lgamma1p(v);
@@ -546,17 +548,11 @@ __device__ __forceinline__ void scalar_order_setup(ScalarOrder& so, double v) {
 
 template <int KIND>
 __device__ __forceinline__ double mu_expr_so(const ScalarOrder& so, double x, int counts) {
+  if (KIND == KIND_I && so.mu_general) return mu_expr_n<KIND>(so.v, x, counts, 20);   // the same for the whole block
   const int n = __reduce_max_sync(0xffffffffu, counts & 255);
-  const double rx = ix_rcp_call(8.0 * x);
-  const uint64_t W = (uint64_t)ix_fix(rx, 64 + so.muj);   // below 2^63
-  // Horner on the sums plus 2^62 (positive: the short unsigned product), the
-  // bias's product taken off again
-  const uint64_t bias = W >> 2;
-  uint64_t acc = (uint64_t)so.mu[n];
-#pragma unroll 2
-  for (int k = n - 1; k >= 0; --k) acc = (uint64_t)so.mu[k] + kt_mulhi(acc, W) - bias;
-  const double S = (double)(long long)(acc - (1ull << 62));
-  return fma(0x1p-54, log_q53_plus(S * S * rx, so.muc), KIND == KIND_I ? x : -x);
+  const double W = ix_rcp_call(so.scale * x);
+  const double S = so_sum(so.mu, W, n);
+  return fma(0x1p-54, log_q53_plus(S * S * W, so.muc), KIND == KIND_I ? x : -x);
 }
 
 __device__ __forceinline__ double series_so(const ScalarOrder& so, double x, int packed) {

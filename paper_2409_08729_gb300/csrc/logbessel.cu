@@ -150,7 +150,7 @@ lb_tiles_kernel(const T* __restrict__ v, int64_t v_stride, T v0, const T* __rest
   const ScalarOrder* so = nullptr;
   if constexpr (SO) {
     __shared__ ScalarOrder SOC;
-    scalar_order_setup<KIND, NT>(SOC, KIND == KIND_K ? fabs((double)v0) : (double)v0);
+    scalar_order_setup<KIND, NT>(SOC, KIND == KIND_K ? fabs((double)v0) : (double)v0, mode);
     so = &SOC;
   }
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
