@@ -8,6 +8,8 @@ stream.  There is no CPU path: calls on CPU tensors raise.
 Paper: Plesner, Sorensen, Hauberg, "Accurate Computation of the Logarithm of
 Modified Bessel Functions on GPUs", ICS 2024 (arXiv 2409.08729).
 """
+import ctypes
+
 import torch
 
 from . import _binding
@@ -30,6 +32,15 @@ def _dtype_code(dt):
     raise TypeError("log-Bessel functions take float64 or float32 tensors, got %s" % dt)
 
 
+def _order(v, x):
+    """An order given as a number, as a tensor of the type the call computes in
+    (orders past single precision's range round to an infinity there).  A fill
+    on the stream: no copy from the host."""
+    dt = x.dtype if x.dtype in (torch.float32, torch.float64) else torch.float64
+    v = float(v)
+    return torch.full((1,), ctypes.c_float(v).value if dt == torch.float32 else v, dtype=dt, device=x.device)
+
+
 def _prep(v, x):
     """Broadcast (v, x) to CUDA tensors of a common float dtype.
 
@@ -41,7 +52,7 @@ def _prep(v, x):
         raise ValueError("x must be on a CUDA device (the library has no CPU path)")
     dt = x.dtype if x.dtype in (torch.float32, torch.float64) else torch.float64
     if not isinstance(v, torch.Tensor):
-        v = torch.full((1,), float(v), dtype=dt, device=x.device)   # a fill on the stream, no copy from the host
+        v = _order(v, x)
     if v.device != x.device:
         raise ValueError("v and x must be on the same device")
     v = v.to(dt)
@@ -123,7 +134,7 @@ class _LogBesselFn(torch.autograd.Function):
 def _with_grad(kind, v, x, mode, out):
     if out is None and isinstance(x, torch.Tensor) and x.requires_grad and torch.is_grad_enabled():
         if not isinstance(v, torch.Tensor):
-            v = torch.tensor(float(v), dtype=x.dtype, device=x.device)
+            v = _order(v, x)
         return _LogBesselFn.apply(v, x, kind, mode)
     return _call("logbessel_i" if kind == "i" else "logbessel_k", v, x, mode, out)
 
