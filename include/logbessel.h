@@ -284,8 +284,8 @@ lb_status logbessel_math_eval(int which, const double* in, double* out, int64_t 
  * Results of host requests are copied back into the caller's buffer.
  *
  *   arena_bytes  device memory for request buffers (>= 1 MiB); a host
- *                request needs 3 n elements (v, x, out), a log K request
- *                also its queues: 24 n bytes (FP64, LB_TIGHT: six rule
+ *                request needs 3 n elements (v, x, out), an FP64 log K
+ *                request also its queues: 24 n bytes (LB_TIGHT: six
  *                classes) or 4 n bytes; each part rounded to 256 B
  *   max_slots    requests resident on the device at once (1..4096)
  *   ctas_per_sm  persistent thread blocks per SM (1..8)
@@ -314,7 +314,7 @@ lb_status logbessel_math_eval(int which, const double* in, double* out, int64_t 
  * stay valid until lb_server_wait returns LB_OK), or NULL when they are
  * already complete.  When lb_server_wait returns LB_OK the results are in
  * out and the server no longer reads v and x.  The arena then holds only the
- * K queues (none for log I).
+ * queues of FP64 log K (nothing otherwise).
  */
 typedef struct lb_server lb_server;
 typedef struct {

@@ -71,11 +71,11 @@ struct SlotDesc {          // mapped host memory: written by the host, read by t
   int kind;                // 0 = I, 1 = K
   int dtype;               // LB_F64 or LB_F32
   int mode;
-  int nclass;              // K: queues (kKClasses in FP64 tight mode, else 1); I: 0
+  int nclass;              // FP64 K: queues (kKClasses in tight mode, else 1); 0 otherwise
   long long n;
   long long v_stride;
   unsigned long long v, x, out;   // device addresses (arena, or the caller's for device requests)
-  unsigned long long queue;       // K: nclass queues of n uint32 pair offsets each (arena)
+  unsigned long long queue;       // nclass queues of n uint32 pair offsets each (arena)
   long long ntiles;
   long long kitems;        // stage B items published for the request (written before they are)
 };
@@ -100,7 +100,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 
 // Shared memory of the persistent kernel: one tile, the exponential's
-// table (FP64 K windows) or the node table of an FP32 K window with one order.
+// table (FP64 K windows) or the warps' pair lists (FP32 tight mode).
 union ServeShared {
   TileShared<double, LB_THREADS, LB_ITEMS> d;
   TileShared<float, LB_THREADS, LB_ITEMS> f;
@@ -235,8 +235,7 @@ lb_serve_kernel(Ctl* ctl, const SlotDesc* slots, const WorkItem* ring, int ring_
         pos.store((unsigned long long)got + 1ull, cuda::memory_order_relaxed);
         item = ring[got % ring_cap];
         desc = slots[item.slot];
-        fam = item.type == 0 ? (desc.dtype == LB_F64 ? 0 : 2) + desc.kind
-                             : (desc.dtype == LB_F64 ? 4 + (item.type - 1) : 4 + kKClasses);
+        fam = item.type == 0 ? (desc.dtype == LB_F64 ? 0 : 2) + desc.kind : 4 + (item.type - 1);
       }
       t_item = global_ns();
       atomicAdd(dstat, t_item - t_free);           // claiming, and waiting for work
@@ -280,7 +279,7 @@ lb_serve_kernel(Ctl* ctl, const SlotDesc* slots, const WorkItem* ring, int ring_
         if (old + nt == d.ntiles) {                // the request's last tile
           tiles_done[it.slot] = 0;                 // ready for the slot's next request
           bool more = false;
-          if (d.kind == 1) {
+          if (d.nclass > 0) {
             __threadfence();
             for (int c = 0; c < d.nclass; ++c) {
               const unsigned m = *(volatile unsigned*)(qc + c);
@@ -370,7 +369,7 @@ struct Request {
     if (device) return 0;
     return round256((size_t)(v_stride ? n : 1) * elem) + 2 * round256((size_t)n * elem);
   }
-  size_t queue_bytes() const { return kind == 1 ? round256((size_t)nclass * (size_t)n * 4) : 0; }
+  size_t queue_bytes() const { return round256((size_t)nclass * (size_t)n * 4); }
 };
 
 }  // namespace
@@ -563,7 +562,7 @@ void lb_server::publish_k(Request* r) {
         it.begin = (int)b;
         it.end = (int)(b + w < m ? b + w : m);
         it.type = 1 + c;
-        hold(r->dtype == LB_F64 ? 4 + c : 4 + kKClasses, it, t);
+        hold(4 + c, it, t);
       }
     }
   }
@@ -619,7 +618,7 @@ bool lb_server::step(std::vector<Request*>& finished) {
     sd.kind = r->kind;
     sd.dtype = r->dtype;
     sd.mode = r->mode;
-    sd.nclass = r->kind == 1 ? r->nclass : 0;
+    sd.nclass = r->nclass;
     sd.n = r->n;
     sd.v_stride = r->v_stride;
     sd.v = (unsigned long long)dv;
@@ -740,7 +739,8 @@ void lb_server::loop() {
 
 lb_status lb_server::submit(Request* r, long long* ticket) {
   r->elem = r->dtype == LB_F64 ? 8 : 4;
-  r->nclass = (r->kind == 1 && r->dtype == LB_F64 && r->mode == LB_TIGHT) ? kKClasses : 1;
+  // FP32 log K (tight mode only) evaluates its integrals in the tile items: no queue, and no arena for one
+  r->nclass = r->kind == 0 || r->dtype != LB_F64 ? 0 : (r->mode == LB_TIGHT ? kKClasses : 1);
   const size_t need = r->data_bytes() + r->queue_bytes();
   if (need > arena.size) {                         // arena.size is fixed after creation
     delete r;
