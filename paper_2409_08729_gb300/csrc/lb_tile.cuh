@@ -475,23 +475,20 @@ __device__ __forceinline__ double kint_warp_batch(double vi, double xi, int m, i
   return pre + mine;
 }
 
-// One pair per lane, `ppw` pairs per warp, tight mode (FP64): for calls with
-// too few pairs for the tiles to fill the GPU.  The groups of expressions
-// present in the warp run one after another; lanes outside the group run on
-// its first pair's arguments, so that the warp stays together, and drop the
-// result.  One kernel and no queue; tab: 16 KB of shared memory for the K
-// integral's table (filled if a pair of the block needs it).
+// One pair per warp, tight mode (FP64): for calls with too few pairs for the
+// tiles to fill the GPU.  Every lane holds the pair (i, the same for the warp)
+// and computes the same.  One kernel and no queue; tab: 16 KB of shared memory
+// for the K integral's table (filled if a pair of the block needs it).
 template <int KIND, bool DX, int NT>
-__device__ __forceinline__ void warp_pairs64(const double* __restrict__ v, int64_t v_stride, double v0,
-                                             const double* __restrict__ x, double* __restrict__ out, int64_t i,
-                                             bool valid, double vmf_d, unsigned long long* tab) {
+__device__ __forceinline__ void warp_pair64(const double* __restrict__ v, int64_t v_stride, double v0,
+                                            const double* __restrict__ x, double* __restrict__ out, int64_t i,
+                                            bool valid, double vmf_d, unsigned long long* tab) {
   double vi = valid ? (v_stride ? v[i] : v0) : 1.0;
   const double xi = valid ? x[i] : 1.0;
   if constexpr (KIND == KIND_K) vi = fabs(vi);
   double val = 0.0;
-  const bool edge = tile_special<KIND, DX, double>(vi, xi, &val);
   int r = R_SPECIAL, n = 0;
-  if (valid && !edge) {
+  if (valid && !tile_special<KIND, DX, double>(vi, xi, &val)) {
     r = tile_classify<KIND, DX, double>(vi, xi, MODE_TIGHT);
     tile_key<KIND, DX, double, true>(r, vi, xi, &n);
     if (r == R_MU20) n = mu_counts(f32_cut(vi), f32_cut(xi));
@@ -504,21 +501,11 @@ __device__ __forceinline__ void warp_pairs64(const double* __restrict__ v, int64
       __syncthreads();
     }
   }
-  unsigned todo = __ballot_sync(0xffffffffu, r != R_SPECIAL);
-  while (todo) {
-    const int lead = __ffs(todo) - 1, g = __shfl_sync(0xffffffffu, r, lead);
-    const bool in = r == g;
-    const unsigned members = __ballot_sync(0xffffffffu, in);
-    const double vl = __shfl_sync(0xffffffffu, vi, lead), xl = __shfl_sync(0xffffffffu, xi, lead);
-    const int nl = __shfl_sync(0xffffffffu, n, lead);
-    const double f = tile_expr<KIND, DX, double, false>(g, in ? vi : vl, in ? xi : xl, in ? n : nl, nullptr, tab);
-    if (in) val = f;
-    todo &= ~members;
-  }
+  if (r != R_SPECIAL) val = tile_expr<KIND, DX, double, false>(r, vi, xi, n, nullptr, tab);
   if constexpr (KIND == KIND_I) {
     if (valid && vmf_d >= 0.0) val = vmf_form<DX>(vmf_d, xi, val);
   }
-  if (valid) out[i] = val;
+  if (valid && (threadIdx.x & 31) == 0) out[i] = val;
 }
 
 // FP32 pairs in tight mode (log I or log K).  Each warp works by itself, with

@@ -182,16 +182,15 @@ lb_tiles_kernel(const T* __restrict__ v, int64_t v_stride, T v0, const T* __rest
   }
 }
 
-// Calls of few pairs: see warp_pairs64.
+// Calls of few pairs: see warp_pair64.
 template <int KIND, bool DX>
 __global__ void __launch_bounds__(LB_SMALL_THREADS)
 lb_small_kernel(const double* __restrict__ v, int64_t v_stride, double v0, const double* __restrict__ x,
-                double* __restrict__ out, int64_t n, int ppw, double vmf_d) {
+                double* __restrict__ out, int64_t n, double vmf_d) {
   if (v_stride == 0 && v) v0 = v[0];
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * LB_SMALL_THREADS + threadIdx.x) >> 5, i = warp * ppw + lane;
+  const int64_t i = ((int64_t)blockIdx.x * LB_SMALL_THREADS + threadIdx.x) >> 5;
   __shared__ __align__(16) unsigned long long tab[KIND == KIND_K ? 2048 : 2];
-  warp_pairs64<KIND, DX, LB_SMALL_THREADS>(v, v_stride, v0, x, out, i, lane < ppw && i < n, vmf_d, tab);
+  warp_pair64<KIND, DX, LB_SMALL_THREADS>(v, v_stride, v0, x, out, i, i < n, vmf_d, tab);
 }
 
 // K integral, tight FP64: one thread per queued pair (lb_ktrap.cuh).  A
@@ -594,13 +593,9 @@ lb_status run_impl(const T* v, int64_t v_stride, const T* x, T* out, int64_t n, 
     if (mode == MODE_TIGHT && forced_region < 0) return run_tiles32<KIND>(v, v_stride, x, out, n, st);
   } else if (mode == MODE_TIGHT && forced_region < 0) {
     if (total_n <= LB_SMALL_N) {
-      // as few pairs per warp as 16 warps per SM allow
-      const int64_t most = (int64_t)sms * 16, want = (n + most - 1) / most;
-      const int ppw = (int)(want < 32 ? want : 32);
-      const int64_t warps = (n + ppw - 1) / ppw;
-      const int grid = (int)((warps * 32 + LB_SMALL_THREADS - 1) / LB_SMALL_THREADS);
+      const int grid = (int)((n * 32 + LB_SMALL_THREADS - 1) / LB_SMALL_THREADS);   // a warp per pair
       return launch(PS_TILES, st, [&] {
-        lb_small_kernel<KIND, DX><<<grid, LB_SMALL_THREADS, 0, st>>>(v, v_stride, v0, x, out, n, ppw, vmf_d);
+        lb_small_kernel<KIND, DX><<<grid, LB_SMALL_THREADS, 0, st>>>(v, v_stride, v0, x, out, n, vmf_d);
       });
     }
     if (KIND == KIND_K && total_n < kMidInTile)
