@@ -526,6 +526,21 @@ struct Warp32 {
   int count[16];
 };
 
+// The pairs that warp_pairs32 does not list or evaluate in line: domain edges,
+// v or x above 1e18, x below kTinyX32.  Called, so that the loop's code stays
+// small.
+template <int KIND>
+static __device__ __noinline__ float edge32(float v, float x) {
+  float r;
+  if (special_value32<KIND>(v, x, &r)) return r;
+  if (v <= 1e18f && x < 1.0f) {
+    if (v * v >= kAllR2) return u_all32<true>(KIND, v, x, v * v);
+    return KIND == KIND_I ? series_all32(v, x) : kt_small32(v, x);
+  }
+  const int g = classify32(v, x, MODE_TIGHT, KIND == KIND_K ? WIDE_K : WIDE_I);
+  return g == R_MU20 ? mu_expr32<KIND, 20>(v, x) : u_expr32<KIND, 4>(v, x);
+}
+
 // Sort key of a listed pair, 0 .. 15, in order of decreasing work.
 template <int KIND>
 __device__ __forceinline__ int key32(float v, float x) {
@@ -617,19 +632,13 @@ __device__ __forceinline__ void warp_pairs32(Warp32& W, const float* __restrict_
 #pragma unroll
     for (int e = 0; e < VEC; ++e) {
       const float xi = xx[e], vi = KIND == KIND_K ? fabsf(vv[e]) : vv[e];
-      float sp;
-      // one test for the domain edges and for squares out of range
-      if (!(xi > 0.0f && xi <= 1e18f && vi >= 0.0f && vi <= 1e18f)) {
-        if (special_value32<KIND>(vi, xi, &sp)) {
-          rr[e] = sp;
-        } else {
-          const int r = classify32(vi, xi, MODE_TIGHT, KIND == KIND_K ? WIDE_K : WIDE_I);
-          rr[e] = r == R_MU20 ? mu_expr32<KIND, 20>(vi, xi) : u_expr32<KIND, 4>(vi, xi);   // v or x > 1e18
-        }
+      // one test for the domain edges, squares out of range and quotients that underflow
+      if (!(xi >= kTinyX32 && xi <= 1e18f && vi >= 0.0f && vi <= 1e18f)) {
+        rr[e] = edge32<KIND>(vi, xi);
       } else {
         const float s2 = fmaf(vi, vi, xi * xi);
         if (s2 < kAllR2) fb |= 1u << e;
-        rr[e] = u_all32(KIND, vi, xi, s2);
+        rr[e] = u_all32<false>(KIND, vi, xi, s2);
       }
     }
     // a listed pair's result is written after this by the same warp; its slot
