@@ -517,8 +517,8 @@ __device__ __forceinline__ void warp_pair64(const double* __restrict__ v, int64_
 // at a time.  Nothing else is binned: binning every pair by region, as the
 // FP64 tiles do, costs more instructions than the one merged expansion.  A
 // pair's result depends on the pair alone.  The listed pairs' arguments are
-// read again from global memory; their outputs are not written before (out
-// may be x).
+// read again from global memory; their outputs are not written before where out
+// is x or v.
 constexpr int kList32 = 256 + 128;                         // entries before a flush, and one slice's
 struct Warp32 {
   uint32_t raw[kList32], list[kList32];                    // offsets from the base of v, x and out
@@ -603,7 +603,7 @@ __device__ __forceinline__ void warp_pairs32(Warp32& W, const float* __restrict_
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const float v0 = v_stride ? 0.0f : v[0];
-  const bool in_place = out == x;
+  const bool in_place = out == x || out == v;
   int cnt = 0;                                             // entries in the list (warp-uniform)
   for (int64_t s = begin + warp * (32 * VEC); s < end; s += nwarps * (32 * VEC)) {
     const int64_t i = s + lane * VEC;
@@ -642,7 +642,7 @@ __device__ __forceinline__ void warp_pairs32(Warp32& W, const float* __restrict_
       }
     }
     // a listed pair's result is written after this by the same warp; its slot
-    // may hold anything until then, except its argument when out is x
+    // may hold anything until then, except its argument or its order when out is x or v
     if (whole && (fb == 0 || !in_place)) {
       if (VEC == 4) *reinterpret_cast<float4*>(out + i) = make_float4(rr[0], rr[1 % VEC], rr[2 % VEC], rr[3 % VEC]);
     } else {
