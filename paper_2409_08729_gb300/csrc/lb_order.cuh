@@ -5,8 +5,8 @@
 // multiply-add per term.  In W = xmin / (2x), xmin the smallest x at which the
 // dispatch takes mu_20 for the order, the coefficients are b_k = a_k /
 // (4 xmin)^k, and with muq the exponent of the largest of them the sums are
-// kept in Q(59 - muq): as W <= 1/2, every Horner sum stays within +-2^61, and S
-// is within 2^(muq - 57) (a truncation and a coefficient's rounding per step,
+// kept in Q(60 - muq): as W <= 1/2, every Horner sum stays within +-2^62, and S
+// is within 2^(muq - 58) (a truncation and a coefficient's rounding per step,
 // halved by the next).
 //
 // That is an absolute bound, and log I's S is small where v^2/(2x) is large
@@ -14,7 +14,7 @@
 // by xmin itself.  muq is then at most 5 in tight mode; one power of two for
 // all orders below 15.4 left it at 11 to 14 for orders from 13 on and log I up
 // to 5.3e-15 off (v = 13.59, x = 30.1; now 3.3e-16, the expansion's truncation
-// included).  Where it is above 5 all the same (the paper's dispatch, log I,
+// included).  Where it is above 6 all the same (the paper's dispatch, log I,
 // orders about 15, x from 30 on) the general form serves (so_general).  The
 // finer coefficients cost 0.5 % (order 8, 20M pairs: 869 -> 873 us).
 //
@@ -97,23 +97,23 @@ LB_IX_FN int so_size(double b) {
 
 // Whether mu_20 takes the general form for this order.  Above xmin = 2^14 the
 // size of x itself makes any such error small.
-LB_IX_FN bool so_general(int kind, int muq, double scale) { return kind == 0 && muq > 5 && scale > 0x1p-13; }
+LB_IX_FN bool so_general(int kind, int muq, double scale) { return kind == 0 && muq > 6 && scale > 0x1p-13; }
 
-// b_k in Q(59 - muq), plus 2^62 (nothing where it overflows: orders past 1e150,
+// b_k in Q(60 - muq), plus 2^62 (nothing where it overflows: orders past 1e150,
 // whose x is so large that only the leading 1 counts).
 LB_IX_FN long long so_coef(double b, double bl, int muq) {
   if (!(fabs(b) < 0x1p51)) return 1ll << 62;
-  return ix_fix(b, 59 - muq) + ix_fix(bl, 59 - muq) + (1ll << 62);
+  return ix_fix(b, 60 - muq) + ix_fix(bl, 60 - muq) + (1ll << 62);
 }
 
-// The logarithm's constant, Q53: log I = x + (log((S 2^(59 - muq))^2 W) + it) / 2,
+// The logarithm's constant, Q53: log I = x + (log((S 2^(60 - muq))^2 W) + it) / 2,
 // with 1/x = scale W.
 LB_IX_FN long long so_log_const(int kind, int muq, double scale) {
-  return (((kind == 0 ? kSoLogI56 : kSoLogK56) - 2 * (59 - muq) * kLn2Q56 + 4) >> 3) + ix_log_q53(scale);
+  return (((kind == 0 ? kSoLogI56 : kSoLogK56) - 2 * (60 - muq) * kLn2Q56 + 4) >> 3) + ix_log_q53(scale);
 }
 
-// S 2^(59 - muq) by Horner's rule, n terms past the first; W = 1/(scale x).  On
-// the sums plus 2^62 (positive: the short unsigned product), the bias's
+// S 2^(60 - muq) by Horner's rule, n terms past the first; W = 1/(scale x).  On
+// the sums plus 2^62 (from 0 to 2^63: the short unsigned product), the bias's
 // product taken off again.
 LB_IX_FN double so_sum(const long long* b, double W, int n) {
   const uint64_t w = (uint64_t)ix_fix(W, 64);              // below 2^63

@@ -2,12 +2,12 @@
 block's set-up and of the fixed-point sum, over the orders at which the scale
 or the form changes, in both dispatches.
 
-The sum against the exact (rational) one: within 2^(muq - 57) absolute.  log I
-in tight mode: muq <= 5 and S >= 0.048 (order 13.59 at x = 30), so 4.6e-15
-relative against a result of the size of x >= 30, 1.5e-16 x; the rounding of W
-moves S by v^2/(2x) <= 3.1 times 2^-52, 0.2e-16 x.  log K: smaller, S >= 0.9
-where v is small and above 1 where muq is not 0.  The paper's dispatch: muq <= 5
-in this form, S as in tight mode.  Bound taken: 2e-16 x.
+The sum against the exact (rational) one: within 2^(muq - 58) absolute.  log I
+in tight mode: muq <= 5 and S >= 0.048 (order 13.59 at x = 30), so 2.3e-15
+relative against a result of the size of x >= 30, 0.8e-16 x; the rounding of W
+moves S by v^2/(2x) <= 3.7 times 2^-52, 0.3e-16 x.  log K: smaller, S >= 0.9
+where v is small and above 1 where muq is not 0.  The paper's dispatch: muq <= 6
+in this form, S >= 0.027: 1.7e-16 x.  Bound taken: 2e-16 x.
 The values against the oracle, in units of the error metric: the expansion's
 truncation 3.1e-16, the sum 2e-16, logarithm and roundings 2.3e-16: 1e-15."""
 import ctypes
@@ -58,7 +58,7 @@ extern "C" int order(int kind, int tight, double v, const double* x, double* S, 
     terms[i] = lb_mut[cw * (LB_MUT_A_CELLS + 1) + ca] & 255;
     const double W = ix_rcp(scale * x[i]), s = so_sum(mu, W, terms[i]);
     *Wmax = fmax(*Wmax, W);
-    S[i] = ldexp(s, muq - 59);
+    S[i] = ldexp(s, muq - 60);
     f[i] = fma(0x1p-54, (double)(ix_log_q53(s * s * W) + so_log_const(kind, muq, scale)), kind == 0 ? x[i] : -x[i]);
   }
   return muq | (int)so_general(kind, muq, scale) << 8;
@@ -111,7 +111,7 @@ def test_sum_against_the_exact_sum(order, kind, tight):
         x = x0 * (1.0 + np.concatenate([[1e-9, 1e-3, 0.01, 0.05], np.geomspace(0.1, 30.0, 20)]))
         S, _, terms, W, muq, general = order(kind, tight, v, x)
         assert 0.49 < W < 0.5, v
-        assert muq <= (5 if kind == 0 else 8) or (general and not tight) or x0 > 2.0 ** 14, (v, muq)
+        assert muq <= (6 if kind == 0 else 8) or (general and not tight) or x0 > 2.0 ** 14, (v, muq)
         if general:
             continue
         for xi, si, n in zip(x, S, terms):
