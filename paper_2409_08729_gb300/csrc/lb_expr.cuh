@@ -494,6 +494,8 @@ struct ScalarOrder {
   bool mu_general;                      // so_general
   long long muc;                        // so_log_const
   long long mu[21];                     // so_coef of b_0 .. b_20
+  int uk;                               // so_u_terms
+  long long u[40];                      // so_u_coef
   double ser[91];                       // 1 / (k (k + v)), k = 1..90
   dfloat serd[91];                      // ser[] in double-float
 };
@@ -538,11 +540,16 @@ __device__ __forceinline__ void scalar_order_setup(ScalarOrder& so, double v, in
   } else if (tid < 64) {
     if (tid == 32) so.lg1 = lgamma1p(v);
   }
-  if (NT > 64 ? tid >= 64 : tid >= 32)
-    for (int k = tid - (NT > 64 ? 63 : 31); k <= 90; k += NT - (NT > 64 ? 64 : 32)) {
-      so.ser[k] = 1.0 / ((double)k * ((double)k + v));
-      so.serd[k] = df_from_double(so.ser[k]);
-    }
+  static_assert(NT >= 224, "warps for every part");
+  if (tid >= 64 && tid < 154) {
+    const int k = tid - 63;
+    so.ser[k] = 1.0 / ((double)k * ((double)k + v));
+    so.serd[k] = df_from_double(so.ser[k]);
+  } else if (tid >= 160 && tid < 200) {
+    const int K = so_u_terms(v, mode), m = tid - 160;
+    if (m <= 3 * K) so.u[m] = so_u_coef(KIND, v, K, m, lb_debye_c);
+    if (m == 0) so.uk = K;
+  }
   __syncthreads();
 }
 

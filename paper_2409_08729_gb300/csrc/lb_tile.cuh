@@ -163,8 +163,10 @@ __device__ __forceinline__ T tile_expr(int r, T v, T x, int n, const ScalarOrder
         else if constexpr (SO) return series_so(*so, x, n);
         else return series_log_i_n(v, x, n);
       default: {
-        const int Kmax = __reduce_max_sync(0xffffffffu, n);
         const double s = fma(v, v, x * x);
+        if constexpr (SO)
+          if (so->uk) return uni_ok(s, x) ? so_u(KIND, so->u, 3 * so->uk, v, x, s) : u_expr<KIND>(v, x, n);
+        const int Kmax = __reduce_max_sync(0xffffffffu, n);
         return uni_ok(s, x) ? u_fx(KIND, v, x, s, n, Kmax) : u_expr<KIND>(v, x, n);
       }
     }

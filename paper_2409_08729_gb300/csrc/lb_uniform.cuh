@@ -81,6 +81,17 @@ LB_IX_FN uint64_t uni_step(int kind, uint64_t acc, uint64_t h, uint64_t c0) {
   return kind ? c0 - m : c0 + m;
 }
 
+// log I (kind 0) or log K from the sum S (Q62, below 2), r and q = 1/r.
+LB_IX_FN double uni_log(int kind, double v, double x, double r, double q, uint64_t S) {
+  // S^2 / r: Q62 x Q62, then the 53 bits of 1/r
+  const uint64_t bq = ix_bits(q);
+  const uint64_t W = kt_mulhi(kt_mulhi(S, S) << 2, ((bq & 0x000fffffffffffffull) | 0x0010000000000000ull) << 10);   // Q60
+  const long long lw = kt_logq(ix_pack(W, 1021 - (int)(bq >> 52)));
+  const double a = (double)(kt_logq(x) - kt_logq(v + r)), w = v * 0x1p-53;
+  if (kind == 0) return fma(w, a, fma(0x1p-54, (double)(lw - kHalfLog2PiQ53x2), r));
+  return -fma(w, a, fma(-0x1p-54, (double)(lw + kLogHalfPiQ53), r));
+}
+
 // log I (kind 0) or log K of one pair with s = v^2 + x^2, uni_ok; K: the
 // pair's terms, Kmax: the warp's largest.
 LB_IX_FN double u_fx(int kind, double v, double x, double s, int K, int Kmax) {
@@ -102,13 +113,7 @@ LB_IX_FN double u_fx(int kind, double v, double x, double s, int K, int Kmax) {
     if (k > K) acc = kUniBias;
   }
   const uint64_t S = uni_step(kind, acc, u.h, c0) + (1ull << 56) - kUniBias;   // Q56
-  // S^2 / r: Q62 x Q62, then the 53 bits of 1/r
-  const uint64_t bq = ix_bits(q);
-  const uint64_t W = kt_mulhi(kt_mulhi(S << 6, S << 6) << 2, ((bq & 0x000fffffffffffffull) | 0x0010000000000000ull) << 10);   // Q60
-  const long long lw = kt_logq(ix_pack(W, 1021 - (int)(bq >> 52)));
-  const double a = (double)(kt_logq(x) - kt_logq(v + r)), w = v * 0x1p-53;
-  if (kind == 0) return fma(w, a, fma(0x1p-54, (double)(lw - kHalfLog2PiQ53x2), r));
-  return -fma(w, a, fma(-0x1p-54, (double)(lw + kLogHalfPiQ53), r));
+  return uni_log(kind, v, x, r, q, S << 6);
 }
 
 // Terms for the x-derivative, whose sum's term k is k times the value's: the

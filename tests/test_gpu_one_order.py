@@ -14,8 +14,8 @@ import oracle
 import paper_2409_08729_gb300 as lb
 
 pytestmark = pytest.mark.gpu
-ORDERS = [0.0, 0.3, 2.5, 8.0, 9.4, 10.9, 11.0, 12.0, 12.6964, 13.3, 13.59, 13.6, 14.5, 15.0, 15.39, 16.0, 17.0, 28.5,
-          100.0]
+ORDERS = [0.0, 0.3, 2.5, 8.0, 9.4, 10.0, 10.001, 10.9, 11.0, 12.0, 12.6964, 13.3, 13.59, 13.6, 14.5, 15.0, 15.39, 16.0,
+          17.0, 20.0, 24.0, 28.0, 28.5, 70.0, 70.5, 100.0, 230.5, 1e4]
 
 
 def _arguments(v, rng):

@@ -1,6 +1,6 @@
-"""mu_20 of a call with one order (csrc/lb_order.cuh): the host build of the
-block's set-up and of the fixed-point sum, over the orders at which the scale
-or the form changes, in both dispatches.
+"""mu_20 and U_K of a call with one order (csrc/lb_order.cuh): the host build of
+the block's set-up and of the fixed-point sums, over the orders at which a
+scale, a degree or the form changes, in both dispatches.
 
 The sum against the exact (rational) one: within 2^(muq - 58) absolute.  log I
 in tight mode: muq <= 5 and S >= 0.048 (order 13.59 at x = 30), so 2.3e-15
@@ -9,7 +9,9 @@ moves S by v^2/(2x) <= 3.7 times 2^-52, 0.3e-16 x.  log K: smaller, S >= 0.9
 where v is small and above 1 where muq is not 0.  The paper's dispatch: muq <= 6
 in this form, S >= 0.027: 1.7e-16 x.  Bound taken: 2e-16 x.
 The values against the oracle, in units of the error metric: the expansion's
-truncation 3.1e-16, the sum 2e-16, logarithm and roundings 2.3e-16: 1e-15."""
+truncation 3.1e-16, the sum 2e-16, logarithm and roundings 2.3e-16: 1e-15.
+U_K's polynomial: truncation 4e-16, the sum 2^-54, its three logarithms (2^-53
+each, times v) 2.2e-16, two roundings of the result 2.2e-16: 1e-15."""
 import ctypes
 import os
 import subprocess
@@ -23,6 +25,13 @@ import oracle
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2409_08729_gb300", "csrc")
 TOL = 1e-15
 SRC = r'''
+#define __constant__
+#define __host__
+#define __device__
+#define __forceinline__ inline
+template <typename T> T lb_fma(T a, T b, T c);
+#include "lb_df.cuh"
+#include "debye_uk.h"
 #include "lb_order.cuh"
 #define LB_MUT_TABLE static const
 #include "muterms_table.h"
@@ -63,6 +72,18 @@ extern "C" int order(int kind, int tight, double v, const double* x, double* S, 
   }
   return muq | (int)so_general(kind, muq, scale) << 8;
 }
+// returns K; the values, and the largest of the coefficients past the first
+extern "C" int poly(int kind, int mode, double v, const double* x, double* f, long n, double* cmax) {
+  const int K = so_u_terms(v, mode);
+  long long c[40];
+  *cmax = 0.0;
+  for (int m = 0; m <= 3 * K && K; ++m) {
+    c[m] = so_u_coef(kind, v, K, m, lb_debye_c);
+    if (m) *cmax = fmax(*cmax, fabs((double)c[m] * 0x1p-61));
+  }
+  for (long i = 0; i < n && K; ++i) f[i] = so_u(kind, c, 3 * K, v, x[i], fma(v, v, x[i] * x[i]));
+  return K;
+}
 '''
 
 
@@ -82,6 +103,7 @@ def order(tmp_path_factory):
         r = L.order(kind, int(tight), ctypes.c_double(v), *(a.ctypes.data_as(ctypes.c_void_p) for a in (x, S, f, t)),
                     ctypes.c_long(x.size), ctypes.byref(W))
         return S, f, t, W.value, r & 255, bool(r >> 8)
+    run.poly = L.poly
     return run
 
 
@@ -136,3 +158,35 @@ def test_values_against_oracle(order, kind):
         ref = (oracle.log_k if kind else oracle.log_i)(vv, x)
         err = oracle.rel_err(f, ref, oracle.error_scale("ik"[kind], vv, x))
         assert err.max() <= TOL, (v, x[err.argmax()], err.max())
+
+
+@pytest.mark.parametrize("kind", [0, 1])
+def test_polynomial_against_oracle(order, kind):
+    r = np.random.default_rng(8)
+    seen = set()
+    for v in [10.0000001, 10.5, 12.0, 13.6, 14.001, 16.0, 16.001, 20.0, 28.0, 28.001, 50.0, 70.0, 70.001, 150.0, 230.0, 230.001,
+              1e3, 1e5, 1e8] + list(np.exp(r.uniform(np.log(10.1), np.log(2000.0), 15))):
+        # U_K of the tight dispatch: up to where mu_20 takes over, from the wide ranges' edges on
+        lo = 1e-6 if v > 16 else (14.5 if v > 14 else 17.5 if v > 12 and kind == 0 else 19.5)
+        hi = max(v * v / 3.24, 59.69) if v >= 13.6 else (30.0 if kind == 0 else 22.0 if v >= 12.5 else 20.0)
+        x = np.concatenate([np.exp(r.uniform(np.log(lo), np.log(hi), 250)), lo + (hi - lo) * r.random(250) ** 4, [lo, hi]])
+        x = np.ascontiguousarray(x[x < 1e8])
+        f, cmax = np.empty_like(x), ctypes.c_double()
+        K = order.poly(kind, 0, ctypes.c_double(v), *(a.ctypes.data_as(ctypes.c_void_p) for a in (x, f)),
+                       ctypes.c_long(x.size), ctypes.byref(cmax))
+        assert K == (4 if v > 230 else 6 if v > 70 else 9 if v > 28 else 13) and cmax.value < 0.25
+        seen.add(K)
+        vv = np.full_like(x, v)
+        ref = (oracle.log_k if kind else oracle.log_i)(vv, x)
+        err = oracle.rel_err(f, ref, oracle.error_scale("ik"[kind], vv, x))
+        assert err.max() <= TOL, (v, x[err.argmax()], err.max())
+    assert seen == {4, 6, 9, 13}
+
+
+def test_polynomial_orders(order):
+    """None up to order 10, past 1e150, or where several K serve one order."""
+    x, f, c = np.array([25.0]), np.empty(1), ctypes.c_double()
+    for v, mode, K in [(10.0, 0, 0), (9.0, 1, 0), (-20.0, 0, 0), (np.nan, 0, 0), (np.inf, 0, 0), (1e151, 0, 0), (20.0, 2, 0),
+                       (20.0, 1, 13), (300.0, 1, 13), (300.0, 0, 4)]:
+        assert order.poly(0, mode, ctypes.c_double(v), *(a.ctypes.data_as(ctypes.c_void_p) for a in (x, f)),
+                          ctypes.c_long(1), ctypes.byref(c)) == K, (v, mode)
