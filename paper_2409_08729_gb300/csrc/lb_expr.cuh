@@ -596,9 +596,15 @@ __device__ __forceinline__ double series_so(const ScalarOrder& so, double x, int
 //   d/dx log f = +-1 - (1/x) (1/2 + E/S).
 // The sums as mu_expr_n's: Q <- D_k Q + 20!/(k-1)! and, D_k being
 // proportional to w, R <- D_k (Q + R) beside it; the terms past the leading
-// h in double-float, at most cap terms.
+// h in double-float, at most cap terms.  For half an odd integer the sum ends
+// (D_(v + 1/2) = 0): order 1/2, 5M pairs, x in [1, 100], 575 -> 512 us.
 template <int KIND>
 __device__ __forceinline__ double mu_dx_n(double v, double x, int counts, int cap) {
+  {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v), M = (b & 0xfffffffffffffull) | (1ull << 52);
+    const int p = 1074 - (int)(b >> 52);            // 2v = M / 2^p
+    if (__ffsll((long long)M) - 1 == p) cap = min(cap, (int)(((M >> p) - 1) >> 1));
+  }
   const int n = __reduce_max_sync(0xffffffffu, min(cap, counts & 255));
   const int h = min(n, __reduce_max_sync(0xffffffffu, counts >> 8));
   const double rx = ix_rcp_call(8.0 * x);           // on the integer pipe
