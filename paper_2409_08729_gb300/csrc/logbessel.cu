@@ -533,7 +533,8 @@ lb_status run_tiles32(const float* v, int64_t v_stride, const float* x, float* o
 //   up to LB_SMALL_N  lb_small_kernel alone (tight mode);
 //   below 2^17        tiles of 256 pairs, one per thread, the K fallback in the
 //                     tile (tight mode): one launch and no scratch;
-//   below 2^20        tiles of 512 pairs, two per thread, K fallback queued;
+//   below 2^20        tiles of 512 pairs, two per thread, K fallback queued
+//                     (see large_tiles for what leaves them sooner);
 //   from there        tiles of 2048 pairs, four per thread, K fallback queued.
 // Device time of a call on the mixed-order sweep, log I / log K, us: 1000
 // pairs 12 / 12 (small kernel) against 16 / 15 (256-pair tiles); 4000 pairs 17
@@ -555,6 +556,22 @@ lb_status launch_tiles(int sms, cudaStream_t st, const T* v, int64_t v_stride, T
   });
 }
 
+// Whether a call of n pairs between 2^17 and 2^20 leaves the 512-pair tiles: one
+// wave of them holds 467000 pairs on 152 SMs, one of 2048-pair tiles 934000.  In
+// between, the small ones run a second wave that is partly empty (a quarter of
+// one is made up for by the emptier SMs it runs on).  The large ones take it
+// there for log I's derivative (600000 pairs, order 1/2: 83 us with the small
+// ones, 71 with the large; order 4 85 / 70, mixed sweep 75 / 64; 500000 pairs of
+// U_K 37 / 43) and for the paper's dispatches (whole domain, 600000 pairs, log I
+// 155 / 136, its derivative 176 / 150; order 4, 500000 pairs 106 / 118, 1M 193 /
+// 216).  (The tight values' kernels and log K's derivative are as fast either
+// way.)
+inline bool large_tiles(int sms, int mode, bool dx_i, int64_t n) {
+  constexpr int64_t kMidWave = tiles_ctas(LB_MID_THREADS, false) * LB_MID_THREADS * LB_MID_ITEMS;
+  return (mode != MODE_TIGHT || dx_i) && n > sms * kMidWave / 4 * 5 &&
+         n <= (int64_t)sms * LB_TILES_CTAS_PER_SM * kTile;
+}
+
 // The tile kernel of a pass of n pairs: one order per call has its constants
 // computed per block, where there are enough pairs to pay for that.
 template <int KIND, bool DX, typename T>
@@ -563,10 +580,11 @@ lb_status run_tiles(int sms, cudaStream_t st, const T* v, int64_t v_stride, T v0
                     double vmf_d) {
   if constexpr (sizeof(T) == 8) {
     // (an order known here to be past 16 -- the vMF form's d/2 - 1 usually is --
-    // takes the general kernel: mostly U_K then, which the one-order kernel has
-    // no faster form of.  log C_2048, 1M values: 97 -> 72 us)
+    // takes the general kernel: U_4 sums are short, and the one-order kernel's
+    // set-up pays in large calls only.  log C_2048: 600000 values 54 us against
+    // 58, 1M 78 against 81, 4M 258 against 246)
     const bool so = !DX && v_stride == 0 && forced_region < 0 && (v || (double)v0 <= 16.0);
-    if (total_n < kMid && forced_region < 0) {
+    if (total_n < kMid && forced_region < 0 && !large_tiles(sms, mode, KIND == KIND_I && DX && v, total_n)) {
       if (so && total_n >= kMidInTile)
         return launch_tiles<KIND, DX, T, !DX, LB_MID_THREADS, LB_MID_ITEMS, false>(sms, st, v, v_stride, v0, x, out, n, mode,
                                                                   forced_region, qcount, queue, cap, vmf_d);
