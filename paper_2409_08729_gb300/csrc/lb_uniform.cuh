@@ -81,15 +81,18 @@ LB_IX_FN uint64_t uni_step(int kind, uint64_t acc, uint64_t h, uint64_t c0) {
   return kind ? c0 - m : c0 + m;
 }
 
-// log I (kind 0) or log K from the sum S (Q62, below 2), r and q = 1/r.
+// log I (kind 0) or log K from the sum S (Q62, below 2), r and q = 1/r.  r and
+// v log(x/(v + r)) first, which nearly cancel where the result is small: the
+// rest is then added to what is left, not rounded to the size of r before.
 LB_IX_FN double uni_log(int kind, double v, double x, double r, double q, uint64_t S) {
   // S^2 / r: Q62 x Q62, then the 53 bits of 1/r
   const uint64_t bq = ix_bits(q);
   const uint64_t W = kt_mulhi(kt_mulhi(S, S) << 2, ((bq & 0x000fffffffffffffull) | 0x0010000000000000ull) << 10);   // Q60
   const long long lw = kt_logq(ix_pack(W, 1021 - (int)(bq >> 52)));
   const double a = (double)(kt_logq(x) - kt_logq(v + r)), w = v * 0x1p-53;
-  if (kind == 0) return fma(w, a, fma(0x1p-54, (double)(lw - kHalfLog2PiQ53x2), r));
-  return -fma(w, a, fma(-0x1p-54, (double)(lw + kLogHalfPiQ53), r));
+  const double e = fma(w, a, r);
+  if (kind == 0) return fma(0x1p-54, (double)(lw - kHalfLog2PiQ53x2), e);
+  return fma(0x1p-54, (double)(lw + kLogHalfPiQ53), -e);
 }
 
 // log I (kind 0) or log K of one pair with s = v^2 + x^2, uni_ok; K: the
