@@ -180,7 +180,7 @@ lb_status logbessel_vmf_log_c(lb_dtype dtype, double d, const void* kappa, void*
  * 2 d/dx log I, 3 d/dx log K.  v, x, out are host pointers (pinned memory
  * lets the copies overlap with the computation; pageable memory works but
  * copies synchronously).  The pairs are processed in chunks of `chunk`
- * (0 = 2M pairs; at most 2^26) through four device chunk slots and three
+ * (0 = 2M pairs, 4M in FP32; at most 2^26) through four device chunk slots and three
  * internal streams, so the copy-in of one chunk, the evaluation of the
  * previous one and the copy-out of the one before overlap; when chunk is a
  * multiple of 16384 the first and last pieces are smaller (down to chunk/8)
