@@ -32,8 +32,8 @@ METRIC = "Gevals/s (log I_v and log K_v, FP64)"
 # capture of every launch of one full-size step; empty when the kernels
 # changed since.
 NCU_DRAM_BYTES_PER_STEP = {}
-# Pipe utilisation of each kernel from ncu on 6M pairs of the same workload
-# (profiles/kernels_6m_pairs.md): share of peak issue of the FP64 pipe, the
+# Pipe utilisation of each kernel from ncu on 6M pairs of the same workload:
+# share of peak issue of the FP64 pipe, the
 # ALU pipe, the FMA-heavy pipe (integer multiplies), the FP32 (FMA) pipe and
 # the XU (special-function) pipe while active, and the share of cycles that
 # issue; empty when stale.

@@ -15,8 +15,8 @@ Per pair, in tight mode, with n the pair's own term count (not the warp's):
 
   region          general pair                  one order for the whole call
   mu_K (n terms)  2n + 8     rcp, log           n + 6     rcp, log
-  U_K             K(K+1)/2 + K + 14             the same
-                  rsqrt, 3 log
+  U_K             K(K+1)/2 + K + 14             3K + 13 (orders above 10)
+                  rsqrt, 3 log                  rsqrt, 3 log
   series (n)      4n + 7     rcp, 2 log, lgamma 2n + 5    2 log
   K integral      7 per node, 14 per pair       the same
                   exp: 1 per node, rsqrt, 2 rcp, 2 log per pair
@@ -29,7 +29,8 @@ sum is a polynomial in w: one fma per term.
 U_K: v^2 + x^2, r = (v^2 + x^2) / sqrt, v/r, its square, v + r, the Debye
 polynomial P_k of degree k by Horner (k fmas, k = 1..K), Horner over k in 1/r
 (K fmas), S^2/r (2), the difference of the logarithms, final fmas.  K is the
-pair's own: its region's, or less at large r.
+pair's own: its region's, or less at large r.  With one order above 10 the sum
+is one polynomial in v/r of degree 3K, K the order's (3K fmas).
 Series (the linear fraction of the reading of Eq. "log Iv" with a_0 as
 shift): per term d_k = k(k+v) (fma), A <- d B + y A (mul, fma), B <- d B;
 per pair y = x^2/4, A/B, v+1, x/2, two combining operations.  With one
@@ -144,7 +145,8 @@ def region_ops(region, v, x, shared=False, fp32=False):
         return (n + 6) if (shared and region == 0) else (2 * n + 8)
     if region in REGION_K:
         K = uni_terms(v, x, REGION_K[region])
-        return K * (K + 1) // 2 + K + 14
+        ops = K * (K + 1) // 2 + K + 14
+        return np.where(np.abs(v) > 10.0, 3 * REGION_K[region] + 13, ops) if shared else ops
     n = series_terms(v, x)
     return (2 * n + 5) if shared else (4 * n + 7)
 

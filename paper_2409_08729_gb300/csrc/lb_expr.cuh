@@ -228,7 +228,7 @@ __device__ __forceinline__ int mu_counts(float v, float x) {
   return (int)__ldg(lb_mut + cw * (LB_MUT_A_CELLS + 1) + ca);
 }
 
-// Terms of the power series of log I (series_log_i, series_so): the count
+// Terms of the power series of log I (series_log_i_n, series_so): the count
 // n after which a term falls below 2^-56 of the running sum past the peak
 // index (Eq. "K"), by a single-precision pass; at most 90.  Returned packed
 // with the number h of leading terms kept in FP64: the terms past the peak
@@ -470,10 +470,6 @@ __device__ __forceinline__ double series_log_i_n(double v, double x, int packed)
   double res = ix_log_call(A * ix_rcp_call(B)) - lgamma1p(v);
   if ((__double_as_longlong(v) << 1) != 0) res = fma(v, ix_log_call(0.5 * x), res);   // v != 0, on the bits
   return res;
-}
-
-__device__ __forceinline__ double series_log_i(double v, double x) {
-  return series_log_i_n(v, x, series_terms(f32_cut(v), f32_cut(x)));
 }
 
 // ---------------------------------------------------------------------------
