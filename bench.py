@@ -38,16 +38,16 @@ NCU_DRAM_BYTES_PER_STEP = {}
 # the XU (special-function) pipe while active, and the share of cycles that
 # issue; empty when stale.
 NCU_PIPES = {
-    "lb_tiles_kernel": {"fp64": 0.477, "alu": 0.472, "fma_heavy": 0.429, "fma": 0.252, "xu": 0.019,
-                        "issue_active": 0.661, "launch": "log K, mixed orders, 6M pairs"},
-    "lb_kint_kernel": {"fp64": 0.105, "alu": 0.478, "fma_heavy": 0.420, "fma": 0.210, "xu": 0.011,
-                       "issue_active": 0.539, "launch": "lb_ktrap_kernel after the same call's tiles (one pair in "
+    "lb_tiles_kernel": {"fp64": 0.461, "alu": 0.474, "fma_heavy": 0.430, "fma": 0.253, "xu": 0.019,
+                        "issue_active": 0.663, "launch": "log K, mixed orders, 6M pairs"},
+    "lb_kint_kernel": {"fp64": 0.105, "alu": 0.478, "fma_heavy": 0.419, "fma": 0.210, "xu": 0.011,
+                       "issue_active": 0.538, "launch": "lb_ktrap_kernel after the same call's tiles (one pair in "
                                                         "seven; all classes of the whole domain: alu 0.56, "
                                                         "issue 0.60)"},
 }
 NCU_PIPES_FP32 = {
-    "lb_tiles_kernel": {"fp64": 0.0, "alu": 0.514, "fma_heavy": 0.228, "fma": 0.350, "xu": 0.118,
-                        "issue_active": 0.747, "launch": "lb_tiles32_kernel, log I, mixed orders, 6M pairs"},
+    "lb_tiles_kernel": {"fp64": 0.0, "alu": 0.505, "fma_heavy": 0.227, "fma": 0.353, "xu": 0.119,
+                        "issue_active": 0.738, "launch": "lb_tiles32_kernel, log I, mixed orders, 6M pairs"},
 }
 UNIT = "Gevals/s"
 WORKLOAD = "paper-shaped sweep: v=2^0..2^10 x 20M x~U[1,100] per order, log I + log K, per-order + mixed-order calls"

@@ -317,11 +317,11 @@ lb_kint_kernel(const double* __restrict__ v, int64_t v_stride, const double* __r
 }
 
 // FP32, tight mode: see warp_pairs32.  Bound by issue: log I over mixed
-// orders, 24M pairs, 131 us (387 with the binned tiles), 155 thread
-// instructions per pair, issue 75 %, ALU 51 %, DRAM 17 % at 6M pairs; log K
-// over the whole domain, 16M pairs, 196 us (2670 with a warp per integral; 217
-// with the edges' code in the loop instead of called), issue 69 % and
-// instruction fetch, as its warps are in different loops.
+// orders, 24M pairs, 128 us (387 with the binned tiles), 155 thread
+// instructions per pair, issue 74 %, ALU 51 %, DRAM 17 % at 6M pairs; log K
+// over the whole domain, 16M pairs, 195 us (2670 with a warp per integral; 217,
+// issue 69 % and waits for instructions, with the edges' code in the loop
+// instead of called), issue 75 %.
 template <int KIND, int VEC>
 __global__ void __launch_bounds__(LB_THREADS, LB_TILES32_CTAS_PER_SM)
 lb_tiles32_kernel(const float* __restrict__ v, int64_t v_stride, const float* __restrict__ x,
