@@ -488,7 +488,7 @@ struct ScalarOrder {
   double v, lg1;                        // v, lgamma(v + 1)
   double scale;                         // so_scale
   bool mu_general;                      // so_general
-  long long muc;                        // so_log_const
+  long long muc;                        // so_log_const and log(scale), Q53
   long long mu[21];                     // so_coef of b_0 .. b_20
   int uk;                               // so_u_terms
   long long u[40];                      // so_u_coef
@@ -507,6 +507,8 @@ __device__ __forceinline__ void scalar_order_setup(ScalarOrder& so, double v, in
     const int k = tid < 20 ? tid : 20;
     const double rf = __ldg(&lb_rfact[k][0]), rfl = __ldg(&lb_rfact[k][1]);
     const double scale = so_scale(KIND, mode == MODE_TIGHT, v);
+    long long ls = ix_log_q53(scale);
+    asm volatile("" : "+l"(ls));                    // here: its table reads wait beside the products
     double bl, b = so_ratio(KIND, v, k < 1 ? 1 : k, scale, bl);
     if (tid == 0) { b = 1.0; bl = 0.0; }
     if (so_pairs(v)) {
@@ -531,12 +533,12 @@ __device__ __forceinline__ void scalar_order_setup(ScalarOrder& so, double v, in
       so.v = v;
       so.scale = scale;
       so.mu_general = so_general(KIND, muq, scale);
-      so.muc = so_log_const(KIND, muq, scale);
+      so.muc = so_log_const(KIND, muq) + ls;
     }
   } else if (tid < 64) {
     if (tid == 32) so.lg1 = lgamma1p(v);
   }
-  static_assert(NT >= 224, "warps for every part");
+  static_assert(NT >= 256, "warps for every part");
   if (tid >= 64 && tid < 154) {
     const int k = tid - 63;
     so.ser[k] = 1.0 / ((double)k * ((double)k + v));

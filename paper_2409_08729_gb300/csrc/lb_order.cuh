@@ -77,10 +77,12 @@ LB_IX_FN double so_ratio(int kind, double v, int k, double scale, double& lo) {
 }
 
 // Whether the coefficients are formed as pairs of doubles: where log I's S is
-// 0.05 the terms reach 5, and coefficients rounded to doubles would cost log S
-// 20 roundings.  Below 9.5 S is above 0.14 and the terms below 2 (and the pairs
-// would cost every block 1 us).
-LB_IX_FN bool so_pairs(double v) { return v >= 9.5; }
+// 0.02 to 0.1 (orders from 11.5 to 15.4, x about 30) the terms reach 5, and
+// coefficients rounded to doubles would cost log S 20 roundings (order 13.59:
+// mean error 2.4e-16 of the result, 0.4e-16 with the pairs).  Elsewhere log I's S is
+// above 0.08 and both give the same errors; the pairs would cost every block
+// 0.9 us.
+LB_IX_FN bool so_pairs(double v) { return v >= 11.5 && v < 15.4; }
 
 // (b + bl) <- (b + bl) (u + ul)
 LB_IX_FN void so_mul(double& b, double& bl, double u, double ul) {
@@ -107,10 +109,10 @@ LB_IX_FN long long so_coef(double b, double bl, int muq) {
   return ix_fix(b, 60 - muq) + ix_fix(bl, 60 - muq) + (1ll << 62);
 }
 
-// The logarithm's constant, Q53: log I = x + (log((S 2^(60 - muq))^2 W) + it) / 2,
-// with 1/x = scale W.
-LB_IX_FN long long so_log_const(int kind, int muq, double scale) {
-  return (((kind == 0 ? kSoLogI56 : kSoLogK56) - 2 * (60 - muq) * kLn2Q56 + 4) >> 3) + ix_log_q53(scale);
+// The logarithm's constant less log(scale), Q53: with 1/x = scale W,
+// log I = x + (log((S 2^(60 - muq))^2 W) + it + log(scale)) / 2.
+LB_IX_FN long long so_log_const(int kind, int muq) {
+  return ((kind == 0 ? kSoLogI56 : kSoLogK56) - 2 * (60 - muq) * kLn2Q56 + 4) >> 3;
 }
 
 // S 2^(60 - muq) by Horner's rule, n terms past the first; W = 1/(scale x).  On
@@ -144,14 +146,30 @@ LB_IX_FN int so_u_terms(double v, int mode) {
   return mode == 1 ? 13 : v > 230.0 ? 4 : v > 70.0 ? 6 : v > 28.0 ? 9 : 13;
 }
 
-// The coefficient of t^m in Q61; c[k][i]: that of t^(k + 2i) in u_k.
+// The coefficient of t^m in Q61; c[k][i]: that of t^(k + 2i) in u_k.  The terms
+// are k = m, m - 2, .. (at most K) down to m/3, five of them at most: Horner's
+// rule in 1/v^2, then the lowest power of 1/v (a short chain: every block waits
+// for it).
 LB_IX_FN long long so_u_coef(int kind, double v, int K, int m, const double (*c)[14]) {
-  const double iv = kind == 0 ? ix_rcp(v) : -ix_rcp(v);
-  double sum = 0.0, p = 1.0;
-  for (int k = 0; k <= K; ++k) {
-    const int i2 = m - k;
-    if (i2 >= 0 && (i2 & 1) == 0 && i2 <= 2 * k) sum = fma(c[k][i2 >> 1], p, sum);
-    p *= iv;
+  const double iv = kind == 0 ? ix_rcp(v) : -ix_rcp(v), w = iv * iv;
+  int k1 = m < K ? m : K, k0 = (m + 2) / 3;
+  k1 -= (k1 ^ m) & 1;
+  k0 += (k0 ^ m) & 1;
+  double sum = 0.0;
+#if defined(__CUDACC__)
+#pragma unroll
+#endif
+  for (int j = 0; j < 5; ++j) {
+    const int k = k1 - 2 * j;
+    if (k >= k0) sum = fma(sum, w, c[k][(m - k) >> 1]);
+  }
+  double q = iv;
+#if defined(__CUDACC__)
+#pragma unroll
+#endif
+  for (int j = 0; j < 4; ++j) {                             // sum iv^k0, k0 <= 13
+    if ((k0 >> j) & 1) sum *= q;
+    q *= q;
   }
   return ix_fix(sum, 61);
 }

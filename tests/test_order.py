@@ -68,7 +68,7 @@ extern "C" int order(int kind, int tight, double v, const double* x, double* S, 
     const double W = ix_rcp(scale * x[i]), s = so_sum(mu, W, terms[i]);
     *Wmax = fmax(*Wmax, W);
     S[i] = ldexp(s, muq - 60);
-    f[i] = fma(0x1p-54, (double)(ix_log_q53(s * s * W) + so_log_const(kind, muq, scale)), kind == 0 ? x[i] : -x[i]);
+    f[i] = fma(0x1p-54, (double)(ix_log_q53(s * s * W) + so_log_const(kind, muq) + ix_log_q53(scale)), kind == 0 ? x[i] : -x[i]);
   }
   return muq | (int)so_general(kind, muq, scale) << 8;
 }
